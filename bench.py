@@ -280,7 +280,7 @@ def step_traffic():
 
 
 # the sources the body-free step's kernels and their launches are built from
-STEP_SOURCES = ("common.cuh", "transfer.cuh", "transfer.cu", "fft.cu", "fft.cuh", "fft_reg.cuh", "dfloat.cuh",
+STEP_SOURCES = ("common.cuh", "transfer.cuh", "transfer.cu", "fft.cu", "fft.cuh", "fft_reg.cuh", "fixpt.cuh", "fixfft.cu",
                 "lgf.cu", "api.cu", "tune.cu")
 
 

@@ -23,7 +23,7 @@ void free_plan(pf_plan p) {
     for (cudaEvent_t e : p->tm.pool) cudaEventDestroy(e);
     void* own[] = {p->T1, p->T2a, p->T2b, p->w, p->uv, p->tile_count, p->gmax, p->tile_start, p->bin_off,
                    p->pos, p->recs, p->stage, p->stage_out, p->diag, p->rhs64, p->nz_idx, p->nz_val, p->vent_idx, p->vent_val,
-                   p->d_status, p->d_oob};
+                   p->d_status, p->d_oob, p->fx_exp};
     for (void* q : own)
         if (q) cudaFree(q);
     if (p->pscr) cudaFree(p->pscr);
@@ -33,10 +33,9 @@ void free_plan(pf_plan p) {
     }
     if (p->shared && --p->shared->refs == 0) {
         void* tables[] = {p->G, p->H64, p->H32, p->Hu64, p->Hv64, p->Hu32, p->Hv32, p->twP64, p->twQ64, p->twP32,
-                          p->twQ32, p->tw256_64, p->tw256_32};
+                          p->twQ32, p->tw256_64, p->tw256_32, p->twP_fx, p->twQ_fx};
         for (void* q : tables)
             if (q) cudaFree(q);
-        if (p->shared->df) cudaFree(p->shared->df);
         delete p->shared;
     }
 }
@@ -95,6 +94,11 @@ pf_status plan_init(pf_plan p) {
     twiddles(t256f, 256);
     PF_TRY(upload(p, &p->tw256_64, t256d));
     PF_TRY(upload(p, &p->tw256_32, t256f));
+    std::vector<int4> fx;
+    fx_twiddles(fx, P);
+    PF_TRY(upload(p, &p->twP_fx, fx));
+    fx_twiddles(fx, Q);
+    PF_TRY(upload(p, &p->twQ_fx, fx));
     PF_TRY(plan_workspaces(p));
     return lgf_build(p);
 }
@@ -120,6 +124,7 @@ pf_status plan_workspaces(pf_plan p) {
     PF_CUDA(p, cudaMalloc(&p->gmax, (BIN_MAX_BLOCKS + 1) * sizeof(double)));
     PF_CUDA(p, cudaMalloc(&p->tile_start, (size_t)p->tile_slots * sizeof(int)));
     PF_CUDA(p, cudaMalloc(&p->diag, PF_DIAG_DOUBLES * sizeof(double)));
+    PF_CUDA(p, cudaMalloc(&p->fx_exp, FXE_INTS * sizeof(int)));
     PF_CUDA(p, cudaMalloc(&p->d_status, sizeof(int)));
     PF_CUDA(p, cudaMalloc(&p->d_oob, sizeof(unsigned long long)));
     // The status words are read before any kernel writes them.  A plain
@@ -198,6 +203,7 @@ pf_status pf_plan_clone(pf_plan src, int32_t precision, void* stream, pf_plan* o
     p->G = src->G; p->H64 = src->H64; p->H32 = src->H32; p->Hu64 = src->Hu64; p->Hv64 = src->Hv64;
     p->Hu32 = src->Hu32; p->Hv32 = src->Hv32; p->twP64 = src->twP64; p->twQ64 = src->twQ64; p->twP32 = src->twP32;
     p->twQ32 = src->twQ32; p->tw256_64 = src->tw256_64; p->tw256_32 = src->tw256_32;
+    p->twP_fx = src->twP_fx; p->twQ_fx = src->twQ_fx;
     // make sure the source's tables are complete before another stream reads them
     if (cudaStreamSynchronize(src->stream) != cudaSuccess) {
         free_plan(p);

@@ -1250,18 +1250,16 @@ void schur_free(pf_schur s) {
 // Full sheet solve on device.  psi_w: real field; vx, vy: device positions of
 // the new vortices (mode KUTTA_SHED).  Results: f (device, ns) and scal[0..2] =
 // (s0, Gamma1, Gamma2) on the device.
-// E_s L^-1 w into ew (ns doubles).  The direct FP64 sum costs 16 ns nx ny
-// multiply-adds at the GPU's low FP64 rate; on larger grids the same quantity
-// comes from an FP64 FFT solve psi = -L^-1 w (FP64 rounding, far below what
-// the ill-conditioned S amplifies into the sheet) read at the stencils.
-// Route of E_s L^-1 w from the field w (no vortex source): the sparse sum when
-// the caller bounds the nonzero nodes and the sum is small (below 2^24
-// multiply-adds its few blocks finish sooner than an FFT's passes), else the
-// FFT solve where the padded torus allows it, else the direct sum.  The sums
-// run on the FP64 pipe; the FFT of an FP64 plan too, so an FP64 plan keeps
-// the direct sum on small grids; that of a mixed plan runs in double-float on
-// the FP32 pipe (about sixty times the FP64 rate on this GPU) and is taken
-// whenever it fits.
+// E_s L^-1 w into ew (ns doubles): the FP64 sum with the LGF, over all nodes
+// or over a list of the nonzero ones, or a 64-bit FFT solve psi = -L^-1 w
+// (fixfft.cu) read at the stencils.
+// Route from the field w (no vortex source): the sparse sum when the caller
+// bounds the nonzero nodes and the sum is small (below 2^24 multiply-adds its
+// few blocks finish sooner than an FFT's passes), else the FFT solve where the
+// padded torus allows it, else the direct sum.  The sums run on the FP64 pipe
+// (two multiply-adds a clock and SM), the FFT on the integer pipe, so an FP64
+// plan keeps the direct sum only below ns nx ny = 2^18, where it takes about
+// as long as the FFT's three launches (128^2: 72 us at ns 64, 2^20, against 25).
 enum FieldRoute { ROUTE_SPARSE, ROUTE_DIRECT, ROUTE_FFT };
 
 FieldRoute field_route(pf_plan p, int ns, int64_t nnz_bound) {
@@ -1273,7 +1271,7 @@ FieldRoute field_route(pf_plan p, int ns, int64_t nnz_bound) {
         (p->rhs_route == PF_RHS_AUTO && nnz_bound >= 0 && 16 * (int64_t)ns * nnz_bound < sparse_max))
         return ROUTE_SPARSE;
     if (fft_ok && (p->rhs_route == PF_RHS_FFT ||
-                   (p->rhs_route == PF_RHS_AUTO && (mixed || (int64_t)ns * M > ((int64_t)1 << 22)))))
+                   (p->rhs_route == PF_RHS_AUTO && (mixed || (int64_t)ns * M > ((int64_t)1 << 18)))))
         return ROUTE_FFT;
     return ROUTE_DIRECT;
 }
@@ -1291,9 +1289,8 @@ pf_status field_route_buffers(pf_plan p, FieldRoute r) {
         if (!p->rhs64) {
             const size_t spec = (size_t)p->ldK * p->ldT * 2 * sizeof(double);
             PF_CUDA(p, cudaStreamSynchronize(p->stream));
-            PF_CUDA(p, cudaMalloc(&p->rhs64, 2 * (size_t)M * sizeof(double) + 2 * spec));
+            PF_CUDA(p, cudaMalloc(&p->rhs64, (size_t)(M + (M & 1)) * sizeof(double) + 2 * spec));
         }
-        PF_TRY(df_tables_ready(p));
     }
     return PF_OK;
 }
@@ -1366,24 +1363,18 @@ pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew, int64_t 
         return PF_OK;
     }
     const size_t spec = (size_t)p->ldK * p->ldT * 2 * sizeof(double);
-    const double* w64;
     double* psi;
     void *T1, *T2;
     if (p->prec == PF_FP64) {      // the plan's own buffers are free during a sheet solve
-        w64 = (const double*)w;
         psi = (double*)p->uv;
         T1 = p->T1;
         T2 = p->T2a;
     } else {
-        double* b = (double*)p->rhs64;
-        psi = b + M;
-        T1 = b + 2 * M;
+        psi = (double*)p->rhs64;
+        T1 = psi + M + (M & 1);
         T2 = (char*)T1 + spec;
-        w64 = nullptr;
     }
-    // FP64 plans: FP64 passes; mixed plans: double-float passes on the FP32 w
-    if (w64) PF_TRY(conv_psi_f64(p, w64, psi, T1, T2));
-    else PF_TRY(conv_psi_df(p, (const float*)w, psi, T1, T2, p->rhs64, s->rows));
+    PF_TRY(conv_psi_fx(p, w, psi, T1, T2, s->rows));
     k_surface_from_psi<<<ceil_div(ns, 128), 128, 0, st>>>(psi, p->nx, ns, s->six, s->siy, s->swx, s->swy, ew);
     PF_LAUNCH_CHECK(p);
     return PF_OK;

@@ -80,12 +80,11 @@ inline int bin_blocks(int64_t nv, int min_span = BIN_MIN_SPAN) {
 // Read-only tables of one grid shape, shared by a plan and its clones.
 struct PlanTables {
     int refs = 1;
-    // double-float copies of H64 and of the FP64 twiddles (H | twP | twQ, one
-    // allocation) for the mixed plans' FFT route of the surface right-hand
-    // side, built by the first plan that needs them
-    std::mutex mu;
-    void* df = nullptr;
 };
+
+// layout of a plan's fx_exp: the largest column exponent, then one exponent per
+// row pair and, per component, per column
+enum { FXE_ROW = 4, FXE_COLA = FXE_ROW + 1028, FXE_COLB = FXE_COLA + 2052, FXE_INTS = FXE_COLB + 2052 };
 
 struct pf_plan_s {
     PlanTables* shared = nullptr;  // owner of G, H*, twiddles (reference counted)
@@ -110,6 +109,9 @@ struct pf_plan_s {
     float2* twQ32 = nullptr;
     double2* tw256_64 = nullptr;   // exp(-2 pi i m / 256), m in [0, 256)
     float2* tw256_32 = nullptr;
+    int4* twP_fx = nullptr;        // twP, twQ in Q62 halves (fixfft.cu)
+    int4* twQ_fx = nullptr;
+    int* fx_exp = nullptr;         // exponents of the fixed-point passes: FXE_* below (per plan)
     // grid work buffers (element size depends on precision)
     size_t esz = 8;
     int ldT = 0;                   // ny rounded up to 4
@@ -278,10 +280,9 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // (defined in the .cu files, used by api.cu)
 pf_status lgf_build(pf_plan p);                                  // lgf.cu
 pf_status conv_solve(pf_plan p, const void* w, void* out, int mode, double Uinf, double Vinf);  // fft.cu
-pf_status conv_psi_f64(pf_plan p, const double* w, double* psi, void* T1, void* T2);           // fft.cu
-pf_status conv_psi_df(pf_plan p, const float* w, double* psi, void* T1, void* T2, void* wdf,
-                      const int* rows);                                                        // fft.cu
-pf_status df_tables_ready(pf_plan p);                                                          // fft.cu
+pf_status conv_fx(pf_plan p, const double* w, double* out, int mode, double Uinf, double Vinf);   // fixfft.cu
+pf_status conv_psi_fx(pf_plan p, const void* w, double* psi, void* T1, void* T2, const int* rows);  // fixfft.cu
+void fx_twiddles(std::vector<int4>& v, int N);                                                   // fixfft.cu
 enum { CONV_PSI = 0, CONV_UV = 1 };
 pf_status vortex_regularize(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
                             const int64_t* dn = nullptr, void* zu = nullptr, void* zv = nullptr);  // transfer.cu

@@ -16,14 +16,11 @@
 //               keep nodes [0, nx).
 #include <type_traits>
 
-#include "dfloat.cuh"
 #include "fft.cuh"
 #include "fft_reg.cuh"
 
-template <> struct real_of<dfc> { using type = dfl; };
-
 template <typename T>
-__global__ void __launch_bounds__(512) k_rows_fwd(const T* __restrict__ w, C_t<T>* __restrict__ T1, int nx, int ny,
+__global__ void __launch_bounds__(256) k_rows_fwd(const T* __restrict__ w, C_t<T>* __restrict__ T1, int nx, int ny,
                                                   int P, const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -49,21 +46,15 @@ __global__ void __launch_bounds__(512) k_rows_fwd(const T* __restrict__ w, C_t<T
 }
 
 template <typename T>
-__global__ void __launch_bounds__(512) k_cols(const C_t<T>* __restrict__ T1, C_t<T>* __restrict__ T2a,
+__global__ void __launch_bounds__(256) k_cols(const C_t<T>* __restrict__ T1, C_t<T>* __restrict__ T2a,
                                               C_t<T>* __restrict__ T2b, int ny, int Q, int mode,
                                               const T* __restrict__ H, const T* __restrict__ Hu,
-                                              const T* __restrict__ Hv, int Hld, const C_t<T>* __restrict__ tw,
-                                              const int* __restrict__ rows) {
+                                              const T* __restrict__ Hv, int Hld, const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);
     C* B = A + Q;
     C* D = B + Q;
-    // rows (nullable, mode CONV_PSI): only output rows rows[0] .. rows[1] are
-    // needed; the row pass takes rows in (even, odd) pairs, so both rows of
-    // every pair that holds a needed one are written (a pair's other row
-    // enters its arithmetic, and must be finite)
-    const int jlo = rows ? max(rows[0], 0) & ~1 : 0, jhi = rows ? min(rows[1] | 1, ny - 1) : ny - 1;
     const int k = blockIdx.x;
     for (int l = threadIdx.x; l < Q; l += blockDim.x)
         A[l] = l < ny ? T1[(size_t)k * ny + l] : cmake<C>(T(0), T(0));
@@ -91,15 +82,14 @@ __global__ void __launch_bounds__(512) k_cols(const C_t<T>* __restrict__ T1, C_t
         for (int l = threadIdx.x; l < Q; l += blockDim.x) Z[l] = Z[l] * H[row + (l <= Q / 2 ? l : Q - l)];
         __syncthreads();
         C* R = block_fft<C, true>(Z, other, Q, tw);
-        for (int j = jlo + (int)threadIdx.x; j <= jhi && j < ny; j += blockDim.x) T2a[(size_t)k * ny + j] = R[j];
+        for (int j = threadIdx.x; j < ny; j += blockDim.x) T2a[(size_t)k * ny + j] = R[j];
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(512) k_rows_inv(const C_t<T>* __restrict__ T2a, const C_t<T>* __restrict__ T2b,
+__global__ void __launch_bounds__(256) k_rows_inv(const C_t<T>* __restrict__ T2a, const C_t<T>* __restrict__ T2b,
                                                   T* __restrict__ out, int nx, int ny, int P, int mode, T Uinf,
-                                                  T Vinf, const C_t<T>* __restrict__ tw,
-                                                  const int* __restrict__ rows) {
+                                                  T Vinf, const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* A = reinterpret_cast<C*>(smem_raw);
@@ -115,8 +105,6 @@ __global__ void __launch_bounds__(512) k_rows_inv(const C_t<T>* __restrict__ T2a
         jb = ja + 1;
         has_b = jb < ny;
         Sb = T2a;
-        // rows (nullable): blocks whose two rows are not read later do nothing
-        if (rows && (jb < rows[0] || ja > rows[1])) return;
     }
     const int h = P / 2;
     for (int k = threadIdx.x; k <= h; k += blockDim.x) {
@@ -483,29 +471,21 @@ static pf_status conv_dispatch(pf_plan p, const T* w, T* out, int mode, T Uinf, 
 
 template <typename T>
 static pf_status conv_solve_t(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                              const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws,
-                              const int* rows = nullptr) {
+                              const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
     using C = C_t<T>;
     const int P = p->P, Q = p->Q, nx = p->nx, ny = p->ny;
-    // the third column buffer holds the second component (mode CONV_UV) only;
-    // the double-float passes of 2048 points and more run 512 threads a block,
-    // one radix-4 butterfly each per pass (their arithmetic, not shared memory,
-    // bounds them; shorter transforms keep 256, which have work for no more)
+    // the third column buffer holds the second component (mode CONV_UV) only
     const size_t sr = 2 * (size_t)P * sizeof(C), sc = (mode == CONV_UV ? 3 : 2) * (size_t)Q * sizeof(C);
-    const bool df = std::is_same<T, dfl>::value;
-    const int ntP = df && P >= 2048 ? 512 : 256, ntQ = df && Q >= 2048 ? 512 : 256;
     PF_CUDA(p, set_smem(k_rows_fwd<T>, sr));
     PF_CUDA(p, set_smem(k_cols<T>, sc));
     PF_CUDA(p, set_smem(k_rows_inv<T>, sr));
     C* T1 = reinterpret_cast<C*>(ws.T1);
     C* T2a = reinterpret_cast<C*>(ws.T2a);
     C* T2b = reinterpret_cast<C*>(ws.T2b);
-    PF_KERNEL(p, "fft_rows_fwd", k_rows_fwd<T><<<(ny + 1) / 2, ntP, sr, p->stream>>>(w, T1, nx, ny, P, twP));
-    PF_KERNEL(p, "fft_cols_conv", k_cols<T><<<P / 2 + 1, ntQ, sc, p->stream>>>(T1, T2a, T2b, ny, Q, mode, H, Hu, Hv, p->Hld, twQ,
-                                                                              rows));
+    PF_KERNEL(p, "fft_rows_fwd", k_rows_fwd<T><<<(ny + 1) / 2, 256, sr, p->stream>>>(w, T1, nx, ny, P, twP));
+    PF_KERNEL(p, "fft_cols_conv", k_cols<T><<<P / 2 + 1, 256, sc, p->stream>>>(T1, T2a, T2b, ny, Q, mode, H, Hu, Hv, p->Hld, twQ));
     const int nb = mode == CONV_UV ? ny : (ny + 1) / 2;
-    PF_KERNEL(p, "fft_rows_inv", k_rows_inv<T><<<nb, ntP, sr, p->stream>>>(T2a, T2b, out, nx, ny, P, mode, Uinf, Vinf, twP,
-                                                                               rows));
+    PF_KERNEL(p, "fft_rows_inv", k_rows_inv<T><<<nb, 256, sr, p->stream>>>(T2a, T2b, out, nx, ny, P, mode, Uinf, Vinf, twP));
     return PF_OK;
 }
 
@@ -515,9 +495,7 @@ pf_status conv_solve(pf_plan p, const void* w, void* out, int mode, double Uinf,
     const bool reg = p->fft_impl == 0 && p->P >= 256 && p->Q >= 256;
     const ConvWs ws{p->T1, p->T2a, p->T2b};
     if (p->prec == PF_FP64) {
-        if (reg)
-            return conv_dispatch<double>(p, (const double*)w, (double*)out, mode, Uinf, Vinf, p->H64, p->Hu64, p->Hv64,
-                                         p->twP64, p->twQ64, p->tw256_64, ws);
+        if (reg) return conv_fx(p, (const double*)w, (double*)out, mode, Uinf, Vinf);
         return conv_solve_t<double>(p, (const double*)w, (double*)out, mode, Uinf, Vinf, p->H64, p->Hu64, p->Hv64,
                                     p->twP64, p->twQ64, ws);
     }
@@ -526,101 +504,4 @@ pf_status conv_solve(pf_plan p, const void* w, void* out, int mode, double Uinf,
                                     p->Hv32, p->twP32, p->twQ32, p->tw256_32, ws);
     return conv_solve_t<float>(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
                                p->Hv32, p->twP32, p->twQ32, ws);
-}
-
-// psi = -L^-1 w in FP64 for either precision of plan, on the register-resident
-// path (P, Q >= 256), with caller-given FP64 workspaces T1, T2 (ldT x ldK
-// complex each): the surface right-hand side of the sheet solves.
-pf_status conv_psi_f64(pf_plan p, const double* w, double* psi, void* T1, void* T2) {
-    if (p->P < 256 || p->Q < 256) return PF_ERR_ARG;
-    return conv_dispatch<double>(p, w, psi, CONV_PSI, 0.0, 0.0, p->H64, p->Hu64, p->Hv64, p->twP64, p->twQ64,
-                                 p->tw256_64, ConvWs{T1, T2, T2});
-}
-
-// ---------------------------------------------------------------- double-float route
-// psi = -L^-1 w for a mixed plan's FP32 w with the shared-memory passes run
-// in double-float (dfloat.cuh): the FP64-class surface right-hand side of the
-// sheet solves at the FP32 pipe's rate.  (The register-resident passes, fully
-// unrolled, grow too large in double-float to compile in reasonable time.)
-// w is widened exactly (lo = 0); psi is returned as doubles (hi + lo).
-
-namespace {
-
-__global__ void k_df_table(const double* __restrict__ src, int64_t n, dfl* __restrict__ dst) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = dfl(src[i]);
-}
-
-__global__ void k_widen_df(const float* __restrict__ w, int64_t n, dfl* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = dfl(w[i], 0.0f);
-}
-
-// in place: element i of a dfl array becomes element i of a double array (same
-// size), over rows rows[0] .. rows[1] (clamped to [0, ny)) of nx elements
-__global__ void k_df_to_double(void* data, int nx, int ny, const int* __restrict__ rows) {
-    const int64_t i0 = (int64_t)max(rows[0], 0) * nx, i1 = (int64_t)(min(rows[1], ny - 1) + 1) * nx;
-    for (int64_t i = i0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < i1; i += (int64_t)gridDim.x * blockDim.x) {
-        const dfl v = reinterpret_cast<const dfl*>(data)[i];
-        reinterpret_cast<double*>(data)[i] = df_to_double(v);
-    }
-}
-
-struct DfTables {
-    const dfl* H;
-    const dfc *twP, *twQ;
-};
-
-pf_status df_tables(pf_plan p, DfTables& t) {
-    PlanTables* sh = p->shared;
-    const size_t nh = (size_t)(p->P / 2 + 1) * p->Hld;
-    std::lock_guard<std::mutex> lock(sh->mu);
-    if (!sh->df) {
-        const size_t bytes = nh * sizeof(dfl) + (size_t)(p->P + p->Q) * sizeof(dfc);
-        void* d = nullptr;
-        PF_CUDA(p, cudaMalloc(&d, bytes));
-        dfl* h = (dfl*)d;
-        dfc* tp = (dfc*)(h + nh);
-        dfc* tq = tp + p->P;
-        k_df_table<<<152 * 2, 256, 0, p->stream>>>(p->H64, (int64_t)nh, h);
-        k_df_table<<<8, 256, 0, p->stream>>>((const double*)p->twP64, 2 * (int64_t)p->P, (dfl*)tp);
-        k_df_table<<<8, 256, 0, p->stream>>>((const double*)p->twQ64, 2 * (int64_t)p->Q, (dfl*)tq);
-        cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);    // complete before any stream reads them
-        if (e != cudaSuccess) {
-            cudaFree(d);
-            snprintf(p->err, sizeof(p->err), "double-float tables: %s", cudaGetErrorString(e));
-            return PF_ERR_CUDA;
-        }
-        sh->df = d;
-    }
-    t.H = (const dfl*)sh->df;
-    t.twP = (const dfc*)(t.H + nh);
-    t.twQ = t.twP + p->P;
-    return PF_OK;
-}
-
-}  // namespace
-
-pf_status df_tables_ready(pf_plan p) {
-    if (p->P < 256 || p->Q < 256) return PF_ERR_ARG;
-    DfTables t;
-    return df_tables(p, t);
-}
-
-// wdf: scratch of nx ny double-floats (8 bytes each); psi: nx ny doubles, of
-// which only rows rows[0] .. rows[1] (device, within [0, ny)) are computed
-pf_status conv_psi_df(pf_plan p, const float* w, double* psi, void* T1, void* T2, void* wdf, const int* rows) {
-    if (p->P < 256 || p->Q < 256) return PF_ERR_ARG;
-    DfTables t;
-    PF_TRY(df_tables(p, t));
-    const int64_t M = (int64_t)p->nx * p->ny;
-    const int nb = (int)std::min<int64_t>(ceil_div(M, 256), 152 * 4);
-    k_widen_df<<<nb, 256, 0, p->stream>>>(w, M, (dfl*)wdf);
-    PF_LAUNCH_CHECK(p);
-    PF_TRY(conv_solve_t<dfl>(p, (const dfl*)wdf, (dfl*)psi, CONV_PSI, dfl(0.0), dfl(0.0), t.H, t.H, t.H, t.twP, t.twQ,
-                             ConvWs{T1, T2, T2}, rows));
-    k_df_to_double<<<nb, 256, 0, p->stream>>>(psi, p->nx, p->ny, rows);
-    PF_LAUNCH_CHECK(p);
-    return PF_OK;
 }

@@ -8,12 +8,14 @@
 // twice.  Forward: X(k) = sum_n x(n) exp(-2 pi i k n / N); inverse: +i,
 // unnormalised.  tw256[m] = exp(-2 pi i m / 256), twN[m] = exp(-2 pi i m / N).
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
+#include "fixpt.cuh"
 
 template <typename C> struct real_of;
 template <> struct real_of<float2> { using type = float; };
 template <> struct real_of<double2> { using type = double; };
-// (double-float complex: dfloat.cuh)
 
 // cos(2 pi m / 16) for a compile-time m
 template <int M>
@@ -28,18 +30,23 @@ __host__ __device__ constexpr double cos16() {
 // x * exp(-+ 2 pi i m / 16) for a compile-time m (forward: minus sign)
 template <typename C, bool INV, int M>
 __device__ __forceinline__ C rot16(C x) {
-    using R = typename real_of<C>::type;
-    constexpr int m = M & 15;
-    if (m == 0) return x;
-    if (m == 4) return INV ? mul_i(x) : mul_mi(x);
-    if (m == 8) { x.x = -x.x; x.y = -x.y; return x; }
-    if (m == 12) return INV ? mul_mi(x) : mul_i(x);
-    constexpr R c = (R)cos16<m>();
-    constexpr R s = (R)(INV ? cos16<m + 12>() : -cos16<m + 12>());   // sin(t) = cos(t - pi/2)
-    C r;
-    r.x = x.x * c - x.y * s;
-    r.y = x.x * s + x.y * c;
-    return r;
+    if constexpr (std::is_same<C, fxc>::value) {
+        static_assert(!INV, "fixed-point inverses exchange real and imaginary parts");
+        return fx_rot16<M>(x);
+    } else {
+        using R = typename real_of<C>::type;
+        constexpr int m = M & 15;
+        if (m == 0) return x;
+        if (m == 4) return INV ? mul_i(x) : mul_mi(x);
+        if (m == 8) { x.x = -x.x; x.y = -x.y; return x; }
+        if (m == 12) return INV ? mul_mi(x) : mul_i(x);
+        constexpr R c = (R)cos16<m>();
+        constexpr R s = (R)(INV ? cos16<m + 12>() : -cos16<m + 12>());   // sin(t) = cos(t - pi/2)
+        C r;
+        r.x = x.x * c - x.y * s;
+        r.y = x.x * s + x.y * c;
+        return r;
+    }
 }
 
 template <typename C, bool INV>
@@ -105,10 +112,10 @@ __device__ __forceinline__ void dft16(C* v) {   // natural order in and out
 
 template <typename C, bool INV, int R>
 __device__ __forceinline__ void dft_r(C* v) {
-    if (R == 16) dft16<C, INV>(v);
-    else if (R == 8) dft8<C, INV>(v);
-    else if (R == 4) dft4<C, INV>(v[0], v[1], v[2], v[3]);
-    else if (R == 2) dft2<C, INV>(v[0], v[1]);
+    if constexpr (R == 16) dft16<C, INV>(v);
+    else if constexpr (R == 8) dft8<C, INV>(v);
+    else if constexpr (R == 4) dft4<C, INV>(v[0], v[1], v[2], v[3]);
+    else if constexpr (R == 2) dft2<C, INV>(v[0], v[1]);
 }
 
 template <typename C, bool INV>
