@@ -101,8 +101,8 @@ __device__ __forceinline__ int fx_shift_of(unsigned mask) { return (32 - __clz(m
 
 // a 2^-d, rounded, halves away from zero: rounding them all up would add the
 // same sign to every element, which a transform collects in its zero
-// frequency, where the Green's function is largest.  d may be negative or
-// beyond 63.
+// frequency, where the Green's function is largest.  fx_round: d > 0;
+// fx_align: d may be negative or beyond 63.
 __device__ __forceinline__ long long fx_round(long long a, long long half, int d) { return (a + half + (a >> 63)) >> d; }
 __device__ __forceinline__ long long fx_align1(long long a, int d) {
     if (d <= 0) return a << (-d);

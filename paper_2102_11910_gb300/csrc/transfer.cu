@@ -95,7 +95,7 @@ pf_status regularize_configured(pf_plan p, const BinWork& bw, const double* X, c
 template <int TILE>
 pf_status interpolate_tiles(pf_plan p, const Geo& geo, const void* uv, int64_t nq, void* uq, void* vq) {
     if (p->prec == PF_FP64)
-        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles<double, TILE>, geo.ntiles, p->tile_threads, 0,
+        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles_f64<TILE>, geo.ntiles, p->tile_threads, 0,
                                                          p->stream, (const Rec<double>*)p->recs, p->tile_start,
                                                          p->tile_count, (const double2*)uv, geo, (double*)uq,
                                                          (double*)vq, p->rec_cap, nq, p->d_status)));

@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "fixpt.cuh"
 
 namespace {
 
@@ -75,19 +76,62 @@ __device__ __forceinline__ Rec<double> make_rec(const Pos<double>& p, int lx, in
     return r;
 }
 
-// M4' weights of the four nodes floor(g)-1 .. floor(g)+2 for fractional part f
-template <typename T>
-__device__ __forceinline__ void m4p_weights(T f, T w[4]) {
-    const T a0 = T(1) + f, a1 = f, a2 = T(1) - f, a3 = T(2) - f;
-    w[0] = T(0.5) * (T(2) - a0) * (T(2) - a0) * (T(1) - a0);
-    w[1] = T(1) - T(2.5) * a1 * a1 + T(1.5) * a1 * a1 * a1;
-    w[2] = T(1) - T(2.5) * a2 * a2 + T(1.5) * a2 * a2 * a2;
-    w[3] = T(0.5) * (T(2) - a3) * (T(2) - a3) * (T(1) - a3);
+// M4' weights of the four nodes floor(g)-1 .. floor(g)+2 for fractional part f.
+// FP32: the cubics term by term (their arithmetic hides behind the shared
+// adds and loads: the nine-operation form below measured no faster there).
+__device__ __forceinline__ void m4p_weights(float f, float w[4]) {
+    const float a0 = 1.0f + f, a1 = f, a2 = 1.0f - f, a3 = 2.0f - f;
+    w[0] = 0.5f * (2.0f - a0) * (2.0f - a0) * (1.0f - a0);
+    w[1] = 1.0f - 2.5f * a1 * a1 + 1.5f * a1 * a1 * a1;
+    w[2] = 1.0f - 2.5f * a2 * a2 + 1.5f * a2 * a2 * a2;
+    w[3] = 0.5f * (2.0f - a3) * (2.0f - a3) * (1.0f - a3);
+}
+// FP64: with t = 1 - f and p = f t the cubics are -p t / 2, t + p (1 - 3/2 f),
+// f + p (1 - 3/2 t) and -p f / 2, nine operations of a pipe that issues two a
+// clock and SM.
+__device__ __forceinline__ void m4p_weights(double f, double w[4]) {
+    const double t = 1.0 - f, p = f * t, h = -0.5 * p;
+    w[0] = h * t;
+    w[1] = fma(p, fma(-1.5, f, 1.0), t);
+    w[2] = fma(p, fma(-1.5, t, 1.0), f);
+    w[3] = h * f;
+}
+
+// The same weights in Q61 as centred halves (fixpt.cuh), from the fraction in
+// Q60: FP64 records' terms are formed on the integer pipe, which issues a 32 x
+// 32 + 64 multiply-add sixteen times as often as the FP64 pipe a multiply.
+// With a = p f and b = p t = p - a the weights are -b/2, t + p - 3/2 a, f + p -
+// 3/2 b, -a/2: their sum is exactly one, each is within 2^-60 of its value.
+constexpr int Q_FRAC = 60, Q_WEIGHT = 61;
+__device__ __forceinline__ long long fx_frac(double f) {       // f in [0, 1): multiples of 2^-60 are exact
+    const long long b = __double_as_longlong(f);
+    const int ef = (int)(b >> 52);
+    if (ef == 0) return 0;
+    const long long m = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+    const int d = 1075 - Q_FRAC - ef;                            // m 2^(ef - 1075) 2^60
+    return d <= 0 ? m << -d : (d > 54 ? 0ll : (m + ((1ll << d) >> 1)) >> d);
+}
+__device__ __forceinline__ long long fx_qmul60(long long a, long long b) {
+    const FxSplit x = fx_split(a), y = fx_split(b);
+    const long long t = (1ll << 28) + fx_mw(x.h, y.l) + fx_mw(x.l, y.h);
+    return (fx_mw(x.h, y.h) << 2) + (t >> 29);
+}
+__device__ __forceinline__ void fx_m4p(double frac, FxSplit (&w)[4]) {
+    const long long f = fx_frac(frac), t = (1ll << Q_FRAC) - f, p = fx_qmul60(f, t), a = fx_qmul60(p, f), b = p - a;
+    w[0] = fx_split(-b);
+    w[1] = fx_split(2 * (t + p) - 3 * a);
+    w[2] = fx_split(2 * (f + p) - 3 * b);
+    w[3] = fx_split(-a);
+}
+// x w 2^-61
+__device__ __forceinline__ long long fx_weigh(FxSplit x, FxSplit w) {
+    const long long t = (1ll << 29) + fx_mw(x.h, w.l) + fx_mw(x.l, w.h);
+    return (fx_mw(x.h, w.h) << 1) + (t >> 30);
 }
 
 // Grid coordinate g of a position; the stencil floor(g)-1 .. floor(g)+2 lies in
 // [0, n) iff 1 <= g < n - 2.  FP64 path: g = (X - x0)/dx, fraction g - floor(g)
-// exact.  Mixed path: one FMA, then the integer and fractional parts are read
+// exact (the binning passes: split_div).  Mixed path: one FMA, then the integer and fractional parts are read
 // from the bits of g (no further FP64 work); the fraction is truncated to 24 bits.
 __device__ __forceinline__ bool split(double X, double x0, double dx, double, double, int n, long long, int& c,
                                       double& f) {
@@ -166,16 +210,44 @@ struct Geo {
     double inv_dx2;            // 1/dx^2
     long long xlim, ylim;      // bit patterns of (double)(nx - 2), (double)(ny - 2)
     int nx, ny, ntx, ntiles;
+    int recip;                 // dx and 1/dx far from the ends of the double range: loc_split divides by 1/dx
 };
 
 // the split used by the locate pass: fixed-point fraction (mixed), exact (FP64)
 __device__ __forceinline__ bool loc_split(double X, const Geo& g, int axis, int& c, unsigned& fr) {
     return split_fixed(X, g.inv_dx, axis ? g.cy : g.cx, axis ? g.ylim : g.xlim, c, fr);
 }
-__device__ __forceinline__ bool loc_split(double X, const Geo& g, int axis, int& c, double& f) {
-    return split(X, axis ? g.y0 : g.x0, g.dx, 0.0, 0.0, axis ? g.ny : g.nx, 0, c, f);
+// g = (X - x0)/dx as the division gives it, from the rounded reciprocal: two
+// corrections by exact residuals (Markstein's theorem: with the correctly
+// rounded reciprocal the second one rounds correctly).  Range test, cell and
+// fraction from the bits of g, so that a coordinate costs six FP64
+// instructions instead of a division's fifteen and six more (k_locate at 1e6
+// vortices: 60 -> 33 us).
+__device__ __forceinline__ bool loc_split(double X, const Geo& geo, int axis, int& c, double& f) {
+    const double x0 = axis ? geo.y0 : geo.x0;
+    if (!geo.recip) return split(X, x0, geo.dx, 0.0, 0.0, axis ? geo.ny : geo.nx, 0, c, f);
+    const double d = X - x0;
+    double g = d * geo.inv_dx;
+    g = fma(fma(-g, geo.dx, d), geo.inv_dx, g);
+    g = fma(fma(-g, geo.dx, d), geo.inv_dx, g);
+    const long long gb = __double_as_longlong(g);
+    if (gb < 0x3FF0000000000000ll || gb >= (axis ? geo.ylim : geo.xlim)) return false;
+    const int e = (int)(gb >> 52) - 1023;                               // 0 .. 10
+    const long long m = (gb & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+    c = (int)(m >> (52 - e));
+    const long long r = m & ((1ll << (52 - e)) - 1);                    // fraction 2^(52 - e)
+    const int lz = __clzll(r);                                          // leading bit to bit 52
+    f = r == 0 ? 0.0 : __longlong_as_double((r << (lz - 11)) + ((long long)(1023 + 10 + e - lz) << 52));
+    return true;
 }
 template <typename T> using Frac = typename std::conditional<sizeof(T) == 4, unsigned, double>::type;
+
+// max(m, |g|), a NaN ignored; the doubles compared as integers
+__device__ __forceinline__ float abs_max(float m, float g) { return fmaxf(m, fabsf(g)); }
+__device__ __forceinline__ double abs_max(double m, double g) {
+    const long long a = __double_as_longlong(g) & 0x7FFFFFFFFFFFFFFFll;
+    return a <= 0x7FF0000000000000ll && a > __double_as_longlong(m) ? __longlong_as_double(a) : m;
+}
 
 // The vortex count and block span of a binning pass: the launch's own, or,
 // when dn is given (a captured step replayed at a growing count), dn[0] with
@@ -239,7 +311,7 @@ __global__ void __launch_bounds__(NT) k_locate(const double* __restrict__ X, con
             }
             make_pos(p, ci, cj, fx, fy, gs[k]);
             pos[q] = p;
-            gm = fmax(gm, (T)fabs(p.g));           // |Gamma| as the record carries it
+            gm = abs_max(gm, p.g);                 // |Gamma| as the record carries it
             const int tx0 = (ci - 1) / TILE, tx1 = (ci + 2) / TILE;
             const int ty0 = (cj - 1) / TILE, ty1 = (cj + 2) / TILE;
             for (int ty = ty0; ty <= ty1; ++ty)
@@ -448,7 +520,6 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : 4) k_scatter(const Pos<T>
 // fixed-point scale 2^sh as a floating-point number, sh in [-60, 100]
 template <typename T> __device__ __forceinline__ T pow2(int sh);
 template <> __device__ __forceinline__ float pow2<float>(int sh) { return __int_as_float((sh + 127) << 23); }
-template <> __device__ __forceinline__ double pow2<double>(int sh) { return __longlong_as_double((long long)(sh + 1023) << 52); }
 
 // x = hi * 2^16 + lo + e, |lo| <= 2^15, |e| <= 1/2, for |x| < 2^38, with FP32
 // adds only (no conversion instructions, which issue at 1/8 rate): adding
@@ -480,15 +551,44 @@ __device__ __forceinline__ void split_hilo(float x, int& hi, int& lo) {
 constexpr int ACC_HALO = 3;
 template <int TILE> struct AccW { static constexpr int value = TILE + 6; };
 
-enum { DEP_SPLIT32 = 0, DEP_F32_64 = 1, DEP_F64_64 = 2 };
+enum { DEP_SPLIT32 = 0, DEP_F32_64 = 1 };
+
+// FP64 records: Gamma on the largest |Gamma|'s scale below 2^58, both weights
+// applied in fixed point, the term rounded once to the tile's scale (drop bits
+// less) and added as two 32-bit words, the low one's carry to the high one.
+// (A 64-bit shared add is a compare-and-swap loop: 3.7 lanes a clock and SM
+// against 11.7 for the two adds with the carry.)  1e6 vortices on 1024^2: 259
+// us with FP64 products and 64-bit adds, 53 us.
+template <int ACC_W>
+__device__ __forceinline__ void deposit_one_fx(const Rec<double>& rc, int gexp, int drop, unsigned* acc_lo,
+                                               unsigned* acc_hi, int* bad) {
+    if (((__double2hiint(rc.g) >> 20) & 0x7FF) == 0x7FF) *bad = 1;      // not finite: the tile becomes NaN
+    FxSplit wx[4], wy[4];
+    fx_m4p(rc.fx, wx);
+    fx_m4p(rc.fy, wy);
+    const FxSplit g = fx_split(fx_from_double(rc.g, gexp));
+    const int base = (rec_ly(rc) - 1 + ACC_HALO) * ACC_W + (rec_lx(rc) - 1 + ACC_HALO);
+    const long long half = (1ll << drop) >> 1, tie = drop ? -1ll : 0ll;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const FxSplit gy = fx_split(fx_weigh(g, wy[b]));
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int node = base + b * ACC_W + a;
+            const long long y = fx_weigh(gy, wx[a]), x = (y + half + ((y >> 63) & tie)) >> drop;   // halves away from 0
+            const unsigned lo = (unsigned)x, old = atomicAdd(&acc_lo[node], lo);
+            atomicAdd(&acc_hi[node], (unsigned)(x >> 32) + (old + lo < old ? 1u : 0u));
+        }
+    }
+}
 
 template <int MODE, int ACC_W, typename T>
 __device__ __forceinline__ void deposit_one(const Rec<T>& rc, T scale, unsigned long long* acc) {
     int* acc_hi = reinterpret_cast<int*>(acc);
     int* acc_lo = reinterpret_cast<int*>(acc) + ACC_W * ACC_W;
     T wx[4], wy[4];
-    m4p_weights<T>(rec_fx(rc), wx);
-    m4p_weights<T>(rec_fy(rc), wy);
+    m4p_weights(rec_fx(rc), wx);
+    m4p_weights(rec_fy(rc), wy);
     const T gs = rc.g * scale;
     const int base = (rec_ly(rc) - 1 + ACC_HALO) * ACC_W + (rec_lx(rc) - 1 + ACC_HALO);
 #pragma unroll
@@ -503,10 +603,8 @@ __device__ __forceinline__ void deposit_one(const Rec<T>& rc, T scale, unsigned 
                 split_hilo((float)x, hi, lo);
                 atomicAdd(&acc_hi[node], hi);
                 atomicAdd(&acc_lo[node], lo);
-            } else if (MODE == DEP_F32_64) {
-                atomicAdd(&acc[node], (unsigned long long)__float2ll_rn((float)x));
             } else {
-                atomicAdd(&acc[node], (unsigned long long)__double2ll_rn((double)x));
+                atomicAdd(&acc[node], (unsigned long long)__float2ll_rn((float)x));
             }
         }
     }
@@ -524,10 +622,9 @@ __device__ __forceinline__ void load_recs(const Rec<T>* __restrict__ recs, int r
     }
 }
 
-// every record of the tile; rc holds this thread's first REC_U (load_recs at 0)
-template <int MODE, int ACC_W, typename T>
-__device__ __forceinline__ void deposit_records(const Rec<T>* __restrict__ recs, int cnt, T scale,
-                                                unsigned long long* acc, Rec<T> (&rc)[REC_U]) {
+// every record of the tile, given to `one`; rc holds this thread's first REC_U (load_recs at 0)
+template <typename T, typename F>
+__device__ __forceinline__ void deposit_records(const Rec<T>* __restrict__ recs, int cnt, Rec<T> (&rc)[REC_U], F one) {
     const int stride = REC_U * (int)blockDim.x;
     for (int r0 = 0; r0 < cnt; r0 += stride) {
         Rec<T> cur[REC_U];
@@ -536,7 +633,7 @@ __device__ __forceinline__ void deposit_records(const Rec<T>* __restrict__ recs,
         if (r0 + stride < cnt) load_recs(recs, r0 + stride, cnt, rc);
 #pragma unroll
         for (int u = 0; u < REC_U; ++u)
-            if (r0 + u * (int)blockDim.x + (int)threadIdx.x < cnt) deposit_one<MODE, ACC_W, T>(cur[u], scale, acc);
+            if (r0 + u * (int)blockDim.x + (int)threadIdx.x < cnt) one(cur[u]);
     }
 }
 
@@ -614,31 +711,56 @@ __global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs
     }
     Rec<T> rc[REC_U];
     if (cnt > 0) load_recs(recs + start, 0, cnt, rc);               // in flight across the barrier
-    const bool split32 = sizeof(T) == 4 && cnt < 65536;
-    const int sh = tile_shift_of((unsigned)cnt, *gmax_all) - (split32 ? 23 : 0);   // 2^61 -> 2^38 when split
-    const T scale = pow2<T>(sh);
-    __syncthreads();
-    if (sizeof(T) == 8) deposit_records<DEP_F64_64, ACC_W>(recs + start, cnt, scale, acc, rc);
-    else if (split32 && cnt >= DEP_SORT_MIN)        // block-uniform
-        deposit_records_banked<ACC_W>(recs + start, cnt, scale, acc, rc, srt, bcnt, bstart);
-    else if (split32) deposit_records<DEP_SPLIT32, ACC_W>(recs + start, cnt, scale, acc, rc);
-    else deposit_records<DEP_F32_64, ACC_W>(recs + start, cnt, scale, acc, rc);
-    __syncthreads();
-    const int* acc_hi = reinterpret_cast<const int*>(acc);
-    const int* acc_lo = reinterpret_cast<const int*>(acc) + ACC_W * ACC_W;
-    const float inv_dx2f = (float)geo.inv_dx2;
-    for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
-        const int lx = i % TILE, ly = i / TILE;
-        const int gi = tx * TILE + lx, gj = ty * TILE + ly;
-        const int node = (ly + ACC_HALO) * ACC_W + lx + ACC_HALO;
-        if (gi < geo.nx && gj < geo.ny) {
-            long long a;
-            if (split32) a = (long long)acc_hi[node] * 65536ll + (long long)acc_lo[node];
-            else a = (long long)acc[node];
-            T v;
-            if (sizeof(T) == 4) v = (T)(__ll2float_rn(a) * pow2<float>(-sh) * inv_dx2f);
-            else v = (T)(ldexp((double)a, -sh) * geo.inv_dx2);
-            w[(size_t)gj * geo.nx + gi] = v;
+    if constexpr (sizeof(T) == 8) {
+        // terms below 2^58 come drop bits finer than the sums, which stay below 2^63
+        const double gmax = *gmax_all;
+        const int gf = (int)(__double_as_longlong(gmax) >> 52) & 0x7FF, gexp = gf ? gf : 1;
+        const int drop = max(32 - __clz(cnt) - 5, 0);             // count < 2^(drop + 5)
+        const int sh = -(fx_exp(gexp) + drop);
+        unsigned* acc_lo = reinterpret_cast<unsigned*>(acc);
+        unsigned* acc_hi = acc_lo + ACC_W * ACC_W;
+        if (threadIdx.x == 0) bstart[0] = 0;                      // set by a record that is not finite
+        __syncthreads();
+        deposit_records<T>(recs + start, cnt, rc,
+                           [&](const Rec<T>& r) { deposit_one_fx<ACC_W>(r, gexp, drop, acc_lo, acc_hi, &bstart[0]); });
+        __syncthreads();
+        for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
+            const int lx = i % TILE, ly = i / TILE;
+            const int gi = tx * TILE + lx, gj = ty * TILE + ly;
+            const int node = (ly + ACC_HALO) * ACC_W + lx + ACC_HALO;
+            if (gi < geo.nx && gj < geo.ny) {
+                const long long a = (long long)(((unsigned long long)acc_hi[node] << 32) | acc_lo[node]);
+                w[(size_t)gj * geo.nx + gi] = bstart[0] ? __longlong_as_double(0x7FF8000000000000ll)
+                                                        : fx_to_double(a, -sh) * geo.inv_dx2;
+            }
+        }
+    } else {
+        const bool split32 = cnt < 65536;
+        const int sh = tile_shift_of((unsigned)cnt, *gmax_all) - (split32 ? 23 : 0);   // 2^61 -> 2^38 when split
+        const T scale = pow2<T>(sh);
+        __syncthreads();
+        if (split32 && cnt >= DEP_SORT_MIN)             // block-uniform
+            deposit_records_banked<ACC_W>(recs + start, cnt, scale, acc, rc, srt, bcnt, bstart);
+        else if (split32)
+            deposit_records<T>(recs + start, cnt, rc,
+                               [&](const Rec<T>& r) { deposit_one<DEP_SPLIT32, ACC_W, T>(r, scale, acc); });
+        else
+            deposit_records<T>(recs + start, cnt, rc,
+                               [&](const Rec<T>& r) { deposit_one<DEP_F32_64, ACC_W, T>(r, scale, acc); });
+        __syncthreads();
+        const int* acc_hi = reinterpret_cast<const int*>(acc);
+        const int* acc_lo = reinterpret_cast<const int*>(acc) + ACC_W * ACC_W;
+        const float inv_dx2f = (float)geo.inv_dx2;
+        for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
+            const int lx = i % TILE, ly = i / TILE;
+            const int gi = tx * TILE + lx, gj = ty * TILE + ly;
+            const int node = (ly + ACC_HALO) * ACC_W + lx + ACC_HALO;
+            if (gi < geo.nx && gj < geo.ny) {
+                long long a;
+                if (split32) a = (long long)acc_hi[node] * 65536ll + (long long)acc_lo[node];
+                else a = (long long)acc[node];
+                w[(size_t)gj * geo.nx + gi] = __ll2float_rn(a) * pow2<float>(-sh) * inv_dx2f;
+            }
         }
     }
 }
@@ -646,8 +768,8 @@ __global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs
 template <typename T>
 __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int ci, int cj, T fx, T fy, T& su, T& sv) {
     T wx[4], wy[4];
-    m4p_weights<T>(fx, wx);
-    m4p_weights<T>(fy, wy);
+    m4p_weights(fx, wx);
+    m4p_weights(fy, wy);
     su = 0;
     sv = 0;
 #pragma unroll
@@ -669,16 +791,23 @@ __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int c
 // one node before and two after, per direction) in shared memory, then every
 // record whose cell lies in the tile (each vortex has exactly one such record)
 // gathers its 4x4 stencil there and writes its result at its original index.
-template <typename T, int TILE>
-__global__ void __launch_bounds__(256) k_interp_tiles(const Rec<T>* __restrict__ recs,
-                                                      const int* __restrict__ tile_start,
-                                                      const unsigned* __restrict__ tile_count, const C_t<T>* __restrict__ uv,
-                                                      Geo geo, T* __restrict__ uq, T* __restrict__ vq, int64_t rec_cap,
-                                                      int64_t nq, int* __restrict__ status) {
-    using C = C_t<T>;
+//
+// FP64: the patch is held in fixed point below 2^58 of its largest value, as
+// centred halves (16 bytes a node, as the doubles), and the forty products of
+// a record are integer multiply-adds (1e6 vortices on 1024^2: 227 -> 67 us); a
+// patch with an infinity or a NaN keeps its doubles and the FP64 sums.
+template <int TILE>
+__global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __restrict__ recs,
+                                                          const int* __restrict__ tile_start,
+                                                          const unsigned* __restrict__ tile_count,
+                                                          const double2* __restrict__ uv, Geo geo,
+                                                          double* __restrict__ uq, double* __restrict__ vq,
+                                                          int64_t rec_cap, int64_t nq, int* __restrict__ status) {
     constexpr int PATCH = TILE + 3;
-    __shared__ C patch[PATCH * PATCH];
+    __shared__ int4 patch[PATCH * PATCH];
+    __shared__ int top;
     const int t = blockIdx.x;
+    if (threadIdx.x == 0) top = 1;
     pdl_wait();
     const int cnt = (int)tile_count[t];
     if (cnt == 0) return;
@@ -689,16 +818,32 @@ __global__ void __launch_bounds__(256) k_interp_tiles(const Rec<T>* __restrict__
     }
     const int tx = t % geo.ntx, ty = t / geo.ntx;
     const int gi0 = tx * TILE - 1, gj0 = ty * TILE - 1;
+    double2* patchd = reinterpret_cast<double2*>(patch);
+    int ef = 1;
     for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {
         const int gi = gi0 + i % PATCH, gj = gj0 + i / PATCH;
-        C v = cmake<C>(T(0), T(0));
+        double2 v = make_double2(0.0, 0.0);
         if (gi >= 0 && gi < geo.nx && gj >= 0 && gj < geo.ny) v = uv[(size_t)gj * geo.nx + gi];
-        patch[i] = v;
+        patchd[i] = v;
+        ef = max(ef, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
     }
+    __syncthreads();                                  // top is initialised
+    ef = __reduce_max_sync(0xffffffffu, ef);
+    if ((threadIdx.x & 31) == 0) atomicMax(&top, ef);
     __syncthreads();
-    constexpr int U = 4;
+    const int emax = top;
+    const bool finite = emax < 2047;                  // block-uniform
+    if (finite) {
+        for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {       // each thread its own nodes, in place
+            const double2 v = patchd[i];
+            const FxSplit a = fx_split(fx_from_double(v.x, emax)), b = fx_split(fx_from_double(v.y, emax));
+            patch[i] = make_int4(a.h, a.l, b.h, b.l);
+        }
+        __syncthreads();
+    }
+    constexpr int U = 2;
     for (int r0 = 0; r0 < cnt; r0 += U * blockDim.x) {
-        Rec<T> rc[U];
+        Rec<double> rc[U];
         bool ok[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {           // loads first (clamped index)
@@ -706,39 +851,61 @@ __global__ void __launch_bounds__(256) k_interp_tiles(const Rec<T>* __restrict__
             ok[u] = r < cnt;
             rc[u] = recs[start + (ok[u] ? r : cnt - 1)];
         }
-#pragma unroll
+#pragma unroll 1
         for (int u = 0; u < U; ++u) {
-            if (!ok[u]) continue;
-            const int lx = rec_lx(rc[u]), ly = rec_ly(rc[u]);
-            if (lx < 0 || lx >= TILE || ly < 0 || ly >= TILE) continue;  // not home
-            T wx[4], wy[4];
-            m4p_weights<T>(rec_fx(rc[u]), wx);
-            m4p_weights<T>(rec_fy(rc[u]), wy);
-            T su = 0, sv = 0;
+            const Rec<double> c = u == 0 ? rc[0] : rc[1];
+            const int lx = rec_lx(c), ly = rec_ly(c);
+            if (!(u == 0 ? ok[0] : ok[1]) || lx < 0 || lx >= TILE || ly < 0 || ly >= TILE) continue;   // not home
+            double ou, ov;
+            if (finite) {
+                FxSplit wx[4], wy[4];
+                fx_m4p(c.fx, wx);
+                fx_m4p(c.fy, wy);
+                long long su = 0, sv = 0;
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const C* row = patch + (ly + b) * PATCH + lx;    // node (lx - 1 + a, ly - 1 + b)
-                T ru = 0, rv = 0;
+                for (int b = 0; b < 4; ++b) {
+                    const int4* row = patch + (ly + b) * PATCH + lx;    // node (lx - 1 + a, ly - 1 + b)
+                    long long hu = 0, hv = 0, tu = 1ll << 29, tv = 1ll << 29;
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const C c = row[a];
-                    ru += wx[a] * c.x;
-                    rv += wx[a] * c.y;
+                    for (int a = 0; a < 4; ++a) {
+                        const int4 q = row[a];
+                        hu += fx_mw(q.x, wx[a].h);
+                        tu += fx_mw(q.x, wx[a].l) + fx_mw(q.y, wx[a].h);
+                        hv += fx_mw(q.z, wx[a].h);
+                        tv += fx_mw(q.z, wx[a].l) + fx_mw(q.w, wx[a].h);
+                    }
+                    su += fx_weigh(fx_split((hu << 1) + (tu >> 30)), wy[b]);
+                    sv += fx_weigh(fx_split((hv << 1) + (tv >> 30)), wy[b]);
                 }
-                su += wy[b] * ru;
-                sv += wy[b] * rv;
+                ou = fx_to_double(su, fx_exp(emax));
+                ov = fx_to_double(sv, fx_exp(emax));
+            } else {
+                double wx[4], wy[4];
+                m4p_weights(c.fx, wx);
+                m4p_weights(c.fy, wy);
+                ou = ov = 0.0;
+                for (int b = 0; b < 4; ++b) {
+                    const double2* row = patchd + (ly + b) * PATCH + lx;
+                    double ru = 0.0, rv = 0.0;
+                    for (int a = 0; a < 4; ++a) {
+                        ru += wx[a] * row[a].x;
+                        rv += wx[a] * row[a].y;
+                    }
+                    ou += wy[b] * ru;
+                    ov += wy[b] * rv;
+                }
             }
-            if (rc[u].q < 0 || rc[u].q >= nq) {
+            if (c.q < 0 || c.q >= nq) {
                 atomicOr(status, ST_INTERNAL);
                 continue;
             }
-            uq[rc[u].q] = su;
-            vq[rc[u].q] = sv;
+            uq[c.q] = ou;
+            vq[c.q] = ov;
         }
     }
 }
 
-// FP32 variant of k_interp_tiles that reads each stencil row with two 16-byte
+// FP32 variant that reads each stencil row with two 16-byte
 // shared loads: the patch is staged twice as node pairs, starting at even and
 // at odd local x, so that the four nodes px .. px + 3 of a row are the pairs
 // E[px / 2], E[px / 2 + 1] (px even) or O[(px - 1) / 2], O[(px + 1) / 2].
@@ -831,8 +998,8 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f32(const Rec<float>* __re
             const Rec<float> rcu = srt[i * 32 + lane];
             const int lx = rec_lx(rcu), ly = rec_ly(rcu);
             float wx[4], wy[4];
-            m4p_weights<float>(rec_fx(rcu), wx);
-            m4p_weights<float>(rec_fy(rcu), wy);
+            m4p_weights(rec_fx(rcu), wx);
+            m4p_weights(rec_fy(rcu), wy);
             const float4* rows = (lx & 1) ? po + (lx - 1) / 2 : pe + lx / 2;   // node px = lx is the first
             float su = 0.f, sv = 0.f;
 #pragma unroll
@@ -898,6 +1065,7 @@ inline Geo make_geo(int nx, int ny, double dx, double x0, double y0, int tile = 
     g.cx = -x0 / dx;
     g.cy = -y0 / dx;
     g.inv_dx2 = 1.0 / (dx * dx);
+    g.recip = dx > 0x1p-500 && dx < 0x1p500;
     const double lx = (double)(nx - 2), ly = (double)(ny - 2);
     memcpy(&g.xlim, &lx, sizeof(double));
     memcpy(&g.ylim, &ly, sizeof(double));

@@ -190,8 +190,8 @@ __global__ void __launch_bounds__(256) k_vic_advect(const Rec<T>* __restrict__ r
         m.q = -1;
         if (lx >= 0 && lx < BIN_TILE && ly >= 0 && ly < BIN_TILE) {
             T wx[4], wy[4];
-            m4p_weights<T>(rec_fx(rc), wx);
-            m4p_weights<T>(rec_fy(rc), wy);
+            m4p_weights(rec_fx(rc), wx);
+            m4p_weights(rec_fy(rc), wy);
             T su = 0, sv = 0;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
