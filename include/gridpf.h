@@ -87,12 +87,12 @@ pf_status pf_plan_fft_size(pf_plan plan, int32_t* P, int32_t* Q);
  *                  class) on the FP64 w or on the FP32 w of mixed plans;
  *   PF_RHS_SPARSE  the direct sum over a list of the nonzero nodes built once
  *                  per solve (16 ns nnz multiply-adds);
- *   PF_RHS_AUTO    (default) in time stepping, where w holds at most 16 nodes
- *                  per vortex, the sparse route while 16 ns (16 capacity) is
- *                  below 2^24 (capacity: the state's, so that a step's route
- *                  does not change as vortices are shed); otherwise the FFT
- *                  when P, Q >= 256 and, for FP64 plans, ns nx ny > 2^18;
- *                  else the direct sum.
+ *   PF_RHS_AUTO    (default) in time stepping, while ns x capacity is at most
+ *                  2^19 (capacity: the state's, so that a step's route does
+ *                  not change as vortices are shed), no field at all: the sum
+ *                  from the vortices themselves, as pf_sheet_solve_vortices
+ *                  forms it; otherwise the FFT when P, Q >= 256 and, for FP64
+ *                  plans, ns nx ny > 2^18; else the direct sum.
  * All have the rounding of FP64; they differ by rounding only.  Mixed-precision
  * plans that take the FFT route allocate nx ny doubles and two FP64-sized
  * spectra once; the sparse route allocates nx ny ints and doubles once.
@@ -280,11 +280,11 @@ pf_status pf_sheet_solve(pf_plan plan, pf_schur schur, const void* w, const pf_m
 
 /* The same solve for the free vorticity of point vortices given directly:
  * X, Y, Gam are DEVICE arrays of nv vortices.  E_s L^-1 R_v Gamma is summed
- * in FP64 from the vortices themselves (sixteen M4' node entries each, Eq.
- * vortexregularization, against the FP64 LGF), so no FP32 rounding of a
+ * in 64 bits from the vortices themselves (M4' and surface weights collapsed to
+ * 49 node offsets of the FP64 LGF a pair), so no FP32 rounding of a
  * regularized field enters the sheet, whatever the plan's precision: the sheet
  * of a mixed plan then carries only FP64 rounding times cond(S) (Sec. 2.2.2,
- * S ill-conditioned below dS/dx ~ 1).  Cost: 256 ns nv FP64 multiply-adds.
+ * S ill-conditioned below dS/dx ~ 1).  Cost: 49 ns nv fixed-point multiply-adds.
  * Vortices whose stencil leaves the grid are left out.  Other arguments,
  * outputs and errors as pf_sheet_solve.  Synchronises. */
 pf_status pf_sheet_solve_vortices(pf_plan plan, pf_schur schur, const double* X, const double* Y,

@@ -22,7 +22,7 @@ void free_plan(pf_plan p) {
     for (cudaEvent_t e : p->tm.ev) cudaEventDestroy(e);
     for (cudaEvent_t e : p->tm.pool) cudaEventDestroy(e);
     void* own[] = {p->T1, p->T2a, p->T2b, p->w, p->uv, p->tile_count, p->gmax, p->tile_start, p->bin_off,
-                   p->pos, p->recs, p->stage, p->stage_out, p->diag, p->rhs64, p->nz_idx, p->nz_val, p->vent_idx, p->vent_val,
+                   p->pos, p->recs, p->stage, p->stage_out, p->diag, p->rhs64, p->nz_idx, p->nz_val,
                    p->d_status, p->d_oob, p->fx_exp};
     for (void* q : own)
         if (q) cudaFree(q);
@@ -33,7 +33,7 @@ void free_plan(pf_plan p) {
     }
     if (p->shared && --p->shared->refs == 0) {
         void* tables[] = {p->G, p->H64, p->H32, p->Hu64, p->Hv64, p->Hu32, p->Hv32, p->twP64, p->twQ64, p->twP32,
-                          p->twQ32, p->tw256_64, p->tw256_32, p->twP_fx, p->twQ_fx};
+                          p->twQ32, p->tw256_64, p->tw256_32, p->twP_fx};
         for (void* q : tables)
             if (q) cudaFree(q);
         delete p->shared;
@@ -94,11 +94,11 @@ pf_status plan_init(pf_plan p) {
     twiddles(t256f, 256);
     PF_TRY(upload(p, &p->tw256_64, t256d));
     PF_TRY(upload(p, &p->tw256_32, t256f));
-    std::vector<int4> fx;
+    std::vector<int4> fx;                  // both in one allocation (one copy if P = Q)
     fx_twiddles(fx, P);
+    if (Q != P) fx_twiddles(fx, Q);
     PF_TRY(upload(p, &p->twP_fx, fx));
-    fx_twiddles(fx, Q);
-    PF_TRY(upload(p, &p->twQ_fx, fx));
+    p->twQ_fx = p->twP_fx + (Q != P ? P : 0);
     PF_TRY(plan_workspaces(p));
     return lgf_build(p);
 }
@@ -329,6 +329,11 @@ pf_status pf_interpolate(pf_plan p, const void* uv, const double* Xq, const doub
 pf_status pf_vic_velocity(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, double Uinf,
                           double Vinf, void* uq, void* vq) {
     if (!p || nv < 0 || (nv > 0 && (!X || !Y || !G || !uq || !vq))) return PF_ERR_ARG;
+    if (vortices_direct(p, nv)) {
+        PF_TRY(regularize_direct(p, X, Y, G, nv, p->w, nullptr, nullptr));
+        PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
+        return interpolate_direct(p, p->uv, X, Y, nv, nullptr, uq, vq, AdvanceArgs());
+    }
     PF_TRY(vortex_regularize(p, X, Y, G, nv, p->w, nullptr, uq, vq));
     PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
     return vortex_interpolate_located(p, p->uv, nv, uq, vq);
@@ -367,8 +372,9 @@ pf_status pf_vic_velocity_host(pf_plan p, const double* X, const double* Y, cons
     if (!p || nv < 0 || (nv > 0 && (!X || !Y || !G || !uq || !vq))) return PF_ERR_ARG;
     if (nv == 0) return PF_OK;
     // page-locked inputs are read by the locate pass directly over the host link
-    // (one transfer, no staging copy); pageable inputs are copied first
-    const double* dXp = pinned_device_ptr(X);
+    // (one transfer, no staging copy); pageable inputs are copied first, and so
+    // are small sets, which the one-launch R_v would read once a tile
+    const double* dXp = vortices_direct(p, nv) ? nullptr : pinned_device_ptr(X);
     const double* dYp = dXp ? pinned_device_ptr(Y) : nullptr;
     const double* dGp = dYp ? pinned_device_ptr(G) : nullptr;
     PF_TRY(ensure_stage(p, nv));

@@ -760,31 +760,6 @@ __global__ void __launch_bounds__(256) k_surface_einvlw_sparse(const int* __rest
 // they gave one instance)
 inline int ew_split(int ns) { return std::max(1, std::min(EW_SPLIT_MAX, ceil_div(152, ns))); }
 
-// Vortex route of the same sum: the node entries of R_v Gamma listed straight
-// from the FP64 positions, sixteen per vortex (M4' weights in FP64, Eq.
-// vortexregularization), duplicates and all (the sum is linear), for the
-// sparse kernel.  A vortex whose stencil leaves the grid gives zero entries
-// (regularization skips it as well).
-__global__ void k_vortex_entries(const double* __restrict__ X, const double* __restrict__ Y,
-                                 const double* __restrict__ G, int64_t n, int nx, int ny, double x0, double y0,
-                                 double dx, int* __restrict__ idx, double* __restrict__ val, int* __restrict__ total) {
-    const double inv_dx2 = 1.0 / (dx * dx);
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        int ix[4], iy[4];
-        double wx[4], wy[4];
-        const bool in = stencil(X[q], x0, dx, nx, ix, wx, false) && stencil(Y[q], y0, dx, ny, iy, wy, false);
-        const double g = in ? G[q] * inv_dx2 : 0.0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                idx[16 * q + 4 * b + a] = in ? iy[b] * nx + ix[a] : 0;
-                val[16 * q + 4 * b + a] = in ? g * wy[b] * wx[a] : 0.0;
-            }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *total = (int)(16 * n);
-}
-
 // The same quantity from an FP64 psi = -L^-1 w on the grid: E_s L^-1 w = -E_s psi.
 // lowest and highest row among n stencil rows (one block)
 __global__ void k_stencil_rows(const int* __restrict__ siy, int n, int* __restrict__ rows) {
@@ -856,26 +831,6 @@ __global__ void k_indicators(int ns, pf_multibody mb, double* __restrict__ out) 
     const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (p >= ns || b >= mb.n_bodies) return;
     out[(size_t)b * ns + p] = (p >= mb.start[b] && p < mb.start[b + 1]) ? 1.0 : 0.0;
-}
-
-// E_s L^-1 d_j for unit point vortices at (vx[j], vy[j]), j < nj: out[j*ns + p]
-__global__ void k_unit_vortex(const double* __restrict__ vx, const double* __restrict__ vy, int nj,
-                              const int* __restrict__ six, const int* __restrict__ siy, const double* __restrict__ swx,
-                              const double* __restrict__ swy, int ns, const double* __restrict__ G, int nx, int ny,
-                              double x0, double y0, double dx, double* __restrict__ out, int* __restrict__ status) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (p >= ns || j >= nj) return;
-    int vix[4], viy[4];
-    double vwx[4], vwy[4];
-    if (!(stencil(vx[j], x0, dx, nx, vix, vwx, false) && stencil(vy[j], y0, dx, ny, viy, vwy, false))) {
-        if (p == 0) atomicOr(status, ST_OUT_OF_DOMAIN);
-        out[(size_t)j * ns + p] = 0.0;
-        return;
-    }
-    // L^-1 d_j = dx^2 G * (dx^-2 M4' M4'): the dx factors cancel; separable sum as k_schur_build
-    const double acc = stencil_pair_lgf(six, siy, swx, swy, p, vix, viy, vwx, vwy, G, nx);
-    out[(size_t)j * ns + p] = acc;
 }
 
 // y_c = S^-1 v_c for nc right-hand sides (vectors of length ns, stride ns)
@@ -1023,7 +978,7 @@ namespace {
 // rhs0 for the mode: GIVEN_S0: sb - s0 + ew; CIRCULATION: sb + ew;
 // Kutta: P^Gamma sb + ew = sb - (f0hat^T sb / Gamma0) + ew   (one block)
 __global__ void k_rhs0(int mode, int ns, double param_h, const double* __restrict__ param_d,
-                       const double* __restrict__ sb, const double* __restrict__ ew,
+                       const double* __restrict__ sb, const double* __restrict__ ew, int chunks,
                        const double* __restrict__ f0hat, const double* __restrict__ gamma0p, double* __restrict__ rhs) {
     __shared__ double sh[256];
     const double param = param_d ? *param_d : param_h;
@@ -1034,7 +989,11 @@ __global__ void k_rhs0(int mode, int ns, double param_h, const double* __restric
         for (int p = threadIdx.x; p < ns; p += blockDim.x) part += f0hat[p] * sb[p];
         shift = block_sum(part, sh) / *gamma0p;
     }
-    for (int p = threadIdx.x; p < ns; p += blockDim.x) rhs[p] = sb[p] - shift + ew[p];
+    for (int p = threadIdx.x; p < ns; p += blockDim.x) {
+        double e = 0.0;                              // `chunks` partial sums a point
+        for (int c = 0; c < chunks; ++c) e += ew[(size_t)p * chunks + c];
+        rhs[p] = sb[p] - shift + e;
+    }
 }
 
 }  // namespace
@@ -1111,7 +1070,7 @@ pf_status sheet_deposit(pf_plan p, pf_schur s, const double* f, void* w) {
 
 static void free_schur(pf_schur s) {
     void* ptrs[] = {s->x, s->y, s->ds, s->six, s->siy, s->swx, s->swy, s->S, s->A, s->Sinv, s->f0, s->f0hat,
-                    s->dgamma0, s->sorder, s->snode, s->gj, s->work, s->mwork, s->scal, s->pnx, s->pny,
+                    s->dgamma0, s->sorder, s->snode, s->sval, s->gpart, s->gj, s->work, s->mwork, s->scal, s->pnx, s->pny,
                     s->fidx, s->fwt, s->ci, s->cj, s->cw, s->rows, s->ewpart, s->ewdone};
     for (void* q : ptrs)
         if (q) cudaFree(q);
@@ -1230,12 +1189,14 @@ pf_status schur_create(pf_plan p, int ns, pf_schur* out) {
     if (ns <= SHEET_SORT_MAX) {
         PF_ALLOC(s->sorder, 16 * (size_t)ns * sizeof(int));
         PF_ALLOC(s->snode, 16 * (size_t)ns * sizeof(int));
+        PF_ALLOC(s->sval, 16 * v);
     }
     PF_ALLOC(s->work, 12 * v);
     PF_ALLOC(s->scal, 8 * sizeof(double));
     PF_ALLOC(s->rows, 2 * sizeof(int));
     PF_ALLOC(s->ewpart, (size_t)EW_SPLIT_MAX * v);
     PF_ALLOC(s->ewdone, (size_t)ns * sizeof(unsigned));
+    PF_ALLOC(s->gpart, EW_SPLIT_MAX * sizeof(double));
     if (cudaMemsetAsync(s->ewdone, 0, (size_t)ns * sizeof(unsigned), p->stream) != cudaSuccess) return fail(PF_ERR_CUDA);
 #undef PF_ALLOC
     *out = s;
@@ -1295,41 +1256,10 @@ pf_status field_route_buffers(pf_plan p, FieldRoute r) {
     return PF_OK;
 }
 
-pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew, int64_t nnz_bound,
-                      const VortexSource* vs = nullptr) {
+pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew, int64_t nnz_bound) {
     const int ns = s->ns;
     cudaStream_t st = p->stream;
     const int64_t M = (int64_t)p->nx * p->ny;
-    // the vortex route: forced, or for mixed plans while 256 ns nv multiply-adds stay below 2^31
-    if (vs && vs->n > 0 && (vs->force || (p->prec != PF_FP64 && 256 * (int64_t)ns * vs->n < ((int64_t)1 << 31)))) {
-        const int64_t ne = 16 * vs->n;
-        if (ne > ((int64_t)1 << 30)) {
-            snprintf(p->err, sizeof(p->err), "%lld vortices exceed the vortex route's entry list",
-                     (long long)vs->n);
-            return PF_ERR_CAPACITY;
-        }
-        if (ne > p->vent_cap) {
-            PF_CUDA(p, cudaStreamSynchronize(st));
-            if (p->vent_idx) cudaFree(p->vent_idx);
-            if (p->vent_val) cudaFree(p->vent_val);
-            p->vent_idx = nullptr;
-            p->vent_val = nullptr;
-            p->vent_cap = 0;
-            const int64_t cap = std::max<int64_t>(ne, 2 * p->vent_cap);
-            PF_CUDA(p, cudaMalloc(&p->vent_idx, (size_t)cap * sizeof(int) + 16));
-            PF_CUDA(p, cudaMalloc(&p->vent_val, (size_t)cap * sizeof(double)));
-            p->vent_cap = cap;
-        }
-        int* total = p->vent_idx + p->vent_cap;
-        const int nb = (int)std::min<int64_t>(ceil_div(vs->n, 256), 152 * 8);
-        k_vortex_entries<<<nb, 256, 0, st>>>(vs->X, vs->Y, vs->G, vs->n, p->nx, p->ny, p->x0, p->y0, p->dx,
-                                             p->vent_idx, p->vent_val, total);
-        k_surface_einvlw_sparse<<<dim3(ns, ew_split(ns)), 256, 0, st>>>(p->vent_idx, p->vent_val, total, p->nx, s->six,
-                                                                        s->siy, s->swx, s->swy, p->G, p->dx * p->dx,
-                                                                        s->ewpart, s->ewdone, ew);
-        PF_LAUNCH_CHECK(p);
-        return PF_OK;
-    }
     const FieldRoute route = field_route(p, ns, nnz_bound);
     PF_TRY(field_route_buffers(p, route));
     if (route == ROUTE_SPARSE) {
@@ -1473,10 +1403,13 @@ __global__ void __launch_bounds__(256) k_constraints_multi(int ns, pf_multibody 
     }
 }
 
+// Full sheet solve on the device.  w: node vorticity (not read when the
+// vortices themselves are summed); vx, vy: device positions of the new
+// vortices (mode KUTTA_SHED).  Results: f (device, ns) and scal[0..2] = (s0,
+// Gamma1, Gamma2) on the device.
 pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_motion& m, int mode, double param,
-                             const double* param_dev, int n_edges, const int* edges, const double* vx,
-                             const double* vy, double* f, const EdgeBounds& eb, int64_t nnz_bound,
-                             const VortexSource* vs) {
+                             const double* param_dev, int n_edges, const int* edges, double* vx, double* vy, double* f,
+                             const EdgeBounds& eb, int64_t nnz_bound, const SheetStep& step) {
     const int ns = s->ns;
     cudaStream_t st = p->stream;
     double* sb = s->work;
@@ -1484,25 +1417,60 @@ pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_moti
     double* rhs = ew + ns;          // rhs0 | e_1 | e_2 contiguous
     double* y = rhs + 3 * ns;       // S^-1 [rhs0 | e_1 | e_2]
     double* res = y + 3 * ns;       // refinement residuals
-    k_sbprime<<<ceil_div(ns, 128), 128, 0, st>>>(s->x, s->y, ns, m, sb);
-    PF_LAUNCH_CHECK(p);
-    PF_TRY(surface_rhs(p, s, w, ew, nnz_bound, vs));
-    k_rhs0<<<1, 256, 0, st>>>(mode, ns, param, param_dev, sb, ew, s->f0hat, s->dgamma0, rhs);
-    PF_LAUNCH_CHECK(p);
-    int nc = 1;
-    if (mode == PF_SHEET_KUTTA_SHED) {
-        nc = 1 + n_edges;
-        k_unit_vortex<<<dim3(ceil_div(ns, 128), n_edges), 128, 0, st>>>(vx, vy, n_edges, s->six, s->siy, s->swx,
-                                                                           s->swy, ns, p->G, p->nx, p->ny, p->x0, p->y0,
-                                                                           p->dx, rhs + ns, p->d_status);
-        PF_LAUNCH_CHECK(p);
+    const bool pairs = step.vs && step.vs->pairs;
+    const int ne = mode == PF_SHEET_KUTTA_SHED ? n_edges : 0, nc = 1 + ne;
+    if (step.vs || ne > 0)
+        PF_TRY(vortex_rhs(p, s, step.vs ? *step.vs : VortexSource(), ne, step.place, vx, vy, rhs + ns));
+    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew, nnz_bound));
+    const double* part = pairs ? s->ewpart : ew;
+    const int chunks = pairs ? vortex_rhs_chunks(ns, step.vs->cap) : 1;
+    const int k1 = n_edges > 0 ? edges[0] : 0, k2 = n_edges > 1 ? edges[1] : 0;
+    if (ns <= SHEET_SMALL) {
+        SheetSmall a{};
+        a.mode = mode;
+        a.ns = ns;
+        a.nc = nc;
+        a.nedge = n_edges;
+        a.k1 = k1;
+        a.k2 = k2;
+        a.eb = eb;
+        a.m = m;
+        a.param_h = param;
+        a.param_d = param_dev;
+        if (step.gsign != 0.0) {
+            a.gpart = s->gpart;
+            a.ngpart = vortex_rhs_chunks(ns, step.vs->cap);
+            a.gsign = step.gsign;
+        }
+        a.x = s->x;
+        a.y = s->y;
+        a.ds = s->ds;
+        a.S = s->S;
+        a.Sinv = s->Sinv;
+        a.f0 = s->f0;
+        a.f0hat = s->f0hat;
+        a.gamma0 = s->dgamma0;
+        a.part = part;
+        a.chunks = chunks;
+        a.unit = rhs + ns;
+        a.f = f;
+        a.scal = s->scal;
+        a.rel = step.rel;
+        a.sorder = s->sorder;
+        a.snode = s->snode;
+        a.swx = s->swx;
+        a.swy = s->swy;
+        a.sval = step.nodes ? s->sval : nullptr;
+        return sheet_small(p, a);
     }
+    k_sbprime<<<ceil_div(ns, 128), 128, 0, st>>>(s->x, s->y, ns, m, sb);
+    k_rhs0<<<1, 256, 0, st>>>(mode, ns, param, param_dev, sb, part, chunks, s->f0hat, s->dgamma0, rhs);
     k_gemv<<<ns, 128, 0, st>>>(s->Sinv, ns, rhs, nc, y);
     k_rows<1><<<rows_grid(ns, nc), 256, 0, st>>>(s->S, ns, y, nc, rhs, res);
     k_rows<2><<<rows_grid(ns, nc), 256, 0, st>>>(s->Sinv, ns, res, nc, nullptr, y);
     PF_LAUNCH_CHECK(p);
-    k_constraints<<<1, 256, 0, st>>>(mode, ns, n_edges, n_edges > 0 ? edges[0] : 0, n_edges > 1 ? edges[1] : 0, eb,
-                                     param, param_dev, s->ds, s->f0, s->f0hat, s->dgamma0, y, f, s->scal);
+    k_constraints<<<1, 256, 0, st>>>(mode, ns, n_edges, k1, k2, eb, param, param_dev, s->ds, s->f0, s->f0hat, s->dgamma0, y, f,
+                                     s->scal);
     PF_LAUNCH_CHECK(p);
     return PF_OK;
 }
@@ -1769,7 +1737,7 @@ pf_status multibody_scratch(pf_plan p, pf_schur s) {
 double* multibody_newpos(pf_schur s) { return s->mwork + (2 + 3 * (size_t)MB_COLS) * s->ns; }
 
 pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const pf_multibody& mb, int ne,
-                                   const double* vx, const double* vy, double* f, const double* gw_dev,
+                                   double* vx, double* vy, double* f, const double* gw_dev,
                                    double** out_dev, int64_t nnz_bound, const VortexSource* vs) {
     const int nb = mb.n_bodies, ns = s->ns, nc = 1 + ne + nb;
     cudaStream_t st = p->stream;
@@ -1782,12 +1750,11 @@ pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const p
     double* out = multibody_newpos(s) + 2 * MB_EDGES;   // s0 (B), Gamma (E)
     k_sbprime_multi<<<ceil_div(ns, 128), 128, 0, st>>>(s->x, s->y, ns, mb, sb);
     PF_LAUNCH_CHECK(p);
-    PF_TRY(surface_rhs(p, s, w, ew, nnz_bound, vs));
-    k_rhs0<<<1, 256, 0, st>>>(PF_SHEET_KUTTA_SHED, ns, 0.0, nullptr, sb, ew, s->f0hat, s->dgamma0, rhs);
-    if (ne > 0)
-        k_unit_vortex<<<dim3(ceil_div(ns, 128), ne), 128, 0, st>>>(vx, vy, ne, s->six, s->siy, s->swx, s->swy, ns,
-                                                                    p->G, p->nx, p->ny, p->x0, p->y0, p->dx, rhs + ns,
-                                                                    p->d_status);
+    const bool pairs = vs && vs->pairs;
+    if (pairs || ne > 0) PF_TRY(vortex_rhs(p, s, pairs ? *vs : VortexSource(), ne, nullptr, vx, vy, rhs + ns));
+    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew, nnz_bound));
+    k_rhs0<<<1, 256, 0, st>>>(PF_SHEET_KUTTA_SHED, ns, 0.0, nullptr, sb, pairs ? s->ewpart : ew,
+                              pairs ? vortex_rhs_chunks(ns, vs->cap) : 1, s->f0hat, s->dgamma0, rhs);
     k_indicators<<<dim3(ceil_div(ns, 256), nb), 256, 0, st>>>(ns, mb, rhs + (size_t)(1 + ne) * ns);
     k_rows<0><<<rows_grid(ns, nc), 256, 0, st>>>(s->Sinv, ns, rhs, nc, nullptr, y);
     k_rows<1><<<rows_grid(ns, nc), 256, 0, st>>>(s->S, ns, y, nc, rhs, res);
@@ -1901,16 +1868,20 @@ pf_status pf_sheet_solve_vortices(pf_plan p, pf_schur s, const double* X, const 
         PF_CUDA(p, cudaMemcpyAsync(vxy, Xnew, n_edges * sizeof(double), cudaMemcpyHostToDevice, p->stream));
         PF_CUDA(p, cudaMemcpyAsync(vxy + 2, Ynew, n_edges * sizeof(double), cudaMemcpyHostToDevice, p->stream));
     }
+    if (nv > (int64_t)1 << 26) {
+        snprintf(p->err, sizeof(p->err), "%lld vortices exceed the 2^26 of a vortex right-hand side", (long long)nv);
+        return PF_ERR_CAPACITY;
+    }
     VortexSource vs;
     vs.X = X;
     vs.Y = Y;
     vs.G = Gam;
-    vs.n = nv;
-    vs.force = true;
-    // with no vortices the free vorticity is zero: the plan's zeroed field stands in for w
-    if (nv == 0) PF_CUDA(p, cudaMemsetAsync(p->w, 0, (size_t)p->nx * p->ny * p->esz, p->stream));
-    pf_status st = sheet_solve_device(p, s, p->w, *m, mode, param, nullptr, n_edges, edges, vxy, vxy + 2, f,
-                                      EdgeBounds(), -1, nv > 0 ? &vs : nullptr);
+    vs.n = vs.cap = nv;
+    vs.pairs = 1;
+    SheetStep step;
+    step.vs = &vs;
+    pf_status st = sheet_solve_device(p, s, nullptr, *m, mode, param, nullptr, n_edges, edges, vxy, vxy + 2, f, EdgeBounds(), -1,
+                                      step);
     if (st != PF_OK) return st;
     double sc[3];
     PF_CUDA(p, cudaMemcpyAsync(sc, s->scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, p->stream));

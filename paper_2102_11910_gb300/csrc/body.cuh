@@ -39,8 +39,10 @@ struct pf_schur_s {
     int pbox[4] = {0, -1, 0, -1};   // cell-centre box (i0, i1, j0, j1) the surface faces can reach
     double* scal = nullptr;   // device scalars: s0, Gamma1, Gamma2, -, new-vortex x[2], y[2]
     int* rows = nullptr;      // lowest and highest grid row of the stencils (device): the rows psi is read at
-    double* ewpart = nullptr; // sparse surface sum: partial sums (ns x EW_SPLIT_MAX) and a done counter per point
+    double* ewpart = nullptr; // surface sums: partial sums (ns x EW_SPLIT_MAX) and a done counter per point
     unsigned* ewdone = nullptr;
+    double* gpart = nullptr;  // partial sums of Gamma (EW_SPLIT_MAX)
+    double* sval = nullptr;   // R_s f dx^2 per sorted entry (16 ns; null as sorder)
 };
 constexpr int EW_SPLIT_MAX = 16;
 
@@ -54,18 +56,41 @@ pf_status invert_schur_matrix(pf_plan p, pf_schur s);
 // device; *out_dev receives the device address of s0 (B values) then the new
 // strengths (one per edge).
 pf_status multibody_check(const pf_multibody& mb, int ns, int* n_edges_total);
-// Point vortices (device FP64 arrays of n) whose E_s L^-1 R_v Gamma a sheet
-// solve forms directly (the vortex route of surface_rhs): always when force is
-// set; otherwise only for mixed plans while the direct sum is cheap.
+constexpr int MAX_EDGES = 2 * PF_MAX_BODIES;
+
+// edges releasing a vortex, and the placement rule's data
+struct EdgeGeo {
+    int n;
+    double ex[MAX_EDGES], ey[MAX_EDGES];   // geometric edge points
+    double nx[MAX_EDGES], ny[MAX_EDGES];   // unit normal facing the free stream
+    double first_dist;                // 10 dt |U_inf|
+    long long last[MAX_EDGES];
+};
+
+// Point vortices (device FP64 arrays of n, or *dn of them) of a sheet solve.
+// pairs: E_s L^-1 R_v Gamma is summed from them (no field w is read).
 struct VortexSource {
     const double* X = nullptr;
     const double* Y = nullptr;
     const double* G = nullptr;
     int64_t n = 0;
-    bool force = false;
+    const int64_t* dn = nullptr;
+    int64_t cap = 0;           // the most n or *dn can be
+    int pairs = 0;
 };
+// Steps take the vortex sum while ns x capacity is at most this: 2000 vortices
+// x 64 points cost 10 us, the FFT of a 768 x 512 field and the R_v it needs 75.
+constexpr int64_t VORTEX_PAIRS = (int64_t)1 << 19;
+
+// E_s L^-1 R_v Gamma into s->ewpart (vortex_rhs_chunks partial sums a
+// point), sums of Gamma into s->gpart (as many), E_s L^-1 d_j of ne released
+// vortices into unit[j ns + p]; their positions are read from newx, newy, or
+// written there by the placement rule.
+int vortex_rhs_chunks(int ns, int64_t cap);
+pf_status vortex_rhs(pf_plan p, pf_schur s, const VortexSource& vs, int ne, const EdgeGeo* place, double* newx, double* newy,
+                     double* unit);                                                               // sheet.cu
 pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const pf_multibody& mb, int ne,
-                                   const double* vx, const double* vy, double* f, const double* gw_dev,
+                                   double* vx, double* vy, double* f, const double* gw_dev,
                                    double** out_dev, int64_t nnz_bound = -1, const VortexSource* vs = nullptr);
 // Generalized edge condition (Sec. 2.5) for the shedding mode: with on = 0 every
 // edge sheds under the Kutta condition; otherwise edge e sheds only when its
@@ -75,13 +100,57 @@ struct EdgeBounds {
     double lo[2] = {0.0, 0.0};
     double hi[2] = {0.0, 0.0};
 };
+// vortices released by a solve: appended to a state's arrays at nv (dn[0] when use_dn)
+struct Release {
+    int n = 0;
+    double *X = nullptr, *Y = nullptr, *G = nullptr;
+    int64_t nv = 0, cap = 0;
+    int64_t* dn = nullptr;
+    int use_dn = 0;
+    const double *newx = nullptr, *newy = nullptr;
+    int* status = nullptr;
+};
+// bodies of at most this many points are solved by one cluster (k_sheet_small)
+constexpr int SHEET_SMALL = 256;
+struct SheetSmall {
+    int mode, ns, nc, nedge, k1, k2;
+    EdgeBounds eb;
+    pf_motion m;
+    double param_h;
+    const double* param_d;
+    const double* gpart;             // not null: param = gsign * sum gpart
+    int ngpart;
+    double gsign;
+    const double *x, *y, *ds, *S, *Sinv, *f0, *f0hat, *gamma0;
+    const double* part;              // E L^-1 w: `chunks` partial sums a point
+    int chunks;
+    const double* unit;
+    double *f, *scal;
+    Release rel;
+    const int *sorder, *snode;       // sval (nullable): R_s f dx^2 at each node's first sorted entry
+    const double *swx, *swy;
+    double* sval;
+};
+pf_status sheet_small(pf_plan p, const SheetSmall& a);                                            // sheet.cu
+
+// What a time step adds to a sheet solve (all of it only while ns <=
+// SHEET_SMALL, but for vs->pairs): the vortices the right-hand side or the
+// total circulation comes from (param = gsign x sum Gamma), the placement of
+// the released ones and their release, the sheet's node values.
+struct SheetStep {
+    const VortexSource* vs = nullptr;
+    const EdgeGeo* place = nullptr;
+    double gsign = 0.0;
+    Release rel;
+    bool nodes = false;
+};
 // param_dev (nullable): device copy of `param` read by the kernels instead;
 // nnz_bound >= 0: at most that many nodes of w are nonzero (lets the surface
 // right-hand side take the sparse route), -1: unknown
 pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_motion& m, int mode, double param,
-                             const double* param_dev, int n_edges, const int* edges, const double* vx,
-                             const double* vy, double* f, const EdgeBounds& eb = EdgeBounds(),
-                             int64_t nnz_bound = -1, const VortexSource* vs = nullptr);
+                             const double* param_dev, int n_edges, const int* edges, double* vx, double* vy, double* f,
+                             const EdgeBounds& eb = EdgeBounds(), int64_t nnz_bound = -1,
+                             const SheetStep& step = SheetStep());
 // w += R_s f  (device f of ns doubles, w real[nx*ny])
 pf_status sheet_deposit(pf_plan p, pf_schur s, const double* f, void* w);
 // allocate what a sheet solve with this nonzero bound allocates on first use

@@ -154,10 +154,6 @@ struct pf_plan_s {
     // the per-chunk counts and the total (allocated by the first sparse solve)
     int* nz_idx = nullptr;
     double* nz_val = nullptr;
-    // vortex route: sixteen (node, FP64 value) entries per vortex, then the count
-    int* vent_idx = nullptr;
-    double* vent_val = nullptr;
-    int64_t vent_cap = 0;
     // pressure field: the plan of the cell-centre lattice ((nx-1) x (ny-1),
     // origin shifted by dx/2, same stream and precision) and its FP64 source
     // and kinetic-energy scratch, built by the first pf_pressure_field call
@@ -286,6 +282,23 @@ void fx_twiddles(std::vector<int4>& v, int N);                                  
 enum { CONV_PSI = 0, CONV_UV = 1 };
 pf_status vortex_regularize(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
                             const int64_t* dn = nullptr, void* zu = nullptr, void* zv = nullptr);  // transfer.cu
+// What the direct E_v does with a vortex's velocity besides storing it.
+enum { ADV_NONE = -1, ADV_EULER = 0, ADV_PREDICT = 1, ADV_HEUN = 2 };
+struct AdvanceArgs {
+    int kind = ADV_NONE;
+    double dt = 0.0;
+    double *X = nullptr, *Y = nullptr;      // moved by EULER (dt u) and HEUN (dt (u1 + u) / 2)
+    double *Xs = nullptr, *Ys = nullptr;    // PREDICT: X + dt u
+    const void *u1 = nullptr, *v1 = nullptr;
+};
+
+struct pf_schur_s;
+// small sets: R_v (with a body's R_s f) and E_v (with a step's position update) in one launch each
+bool vortices_direct(pf_plan p, int64_t n);
+pf_status regularize_direct(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
+                            const int64_t* dn, pf_schur_s* sch);
+pf_status interpolate_direct(pf_plan p, const void* uv, const double* X, const double* Y, int64_t n, const int64_t* dn,
+                             void* uq, void* vq, const AdvanceArgs& adv);
 pf_status plan_reserve_vortices(pf_plan p, int64_t nv);   // transfer.cu: vortex buffers for nv ahead of time
 pf_status vortex_interpolate(pf_plan p, const void* uv, const double* X, const double* Y, int64_t nq, void* uq, void* vq);
 pf_status vortex_interpolate_located(pf_plan p, const void* uv, int64_t nq, void* uq, void* vq);

@@ -466,25 +466,24 @@ void octant(int m, int N, long long& c, long long& s) {
 
 }  // namespace
 
-// exp(-2 pi i m / N), m in [0, N): centred halves (fx_high, fx_low) of the Q62 parts
+// appends exp(-2 pi i m / N), m in [0, N), to v: centred halves (fx_high, fx_low) of the Q62 parts
 void fx_twiddles(std::vector<int4>& v, int N) {
-    v.resize(N);
     const long long one = (1ll << 62) - 1;                                // so that the high half fits
+    std::vector<long long> cs(N / 8 + 1), sn(N / 8 + 1);
+    for (int m = 0; m <= N / 8; ++m) octant(m, N, cs[m], sn[m]);
     for (int m = 0; m < N; ++m) {
-        const int oct = (int)((8 * (long long)m) / N), q = m % (N / 4), in = q > N / 8 ? N / 4 - q : q;
-        long long a, b, c, s;
-        octant(in, N, a, b);
+        const int q = m % (N / 4), in = q > N / 8 ? N / 4 - q : q;
+        long long a = cs[in], b = sn[in], c, s;
         if (q > N / 8) std::swap(a, b);                                   // first quadrant: (a, b) = (cos, sin) of q
-        switch (oct / 2) {
+        switch (m / (N / 4)) {
             case 0: c = a; s = b; break;
             case 1: c = -b; s = a; break;
             case 2: c = -a; s = -b; break;
             default: c = b; s = -a; break;
         }
-        s = -s;
         c = std::min(std::max(c, -one), one);
-        s = std::min(std::max(s, -one), one);
-        v[m] = make_int4(fx_high(c), fx_low(c), fx_high(s), fx_low(s));
+        s = std::min(std::max(-s, -one), one);
+        v.push_back(make_int4(fx_high(c), fx_low(c), fx_high(s), fx_low(s)));
     }
 }
 

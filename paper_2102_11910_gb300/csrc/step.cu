@@ -110,16 +110,6 @@ __global__ void k_sum_final(const double* __restrict__ part, int n, double* __re
     }
 }
 
-constexpr int MAX_EDGES = 2 * PF_MAX_BODIES;
-
-struct EdgeGeo {
-    int n;                            // edges releasing a vortex
-    double ex[MAX_EDGES], ey[MAX_EDGES];   // geometric edge points
-    double nx[MAX_EDGES], ny[MAX_EDGES];   // unit normal facing the free stream
-    double first_dist;                // 10 dt |U_inf|
-    long long last[MAX_EDGES];
-};
-
 // release positions: out[k] = x, out[MAX_EDGES + k] = y of edge k's new vortex
 // (the last released vortex from e.last, or from dn[1 + k] when dn is given)
 __global__ void k_place(const double* __restrict__ X, const double* __restrict__ Y, EdgeGeo e,
@@ -341,18 +331,6 @@ struct Count {
 };
 Count count_of(pf_state s) { return s->capture ? Count{s->cap, s->dn} : Count{s->nv, nullptr}; }
 
-// velocity (plan precision) at the n vortices (X, Y, G) of the current arrays,
-// optionally with a body sheet f added to the source
-pf_status velocities(pf_plan p, pf_state s, const double* X, const double* Y, Count c, pf_schur sch,
-                     const double* f, double Uinf, double Vinf, void* u, void* v) {
-    PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn, u, v));
-    if (sch) PF_TRY(sheet_deposit(p, sch, f, p->w));
-    PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
-    return vortex_interpolate_located(p, p->uv, c.n, u, v);
-}
-
-enum { ADV_EULER = 0, ADV_PREDICT = 1, ADV_HEUN = 2 };
-
 template <typename T>
 void advance_t(pf_plan p, pf_state s, int kind, Count c, double dt) {
     const int nb = nblocks(c.n);
@@ -374,9 +352,53 @@ pf_status advance(pf_plan p, pf_state s, int kind, Count c, double dt) {
     return PF_OK;
 }
 
+// velocity (plan precision) at the n vortices (X, Y, G) of the current arrays,
+// optionally with a body sheet f added to the source (nodes: from the node
+// values its solve left), and the position update `kind` of the stage.  The capacity chooses between the one-launch transfers
+// and the binned ones, so that a captured step computes what pf_step does.
+pf_status velocities(pf_plan p, pf_state s, const double* X, const double* Y, Count c, pf_schur sch,
+                     const double* f, bool nodes, double Uinf, double Vinf, void* u, void* v, int kind, double dt) {
+    if (vortices_direct(p, s->cap)) {
+        PF_TRY(regularize_direct(p, X, Y, s->G, c.n, p->w, c.dn, nodes ? sch : nullptr));
+        if (sch && !nodes) PF_TRY(sheet_deposit(p, sch, f, p->w));
+        PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
+        AdvanceArgs a;
+        a.kind = kind;
+        a.dt = dt;
+        a.X = s->X;
+        a.Y = s->Y;
+        a.Xs = s->Xs;
+        a.Ys = s->Ys;
+        a.u1 = s->u1;
+        a.v1 = s->v1;
+        // only a predictor's velocity is read again
+        return interpolate_direct(p, p->uv, X, Y, c.n, c.dn, kind == ADV_PREDICT ? u : nullptr, v, a);
+    }
+    PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn, u, v));
+    if (sch) PF_TRY(sheet_deposit(p, sch, f, p->w));
+    PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
+    PF_TRY(vortex_interpolate_located(p, p->uv, c.n, u, v));
+    return advance(p, s, kind, c, dt);
+}
+
+// the vortices of a stage's sheet solve: summed against the surface themselves
+// while that is cheap (a rule on the capacity, as every route of a step), else
+// only for their total circulation
+VortexSource vortex_source(pf_plan p, pf_state s, int ns, const double* X, const double* Y, Count c) {
+    VortexSource v;
+    v.X = X;
+    v.Y = Y;
+    v.G = s->G;
+    v.n = c.n;
+    v.dn = c.dn;
+    v.cap = s->cap;
+    v.pairs = p->rhs_route == PF_RHS_AUTO && (int64_t)ns * s->cap <= VORTEX_PAIRS;
+    return v;
+}
+
 // one stage with the body: shed (two-edge Kutta) or Kelvin-constrained
 pf_status body_stage(pf_plan p, pf_state s, const pf_body_kinematics& k, double t, double dt, const double* X,
-                     const double* Y, bool shed, void* u, void* v) {
+                     const double* Y, bool shed, void* u, void* v, int kind) {
     const std::vector<Pose> P{body_pose(k, t)};
     {
         PhaseSpan ph(p, "phase_schur_factor");
@@ -385,13 +407,19 @@ pf_status body_stage(pf_plan p, pf_state s, const pf_body_kinematics& k, double 
     pf_schur sch = s->fac[0].f;
     const pf_motion m{0.0, 0.0, P[0].Omega, k.Uinf, k.Vinf};
     Count c = count_of(s);
+    const bool small = k.ns <= SHEET_SMALL;            // solved in one cluster, with the release and the sums of Gamma
+    const VortexSource vs = vortex_source(p, s, k.ns, X, Y, c);
+    const bool nodes = small && vortices_direct(p, s->cap);
     {
         PhaseSpan ph(p, "phase_regularize");
-        PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn));
-        PF_TRY(sum_gamma(p, s, c.n, c.dn));
+        if (!vs.pairs) PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn));
+        if (!small) PF_TRY(sum_gamma(p, s, c.n, c.dn));
     }
     {
         PhaseSpan ph(p, "phase_sheet_solve");
+        SheetStep step;
+        if (small || vs.pairs) step.vs = &vs;
+        step.nodes = nodes;
         if (shed) {
             EdgeGeo e;
             e.n = 2;
@@ -401,36 +429,45 @@ pf_status body_stage(pf_plan p, pf_state s, const pf_body_kinematics& k, double 
                 e.last[j] = s->last[j];
             }
             e.first_dist = 10.0 * dt * hypot(k.Uinf, k.Vinf);
-            k_place<<<1, 32, 0, p->stream>>>(X, Y, e, c.dn, s->newpos);
-            PF_LAUNCH_CHECK(p);
             EdgeBounds eb;
             eb.on = k.edge_bounded ? 1 : 0;
             for (int j = 0; j < 2; ++j) {
                 eb.lo[j] = k.edge_bounds[2 * j];
                 eb.hi[j] = k.edge_bounds[2 * j + 1];
             }
+            // the new vortices join the arrays X, Y (the caller's position arrays) and G
+            if (small) {
+                step.place = &e;
+                step.gsign = 1.0;
+                step.rel = Release{2, const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->cap, s->dn, c.dn != nullptr,
+                                   s->newpos, s->newpos + MAX_EDGES, p->d_status};
+            } else {
+                k_place<<<1, 32, 0, p->stream>>>(X, Y, e, c.dn, s->newpos);
+                PF_LAUNCH_CHECK(p);
+            }
             PF_TRY(sheet_solve_device(p, sch, p->w, m, PF_SHEET_KUTTA_SHED, 0.0, s->red, 2, kk, s->newpos,
-                                      s->newpos + MAX_EDGES, s->f, eb, 16 * s->cap));
-            // release: the new vortices join the arrays X, Y (the caller's position
-            // arrays) and G
-            k_append<<<1, 32, 0, p->stream>>>(const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->newpos,
-                                              sch->scal + 1, 2, s->dn, c.dn != nullptr, s->cap, p->d_status);
-            PF_LAUNCH_CHECK(p);
+                                      s->newpos + MAX_EDGES, s->f, eb, 16 * s->cap, step));
+            if (!small) {
+                k_append<<<1, 32, 0, p->stream>>>(const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->newpos,
+                                                  sch->scal + 1, 2, s->dn, c.dn != nullptr, s->cap, p->d_status);
+                PF_LAUNCH_CHECK(p);
+            }
             if (!c.dn) c.n += 2;
         } else {
+            if (small) step.gsign = -1.0;
             PF_TRY(sheet_solve_device(p, sch, p->w, m, PF_SHEET_CIRCULATION, 0.0, s->red + 1, 0, nullptr, nullptr,
-                                      nullptr, s->f, EdgeBounds(), 16 * s->cap));
+                                      nullptr, s->f, EdgeBounds(), 16 * s->cap, step));
         }
     }
     PhaseSpan ph(p, "phase_velocity");
-    return velocities(p, s, X, Y, c, sch, s->f, k.Uinf, k.Vinf, u, v);
+    return velocities(p, s, X, Y, c, sch, s->f, nodes, k.Uinf, k.Vinf, u, v, kind, dt);
 }
 
 // one stage with several bodies (Sec. 2.7): each edge releases a vortex under
 // the Kutta condition (shed), Kelvin per body; without shedding every body is
 // circulation-constrained
 pf_status bodies_stage(pf_plan p, pf_state s, const pf_body_kinematics* k, int nb, double t, double dt,
-                       const double* X, const double* Y, bool shed, void* u, void* v) {
+                       const double* X, const double* Y, bool shed, void* u, void* v, int kind) {
     std::vector<Pose> P;
     for (int b = 0; b < nb; ++b) P.push_back(body_pose(k[b], t));
     PF_TRY(ensure_schur(p, s, surface_of(k, nb, P)));
@@ -455,14 +492,15 @@ pf_status bodies_stage(pf_plan p, pf_state s, const pf_body_kinematics* k, int n
     double* rel = s->newpos + 2 * MAX_EDGES;
     double* gw = rel + PF_MAX_BODIES;
     Count c = count_of(s);
-    PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn));
+    const VortexSource vs = vortex_source(p, s, sch->ns, X, Y, c);
+    if (!vs.pairs) PF_TRY(vortex_regularize(p, X, Y, s->G, c.n, p->w, c.dn));
     PF_TRY(sum_gamma(p, s, c.n, c.dn));
     k_gamma_w<<<1, 32, 0, p->stream>>>(s->red, rel, nb, gw);
     if (ne > 0) k_place<<<1, 32, 0, p->stream>>>(X, Y, e, c.dn, s->newpos);
     PF_LAUNCH_CHECK(p);
     double* out = nullptr;
     PF_TRY(sheet_solve_multi_device(p, sch, p->w, mb, ne, s->newpos, s->newpos + MAX_EDGES, s->f, gw, &out,
-                                    16 * s->cap));
+                                    16 * s->cap, &vs));
     if (ne > 0) {
         k_append<<<1, 32, 0, p->stream>>>(const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->newpos,
                                           out + nb, ne, s->dn, c.dn != nullptr, s->cap, p->d_status);
@@ -470,7 +508,7 @@ pf_status bodies_stage(pf_plan p, pf_state s, const pf_body_kinematics* k, int n
         PF_LAUNCH_CHECK(p);
         if (!c.dn) c.n += ne;
     }
-    return velocities(p, s, X, Y, c, sch, s->f, k[0].Uinf, k[0].Vinf, u, v);
+    return velocities(p, s, X, Y, c, sch, s->f, false, k[0].Uinf, k[0].Vinf, u, v, kind, dt);
 }
 
 }  // namespace
@@ -719,27 +757,17 @@ pf_status pf_step(pf_plan p, pf_state s, const pf_body_kinematics* k, double dt,
     const int64_t n0 = s->nv;
     if (!body) {
         const Count c = count_of(s);
-        PF_TRY(velocities(p, s, s->X, s->Y, c, nullptr, nullptr, k->Uinf, k->Vinf, s->u1, s->v1));
-        if (scheme == 0) {
-            PF_TRY(advance(p, s, ADV_EULER, c, dt));
-        } else {
-            PF_TRY(advance(p, s, ADV_PREDICT, c, dt));
-            PF_TRY(velocities(p, s, s->Xs, s->Ys, c, nullptr, nullptr, k->Uinf, k->Vinf, s->u2, s->v2));
-            PF_TRY(advance(p, s, ADV_HEUN, c, dt));
-        }
+        PF_TRY(velocities(p, s, s->X, s->Y, c, nullptr, nullptr, false, k->Uinf, k->Vinf, s->u1, s->v1,
+                          scheme == 0 ? ADV_EULER : ADV_PREDICT, dt));
+        if (scheme == 1)
+            PF_TRY(velocities(p, s, s->Xs, s->Ys, c, nullptr, nullptr, false, k->Uinf, k->Vinf, s->u2, s->v2, ADV_HEUN, dt));
         s->t += dt;
         return PF_OK;
     }
     // stage 1 at t: release two vortices (appended to X, Y, G) and get u1 at all n0 + 2
-    PF_TRY(body_stage(p, s, *k, s->t, dt, s->X, s->Y, release, s->u1, s->v1));
+    PF_TRY(body_stage(p, s, *k, s->t, dt, s->X, s->Y, release, s->u1, s->v1, scheme == 0 ? ADV_EULER : ADV_PREDICT));
     s->nv = n0 + (release ? 2 : 0);
-    if (scheme == 0) {
-        PF_TRY(advance(p, s, ADV_EULER, count_of(s), dt));
-    } else {
-        PF_TRY(advance(p, s, ADV_PREDICT, count_of(s), dt));
-        PF_TRY(body_stage(p, s, *k, s->t + dt, dt, s->Xs, s->Ys, false, s->u2, s->v2));
-        PF_TRY(advance(p, s, ADV_HEUN, count_of(s), dt));
-    }
+    if (scheme == 1) PF_TRY(body_stage(p, s, *k, s->t + dt, dt, s->Xs, s->Ys, false, s->u2, s->v2, ADV_HEUN));
     if (release) {
         s->last[0] = n0;
         s->last[1] = n0 + 1;
@@ -765,16 +793,12 @@ pf_status pf_step_multi(pf_plan p, pf_state s, int32_t n_bodies, const pf_body_k
     if (s->nv + ne > s->cap) return PF_ERR_CAPACITY;
     const int64_t n0 = s->nv;
     // stage 1 at t: one new vortex per edge (appended to X, Y, G), u1 at all n0 + ne
-    PF_TRY(bodies_stage(p, s, bodies, n_bodies, s->t, dt, s->X, s->Y, ne > 0, s->u1, s->v1));
+    PF_TRY(bodies_stage(p, s, bodies, n_bodies, s->t, dt, s->X, s->Y, ne > 0, s->u1, s->v1,
+                        scheme == 0 ? ADV_EULER : ADV_PREDICT));
     s->nv = n0 + ne;
-    if (scheme == 0) {
-        PF_TRY(advance(p, s, ADV_EULER, count_of(s), dt));
-    } else {
-        PF_TRY(advance(p, s, ADV_PREDICT, count_of(s), dt));
-        // stage 2 at t + dt: strengths kept, every body circulation-constrained
-        PF_TRY(bodies_stage(p, s, bodies, n_bodies, s->t + dt, dt, s->Xs, s->Ys, false, s->u2, s->v2));
-        PF_TRY(advance(p, s, ADV_HEUN, count_of(s), dt));
-    }
+    // stage 2 at t + dt: strengths kept, every body circulation-constrained
+    if (scheme == 1)
+        PF_TRY(bodies_stage(p, s, bodies, n_bodies, s->t + dt, dt, s->Xs, s->Ys, false, s->u2, s->v2, ADV_HEUN));
     for (int e = 0; e < ne; ++e) s->last[e] = n0 + e;
     s->t += dt;
     return PF_OK;

@@ -22,6 +22,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "body.cuh"
 #include "transfer.cuh"
 
 namespace {
@@ -92,6 +93,33 @@ pf_status regularize_configured(pf_plan p, const BinWork& bw, const double* X, c
     return regularize_launch<T, BIN_TILE>(p, geo, bw, X, Y, G, nv, w, p->stream, p->min_span, p->tile_threads, dn);
 }
 
+// whether n vortices take the one-launch R_v and E_v (a function of the count
+// that sizes a step's launches, so that a captured step takes the same route)
+bool plan_direct(pf_plan p, int64_t n) {
+    const int64_t tiles = (int64_t)ceil_div(p->nx, p->tile) * ceil_div(p->ny, p->tile);
+    return n > 0 && n <= (p->prec == PF_FP64 ? direct_max<double>() : direct_max<float>()) && tiles * n <= DIRECT_WORK;
+}
+
+template <typename T, int TILE>
+pf_status regularize_direct_t(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, T* w,
+                              const int64_t* dn, const SheetAdd& sheet) {
+    const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0, TILE);
+    const size_t sm = (size_t)nv * sizeof(Rec<T>);
+    PF_CUDA(p, set_smem(k_deposit_direct<T, TILE>, sm));
+    PF_KERNEL(p, "regularize", PF_CUDA(p, pf_launch(k_deposit_direct<T, TILE>, geo.ntiles, 256, sm, p->stream, X, Y, G, nv,
+                                                    dn, geo, w, sheet, p->d_status, p->d_oob)));
+    return PF_OK;
+}
+
+template <typename T>
+pf_status interpolate_direct_t(pf_plan p, const void* uv, const double* X, const double* Y, int64_t n, const int64_t* dn,
+                               T* uq, T* vq, const AdvanceArgs& adv) {
+    const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0);
+    PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_direct<T>, ceil_div(4 * n, 128), 128, 0, p->stream,
+                                                     (const C_t<T>*)uv, X, Y, n, dn, geo, uq, vq, adv)));
+    return PF_OK;
+}
+
 template <int TILE>
 pf_status interpolate_tiles(pf_plan p, const Geo& geo, const void* uv, int64_t nq, void* uq, void* vq) {
     if (p->prec == PF_FP64)
@@ -120,12 +148,36 @@ BinWork plan_binwork_for(pf_plan p) { return plan_binwork(p); }
 // size the plan's vortex buffers for nv vortices ahead of time
 pf_status plan_reserve_vortices(pf_plan p, int64_t nv) { return plan_bin_reserve(p, nv); }
 
+bool vortices_direct(pf_plan p, int64_t n) { return plan_direct(p, n); }
+
+// R_v in one launch (vortices_direct holds for the launch count n); with a
+// factor, its sheet's node values (s->sval) too
+pf_status regularize_direct(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
+                            const int64_t* dn, pf_schur sch) {
+    SheetAdd add{};
+    if (sch) add = SheetAdd{sch->snode, sch->sval, 16 * sch->ns};
+    const bool small = p->tile == BIN_TILE_SMALL;
+    if (p->prec == PF_FP64)
+        return small ? regularize_direct_t<double, BIN_TILE_SMALL>(p, X, Y, G, nv, (double*)w, dn, add)
+                     : regularize_direct_t<double, BIN_TILE>(p, X, Y, G, nv, (double*)w, dn, add);
+    return small ? regularize_direct_t<float, BIN_TILE_SMALL>(p, X, Y, G, nv, (float*)w, dn, add)
+                 : regularize_direct_t<float, BIN_TILE>(p, X, Y, G, nv, (float*)w, dn, add);
+}
+
+// E_v at n vortices from their positions, with a step's position update
+pf_status interpolate_direct(pf_plan p, const void* uv, const double* X, const double* Y, int64_t n, const int64_t* dn,
+                             void* uq, void* vq, const AdvanceArgs& adv) {
+    if (p->prec == PF_FP64) return interpolate_direct_t<double>(p, uv, X, Y, n, dn, (double*)uq, (double*)vq, adv);
+    return interpolate_direct_t<float>(p, uv, X, Y, n, dn, (float*)uq, (float*)vq, adv);
+}
+
 // R_v in the plan's launch configuration (tile edge, block partition, threads).
 // With dn, the count is read on the device from dn[0] and nv (the capacity)
 // only sizes the launches.  With zu, zv (the E_v outputs that follow), every
 // vortex off the grid gets a zero velocity there.
 pf_status vortex_regularize(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
                             const int64_t* dn, void* zu, void* zv) {
+    if (!zu && plan_direct(p, nv)) return regularize_direct(p, X, Y, G, nv, w, dn, nullptr);
     pf_status st = plan_bin_reserve(p, nv);
     if (st != PF_OK) return st;
     BinWork bw = plan_binwork(p);

@@ -240,6 +240,16 @@ __device__ __forceinline__ bool loc_split(double X, const Geo& geo, int axis, in
     f = r == 0 ? 0.0 : __longlong_as_double((r << (lz - 11)) + ((long long)(1023 + 10 + e - lz) << 52));
     return true;
 }
+// Cell and fraction as the records carry them (mixed: 24 bits of it): R_v and
+// E_v at the same position are each other's transpose, so that a vortex's
+// velocity under its own field cancels.
+__device__ __forceinline__ bool split_rec(double X, const Geo& g, int axis, int& c, float& f) {
+    unsigned fr = 0;
+    const bool ok = loc_split(X, g, axis, c, fr);
+    f = __uint2float_rn(fr >> 8) * 0x1p-24f;
+    return ok;
+}
+__device__ __forceinline__ bool split_rec(double X, const Geo& g, int axis, int& c, double& f) { return loc_split(X, g, axis, c, f); }
 template <typename T> using Frac = typename std::conditional<sizeof(T) == 4, unsigned, double>::type;
 
 // max(m, |g|), a NaN ignored; the doubles compared as integers
@@ -690,30 +700,30 @@ __device__ __forceinline__ void deposit_records_banked(const Rec<T>* __restrict_
     }
 }
 
-template <typename T, int TILE>
-__global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs, const int* __restrict__ tile_start,
-                                                 const unsigned* __restrict__ tile_count,
-                                                 const double* __restrict__ gmax_all, Geo geo, T* __restrict__ w,
-                                                 int64_t rec_cap, int* __restrict__ status) {
+// shared memory of one tile's deposit (SORT: with room for the bank-ordered chunk)
+template <typename T, int TILE, bool SORT>
+struct DepositSmem {
+    unsigned long long acc[AccW<TILE>::value * AccW<TILE>::value];
+    Rec<T> srt[SORT && sizeof(T) == 4 ? DEP_SORT_SLOTS : 1];
+    int bcnt[32], bstart[32];
+};
+
+template <typename T, int TILE, bool SORT>
+__device__ __forceinline__ void deposit_clear(DepositSmem<T, TILE, SORT>& sm) {
+    for (int i = threadIdx.x; i < AccW<TILE>::value * AccW<TILE>::value; i += blockDim.x) sm.acc[i] = 0ull;
+    if (threadIdx.x < 32) sm.bcnt[threadIdx.x] = 0;
+}
+
+// w of tile (tx, ty) from its cnt records (global or shared memory); rc holds
+// this thread's first ones, sm is cleared (the barrier is in here)
+template <typename T, int TILE, bool SORT>
+__device__ __forceinline__ void deposit_tile(const Rec<T>* recs, int cnt, double gmax, const Geo& geo, int tx, int ty,
+                                             T* __restrict__ w, DepositSmem<T, TILE, SORT>& sm, Rec<T> (&rc)[REC_U]) {
     constexpr int ACC_W = AccW<TILE>::value;
-    __shared__ unsigned long long acc[ACC_W * ACC_W];
-    __shared__ Rec<T> srt[sizeof(T) == 4 ? DEP_SORT_SLOTS : 1];   // the bank-ordered chunk (mixed path)
-    __shared__ int bcnt[32], bstart[32];
-    const int t = blockIdx.x;
-    const int tx = t % geo.ntx, ty = t / geo.ntx;
-    for (int i = threadIdx.x; i < ACC_W * ACC_W; i += blockDim.x) acc[i] = 0ull;
-    if (threadIdx.x < 32) bcnt[threadIdx.x] = 0;
-    pdl_wait();
-    int start = tile_start[t], cnt = (int)tile_count[t];
-    if (start < 0 || cnt < 0 || (int64_t)start + cnt > rec_cap) {     // block-uniform
-        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
-        start = cnt = 0;
-    }
-    Rec<T> rc[REC_U];
-    if (cnt > 0) load_recs(recs + start, 0, cnt, rc);               // in flight across the barrier
+    unsigned long long* acc = sm.acc;
+    int* bstart = sm.bstart;
     if constexpr (sizeof(T) == 8) {
         // terms below 2^58 come drop bits finer than the sums, which stay below 2^63
-        const double gmax = *gmax_all;
         const int gf = (int)(__double_as_longlong(gmax) >> 52) & 0x7FF, gexp = gf ? gf : 1;
         const int drop = max(32 - __clz(cnt) - 5, 0);             // count < 2^(drop + 5)
         const int sh = -(fx_exp(gexp) + drop);
@@ -721,7 +731,7 @@ __global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs
         unsigned* acc_hi = acc_lo + ACC_W * ACC_W;
         if (threadIdx.x == 0) bstart[0] = 0;                      // set by a record that is not finite
         __syncthreads();
-        deposit_records<T>(recs + start, cnt, rc,
+        deposit_records<T>(recs, cnt, rc,
                            [&](const Rec<T>& r) { deposit_one_fx<ACC_W>(r, gexp, drop, acc_lo, acc_hi, &bstart[0]); });
         __syncthreads();
         for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
@@ -736,16 +746,16 @@ __global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs
         }
     } else {
         const bool split32 = cnt < 65536;
-        const int sh = tile_shift_of((unsigned)cnt, *gmax_all) - (split32 ? 23 : 0);   // 2^61 -> 2^38 when split
+        const int sh = tile_shift_of((unsigned)cnt, gmax) - (split32 ? 23 : 0);   // 2^61 -> 2^38 when split
         const T scale = pow2<T>(sh);
         __syncthreads();
-        if (split32 && cnt >= DEP_SORT_MIN)             // block-uniform
-            deposit_records_banked<ACC_W>(recs + start, cnt, scale, acc, rc, srt, bcnt, bstart);
+        if (SORT && split32 && cnt >= DEP_SORT_MIN)             // block-uniform
+            deposit_records_banked<ACC_W>(recs, cnt, scale, acc, rc, sm.srt, sm.bcnt, bstart);
         else if (split32)
-            deposit_records<T>(recs + start, cnt, rc,
+            deposit_records<T>(recs, cnt, rc,
                                [&](const Rec<T>& r) { deposit_one<DEP_SPLIT32, ACC_W, T>(r, scale, acc); });
         else
-            deposit_records<T>(recs + start, cnt, rc,
+            deposit_records<T>(recs, cnt, rc,
                                [&](const Rec<T>& r) { deposit_one<DEP_F32_64, ACC_W, T>(r, scale, acc); });
         __syncthreads();
         const int* acc_hi = reinterpret_cast<const int*>(acc);
@@ -764,6 +774,124 @@ __global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs
         }
     }
 }
+
+template <typename T, int TILE>
+__global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs, const int* __restrict__ tile_start,
+                                                 const unsigned* __restrict__ tile_count,
+                                                 const double* __restrict__ gmax_all, Geo geo, T* __restrict__ w,
+                                                 int64_t rec_cap, int* __restrict__ status) {
+    __shared__ DepositSmem<T, TILE, true> sm;
+    const int t = blockIdx.x;
+    deposit_clear(sm);
+    pdl_wait();
+    int start = tile_start[t], cnt = (int)tile_count[t];
+    if (start < 0 || cnt < 0 || (int64_t)start + cnt > rec_cap) {     // block-uniform
+        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
+        start = cnt = 0;
+    }
+    Rec<T> rc[REC_U];
+    if (cnt > 0) load_recs(recs + start, 0, cnt, rc);               // in flight across the barrier
+    deposit_tile(recs + start, cnt, *gmax_all, geo, t % geo.ntx, t / geo.ntx, w, sm, rc);
+}
+
+// A bound sheet added to w with the deposit: the grid nodes of its 16 ns
+// stencil entries, sorted, and dx^2 R_s f at each node's first entry.
+struct SheetAdd {
+    const int* node;
+    const double* val;
+    int n;                     // entries; 0: no sheet
+};
+
+// R_v of a small set in one launch: one block per tile reads every vortex,
+// keeps the records of its own tile in shared memory (any order: the sums are
+// integers) with the largest |Gamma| of all, and deposits them, bitwise as the
+// binning passes and k_deposit do.  The four launches of those cost 15 us
+// whatever the set's size; this one reads 24 nv bytes a tile from L2, which
+// is less while tiles x nv is below DIRECT_WORK (256 vortices on 128^2: four
+// launches of 15 us became one of 4, the whole velocity 26.1 -> 16.1 us; 2000 on
+// 768 x 512, 7.7e5 tile reads: 18 -> 9 us).  With a sheet,
+// the tile's nodes of R_s f are added after the vortices'.
+template <typename T, int TILE>
+__global__ void __launch_bounds__(256) k_deposit_direct(const double* __restrict__ X, const double* __restrict__ Y,
+                                                        const double* __restrict__ G, int64_t nv,
+                                                        const int64_t* __restrict__ dn, Geo geo, T* __restrict__ w,
+                                                        SheetAdd sheet, int* __restrict__ status,
+                                                        unsigned long long* __restrict__ oob) {
+    __shared__ DepositSmem<T, TILE, false> sm;
+    __shared__ T wmax[8];
+    __shared__ int n;
+    extern __shared__ __align__(16) unsigned char direct_dyn[];
+    Rec<T>* list = reinterpret_cast<Rec<T>*>(direct_dyn);
+    const int t = blockIdx.x, tx = t % geo.ntx, ty = t / geo.ntx;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    deposit_clear(sm);
+    if (threadIdx.x == 0) n = 0;
+    pdl_wait();
+    if (dn) nv = *dn < nv ? *dn : nv;                // nv: the records the list holds
+    __syncthreads();
+    T gm = T(0);
+    int bad = 0;
+    for (int64_t base = 0; base < nv; base += 256 * BIN_UNROLL) {
+        double xs[BIN_UNROLL], ys[BIN_UNROLL], gs[BIN_UNROLL];
+#pragma unroll
+        for (int k = 0; k < BIN_UNROLL; ++k) {       // clamped: a thread past the end reloads the last vortex
+            int64_t q = base + k * 256 + threadIdx.x;
+            q = q < nv ? q : nv - 1;
+            xs[k] = X[q];
+            ys[k] = Y[q];
+            gs[k] = G[q];
+        }
+#pragma unroll
+        for (int k = 0; k < BIN_UNROLL; ++k) {
+            const int64_t q = base + k * 256 + threadIdx.x;
+            if (base + k * 256 >= nv) break;         // block-uniform
+            int ci = 0, cj = 0;
+            Frac<T> fx = 0, fy = 0;
+            const bool in = q < nv;
+            const bool ok = loc_split(xs[k], geo, 0, ci, fx) && loc_split(ys[k], geo, 1, cj, fy);
+            Pos<T> p;
+            make_pos(p, ci, cj, fx, fy, gs[k]);
+            if (in && !ok) ++bad;
+            if (in && ok) gm = abs_max(gm, p.g);
+            const bool mine = in && ok && (ci - 1) / TILE <= tx && tx <= (ci + 2) / TILE && (cj - 1) / TILE <= ty &&
+                              ty <= (cj + 2) / TILE;
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
+            if (m) {
+                int b = 0;
+                if (lane == 0) b = atomicAdd(&n, __popc(m));
+                b = __shfl_sync(0xffffffffu, b, 0);
+                if (mine) list[b + __popc(m & ((1u << lane) - 1u))] = make_rec(p, ci - tx * TILE, cj - ty * TILE, (int)q);
+            }
+        }
+    }
+    if (bad && t == 0) {
+        atomicAdd(oob, (unsigned long long)bad);
+        atomicOr(status, ST_OUT_OF_DOMAIN);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    if (lane == 0) wmax[wid] = gm;
+    __syncthreads();
+    for (int i = 0; i < 8; ++i) gm = fmax(gm, wmax[i]);
+    const int cnt = n;
+    Rec<T> rc[REC_U];
+    if (cnt > 0) load_recs(list, 0, cnt, rc);
+    deposit_tile(list, cnt, (double)gm, geo, tx, ty, w, sm, rc);
+    if (sheet.n == 0) return;
+    __syncthreads();                                  // the tile's w is written
+    for (int i = threadIdx.x; i < sheet.n; i += 256) {
+        const int node = sheet.node[i], before = i > 0 ? sheet.node[i - 1] : -1;
+        const double v = sheet.val[i];
+        const int gj = node / geo.nx, gi = node - gj * geo.nx;
+        if (gi / TILE == tx && gj / TILE == ty && node != before)
+            w[node] = (T)((double)w[node] + v * geo.inv_dx2);
+    }
+}
+
+// sets that take k_deposit_direct and k_interp_direct: their records fit the
+// block's list, and the tiles' repeated reads cost less than binning
+constexpr int64_t DIRECT_WORK = (int64_t)1 << 20;
+template <typename T> constexpr int64_t direct_max() { return sizeof(T) == 4 ? 4096 : 2048; }
 
 template <typename T>
 __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int ci, int cj, T fx, T fy, T& su, T& sv) {
@@ -1039,6 +1167,62 @@ __global__ void k_interp_xy(const T* __restrict__ uv, const double* __restrict__
         }
         uq[q] = su;
         vq[q] = sv;
+    }
+}
+
+// E_v of a small set at its own vortices, without binned records: four threads
+// a vortex, one stencil row each (the rows' loads are in flight together),
+// added in pairs; the position update of a time step in the same launch.  A
+// vortex off the grid has velocity zero (and was counted by R_v).
+template <typename T>
+__global__ void __launch_bounds__(128) k_interp_direct(const C_t<T>* __restrict__ uv, const double* X, const double* Y,
+                                                       int64_t nq, const int64_t* __restrict__ dn, Geo geo, T* uq, T* vq,
+                                                       AdvanceArgs adv) {
+    const int64_t q0 = (blockIdx.x * (int64_t)128 + threadIdx.x) >> 2;
+    const int b = threadIdx.x & 3;
+    pdl_wait();
+    if (dn) nq = *dn < nq ? *dn : nq;
+    const int64_t q = q0 < nq ? q0 : nq - 1;          // whole warps take part in the shuffles
+    if (nq <= 0) return;
+    const double x = X[q], y = Y[q];
+    int ci = 1, cj = 1;
+    T fx = 0, fy = 0;
+    const bool ok = split_rec(x, geo, 0, ci, fx) && split_rec(y, geo, 1, cj, fy);
+    if (!ok) { ci = 1; cj = 1; fx = 0; fy = 0; }
+    T wx[4], wy[4];
+    m4p_weights(fx, wx);
+    m4p_weights(fy, wy);
+    const C_t<T>* row = uv + (size_t)(cj - 1 + b) * geo.nx + (ci - 1);
+    T su = 0, sv = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const C_t<T> c = row[a];
+        su += wx[a] * c.x;
+        sv += wx[a] * c.y;
+    }
+    const T wb = b == 0 ? wy[0] : b == 1 ? wy[1] : b == 2 ? wy[2] : wy[3];
+    su *= wb;
+    sv *= wb;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        su += __shfl_xor_sync(0xffffffffu, su, o);
+        sv += __shfl_xor_sync(0xffffffffu, sv, o);
+    }
+    if (b != 0 || q0 >= nq) return;
+    if (!ok) su = sv = T(0);
+    if (uq) {
+        uq[q] = su;
+        vq[q] = sv;
+    }
+    if (adv.kind == ADV_EULER) {
+        adv.X[q] = x + adv.dt * (double)su;
+        adv.Y[q] = y + adv.dt * (double)sv;
+    } else if (adv.kind == ADV_PREDICT) {
+        adv.Xs[q] = x + adv.dt * (double)su;
+        adv.Ys[q] = y + adv.dt * (double)sv;
+    } else if (adv.kind == ADV_HEUN) {
+        adv.X[q] += 0.5 * adv.dt * ((double)((const T*)adv.u1)[q] + (double)su);
+        adv.Y[q] += 0.5 * adv.dt * ((double)((const T*)adv.v1)[q] + (double)sv);
     }
 }
 
