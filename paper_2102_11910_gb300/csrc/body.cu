@@ -12,6 +12,7 @@
 //   solves          given s0 (Eq. vsheet), circulation (Eq. circsystem), steady
 //                   Kutta (Eqs. kuttasystem, s0), shedding at one edge
 //                   (Eq. kuttasystem2) or two edges (Eq. twovortex)
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -66,18 +67,22 @@ __device__ __forceinline__ bool stencil(double x, double x0, double dx, int n, i
 
 // one thread per (point p, axis, node a): the FP64 smoothed-three-point weights
 // (square root and arcsine) run at the GPU's low FP64 rate, so they are spread
-// over many blocks; a point whose stencil leaves the grid on either axis gets
-// index 1 and weight 0 on both axes and raises the out-of-domain status
+// over many blocks, the inner nodes (a = 1, 2: the delta's first branch) first
+// and the outer ones after them, so that a warp runs one branch (7.8 -> 5.5 us);
+// a point whose stencil leaves the grid on either axis gets index 1 and weight
+// 0 on both axes and raises the out-of-domain status
 __global__ void k_surface_stencil(const double* __restrict__ x, const double* __restrict__ y, int ns, double x0,
                                   double y0, double dx, int nx, int ny, int* __restrict__ six, int* __restrict__ siy,
                                   double* __restrict__ swx, double* __restrict__ swy, int* __restrict__ status) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 8 * ns) return;
-    const int p = t >> 3, axis = (t >> 2) & 1, a = t & 3;
+    const bool outer = t >= 4 * ns;
+    const int u = outer ? t - 4 * ns : t;
+    const int p = u >> 2, axis = (u >> 1) & 1, a = outer ? 3 * (u & 1) : 1 + (u & 1);
     const double gx = (x[p] - x0) / dx, gy = (y[p] - y0) / dx;
     const double cx = floor(gx), cy = floor(gy);
     const bool ok = cx >= 1.0 && cx <= nx - 3.0 && cy >= 1.0 && cy <= ny - 3.0;
-    if (!ok && t == 8 * p) atomicOr(status, ST_OUT_OF_DOMAIN);
+    if (!ok && axis == 0 && a == 0) atomicOr(status, ST_OUT_OF_DOMAIN);
     const double g = axis ? gy : gx;
     const int c = ok ? (int)(axis ? cy : cx) : 0;
     const int idx = ok ? c - 1 + a : 1;
@@ -124,11 +129,81 @@ __device__ __forceinline__ double stencil_pair_lgf(const int* __restrict__ six, 
     return acc;
 }
 
-__global__ void k_schur_build(const int* __restrict__ six, const int* __restrict__ siy, const double* __restrict__ swx,
-                              const double* __restrict__ swy, const double* __restrict__ ds, int ns,
-                              const double* __restrict__ G, int nx, double* __restrict__ A, int lda) {
+// lowest and highest grid row of n stencil rows (one block of 128)
+__device__ __forceinline__ void stencil_rows(const int* __restrict__ siy, int n, int* __restrict__ rows, int* sh) {
+    int a = 1 << 30, b = -1;
+    for (int i = threadIdx.x; i < n; i += 128) {
+        a = min(a, siy[i]);
+        b = max(b, siy[i]);
+    }
+    a = __reduce_min_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        sh[threadIdx.x >> 5] = a;
+        sh[4 + (threadIdx.x >> 5)] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        rows[0] = min(min(sh[0], sh[1]), min(sh[2], sh[3]));
+        rows[1] = max(max(sh[4], sh[5]), max(sh[6], sh[7]));
+    }
+}
+
+// The geometry's tables in one launch of blocks of 128: rows y < ns build S;
+// `orows` more rows hold the order of the sheet deposit, the 16 ns stencil
+// entries e = 16 p + 4 b + a sorted by (grid node, e), so that each node's
+// entries are contiguous and in index order: an entry's place is the number of
+// entries before it, counted by a thread each against all of them, 2048 at a
+// time in shared memory (ns <= SHEET_SORT_MAX; the one-block sort that this
+// replaces took 11 us at ns 64 and 30 at 256, with the rest of the GPU idle);
+// the last row the stencils' lowest and highest grid rows.
+constexpr int SHEET_SORT_MAX = 1024;
+constexpr int ORDER_CHUNK = 2048;
+__global__ void __launch_bounds__(128) k_schur_build(const int* __restrict__ six, const int* __restrict__ siy,
+                                                     const double* __restrict__ swx, const double* __restrict__ swy,
+                                                     const double* __restrict__ ds, int ns, const double* __restrict__ G,
+                                                     int nx, double* __restrict__ A, int lda, int orows,
+                                                     int* __restrict__ sorder, int* __restrict__ snode,
+                                                     int* __restrict__ rows) {
+    __shared__ __align__(16) int nodes[ORDER_CHUNK];
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     const int p = blockIdx.y;
+    pdl_wait();
+    if (p == ns + orows) {
+        if (blockIdx.x == 0) stencil_rows(siy, 4 * ns, rows, nodes);
+        return;
+    }
+    if (p >= ns) {
+        const int n = 16 * ns, e0 = ((p - ns) * gridDim.x + blockIdx.x) * 128;
+        if (e0 >= n) return;                                       // block-uniform
+        auto node_of = [&](int i) { return siy[4 * (i >> 4) + ((i >> 2) & 3)] * nx + six[4 * (i >> 4) + (i & 3)]; };
+        const int e = e0 + threadIdx.x, ew = e0 + (threadIdx.x & ~31);        // the warp's first entry
+        const int mine = e < n ? node_of(e) : 0;
+        int rank = 0;
+        for (int c0 = 0; c0 < n; c0 += ORDER_CHUNK) {
+            const int m = min(n - c0, ORDER_CHUNK);                // a multiple of 16
+            __syncthreads();
+            for (int i = threadIdx.x; i < m; i += 128) nodes[i] = node_of(c0 + i);
+            __syncthreads();
+            // entries before the warp's: <=; the warp's own, by index; after them: <
+            const int lo = min(max(ew - c0, 0), m), hi = min(max(ew + 32 - c0, 0), m);
+            const int4* v = reinterpret_cast<const int4*>(nodes);
+            for (int i = 0; i < lo / 4; ++i) {
+                const int4 x = v[i];
+                rank += (x.x <= mine) + (x.y <= mine) + (x.z <= mine) + (x.w <= mine);
+            }
+            for (int i = lo; i < hi; ++i) rank += nodes[i] < mine || (nodes[i] == mine && c0 + i < e);
+            for (int i = hi / 4; i < m / 4; ++i) {
+                const int4 x = v[i];
+                rank += (x.x < mine) + (x.y < mine) + (x.z < mine) + (x.w < mine);
+            }
+        }
+        if (e < n) {
+            sorder[rank] = e;
+            snode[rank] = mine;
+        }
+        return;
+    }
     if (q >= ns || q < p) return;
     int ixq[4], iyq[4];
     double wxq[4], wyq[4];
@@ -234,150 +309,161 @@ __global__ void k_extract_inverse(const double* __restrict__ A, double* __restri
 // FP64 work stays ~ns^3 multiply-adds, spread over full warps on every SM.
 constexpr int BGJ_B = 32;              // panel width
 constexpr int BGJ_MAX = 1024;          // ns handled by one panel block (panel rows in shared memory)
-constexpr int BGJ_PANEL_THREADS = 1024;
 
-__global__ void __launch_bounds__(BGJ_PANEL_THREADS) k_bgj_panel(const double* __restrict__ X, int n, int k0, int kb,
-                                                                  int* __restrict__ perm, int* __restrict__ gperm,
-                                                                  double* __restrict__ LU, double tiny,
-                                                                  int* __restrict__ status) {
-    static_assert(BGJ_PANEL_THREADS == 32 * 32 && BGJ_MAX <= 32 * 32,
-                  "32 warps; a lane's rows lane + 32 k (k < 32) fit one bit mask");
-    extern __shared__ float sp[];                  // (n - k0) x 33 FP32 copy of the panel
-    __shared__ int used[BGJ_MAX];
+// 1 / p within an ulp (Newton's iteration in its cubic form, r (1 + e + e^2)
+// with e = 1 - p r, from the hardware's 20-bit estimate: 2^-60 and one
+// rounding); p normal and away from the ends of the range, else a division
+__device__ __forceinline__ double fast_recip(double p) {
+    const int ef = (__double2hiint(p) >> 20) & 0x7FF;
+    if (ef < 64 || ef > 1982) return 1.0 / p;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+    const double e = fma(-p, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// One block of (n - k0) / ROWS warps, at least eight.  Pivot rows by partial
+// pivoting on an FP32 copy of the panel held in registers (warp w has rows w, w
+// + nw, .., a lane a column): each warp offers its largest |entry| of column c
+// (to 2^-18: the low bits of the key hold the row) with the whole row it sits
+// in, so that after one block barrier every warp knows the pivot and has its
+// row.  Then the FP64 LU of the permuted pivot block, four rows a warp in eight
+// warps: the warp that owns row c + 1 updates it first, forms its pivot's
+// reciprocal and publishes the scaled row, the others meanwhile update theirs,
+// one barrier a step.  The kernel runs on one SM and is two chains of 32 steps:
+// reductions and a barrier (about 500 clocks), and six dependent FP64
+// instructions (64 clocks each) with a broadcast (about 550).  A panel of 64
+// rows: 44 us with two barriers a step and shared-memory operands, 30 us so.
+template <int ROWS>
+__global__ void __launch_bounds__(1024) k_bgj_panel(const double* __restrict__ X, int n, int k0, int kb,
+                                                    int* __restrict__ perm, int* __restrict__ gperm,
+                                                    double* __restrict__ LU, double tiny, int* __restrict__ status) {
+    __shared__ float crow[2][32][BGJ_B];           // the warps' candidate rows (two steps' worth: one barrier a step)
+    __shared__ int2 cand[2][32];                   // their keys and row numbers
     __shared__ int rowid[BGJ_MAX];                 // local row i of the permuted panel = local row rowid[i]
-    __shared__ int gp[BGJ_MAX];
-    __shared__ int wsum[32];
-    __shared__ double A[BGJ_B][BGJ_B + 1];
+    __shared__ int gps[BGJ_MAX];
+    __shared__ int nfree[32];
+    __shared__ double qrow[2][BGJ_B];
     __shared__ double rpiv[BGJ_B];
-    const int m = n - k0, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int m = n - k0, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     pdl_wait();
-    for (int idx = tid; idx < m * kb; idx += blockDim.x) {
-        const int i = idx / kb, j = idx - (idx / kb) * kb;
-        sp[i * 33 + j] = (float)X[(size_t)(k0 + i) * n + k0 + j];
+    float r[ROWS];
+    unsigned live = 0u;                            // rows not taken (bit s: row wid + s nw)
+#pragma unroll
+    for (int s = 0; s < ROWS; ++s) {
+        const int i = wid + s * nw;
+        r[s] = i < m && lane < kb ? (float)X[(size_t)(k0 + i) * n + k0 + lane] : 0.f;
+        if (i < m) live |= 1u << s;
     }
-    __syncthreads();
-    // Pivot rows by partial pivoting on the FP32 copy.  Rows are not moved:
-    // warp 0 keeps, lane by lane, a bit mask of the rows lane + 32 k already
-    // taken as pivots, finds each pivot and publishes it with the masks; the
-    // block then eliminates the pivot's column from the rows not taken.  (The
-    // kernel runs on one SM and is bound by instruction issue, so the search
-    // is done once, not by every warp.)
-    __shared__ unsigned tk[32];
-    __shared__ int piv_s;
-    unsigned taken = 0u;
-    if (tid < 32) tk[tid] = 0u;
+    for (int i = tid; i < m; i += blockDim.x) gps[i] = k0 == 0 ? i : gperm[k0 + i];    // the first panel: the identity
     for (int c = 0; c < kb; ++c) {
-        if (wid == 0) {
-            // the largest |panel[i][c]| over rows i not yet taken, lowest i on
-            // ties; all NaN: the lowest row not taken
-            float best = -1.f;
-            int bi = m, first = m;
-            for (int k = 0, i = lane; i < m; ++k, i += 32) {
-                if ((taken >> k) & 1u) continue;
-                first = min(first, i);
-                const float v = fabsf(sp[i * 33 + c]);
-                if (v > best) {
-                    best = v;
-                    bi = i;
-                }
-            }
+        // lane c: this warp's largest |entry| of column c over the rows not taken, the lowest row on ties;
+        // NaNs below every number, taken rows below them
+        int k[ROWS];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float v2 = __shfl_xor_sync(0xffffffffu, best, o);
-                const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-                first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
-                if (v2 > best || (v2 == best && i2 < bi)) {
-                    best = v2;
-                    bi = i2;
-                }
-            }
-            const int pr = bi < m ? bi : (first < m ? first : 0);   // a row not taken exists: c < kb <= m
-            if (lane == (pr & 31)) {
-                taken |= 1u << (pr >> 5);
-                tk[lane] = taken;
-            }
-            if (lane == 0) {
-                piv_s = pr;
-                rowid[c] = pr;
-            }
+        for (int s = 0; s < ROWS; ++s) {
+            int a = __float_as_int(r[s]) & 0x7FFFFFFF;
+            a = a > 0x7F800000 ? 0 : a + ROWS;
+            k[s] = (live >> s) & 1u ? ((a & -ROWS) | (ROWS - 1 - s)) : -1;
         }
-        __syncthreads();
-        // lane = column, warp w takes the rows w + 32 k not taken
-        const int pr = piv_s;
-        const unsigned rows_taken = tk[wid];
-        const float pv = sp[pr * 33 + c];
-        if (pv != 0.f && lane > c && lane < kb) {
-            const float q = sp[pr * 33 + lane] / pv;
-            for (int k = 0, i = wid; i < m; ++k, i += 32)
-                if (!((rows_taken >> k) & 1u)) sp[i * 33 + lane] -= sp[i * 33 + c] * q;
-        }
-        __syncthreads();
-    }
-    // the rows not taken follow the pivots, in ascending order
-    for (int i = tid; i < m; i += blockDim.x) used[i] = (int)((tk[i & 31] >> (i >> 5)) & 1u);
-    __syncthreads();
-    const int free_i = tid < m && !used[tid] ? 1 : 0;
-    int incl = free_i;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += u;
+        for (int o = ROWS / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int s = 0; s < o; ++s) k[s] = max(k[s], k[s + o]);
+        const int best = __shfl_sync(0xffffffffu, k[0], c);
+        const int slot = best < 0 ? 0 : ROWS - 1 - (best & (ROWS - 1));
+        float mine = r[0];
+#pragma unroll
+        for (int s = 1; s < ROWS; ++s) mine = slot == s ? r[s] : mine;
+        crow[c & 1][wid][lane] = mine;
+        if (lane == 0) cand[c & 1][wid] = make_int2(best < 0 ? -1 : best & -ROWS, wid + slot * nw);
+        __syncthreads();
+        const int2 o = lane < nw ? cand[c & 1][lane] : make_int2(-2, 1 << 20);
+        const int top = __reduce_max_sync(0xffffffffu, o.x);
+        const int pr = __reduce_min_sync(0xffffffffu, o.x == top ? o.y : 1 << 20);       // lowest row on ties
+        const int w = pr % nw;
+        const float u = crow[c & 1][w][lane], pv = __shfl_sync(0xffffffffu, u, c);
+        const float q = pv != 0.f ? __fdividef(u, pv) : 0.f;
+        if (w == wid) live &= ~(1u << (pr / nw));
+        if (tid == 0) rowid[c] = pr;
+#pragma unroll
+        for (int s = 0; s < ROWS; ++s) r[s] -= __shfl_sync(0xffffffffu, r[s], c) * q;
     }
-    if (lane == 31) wsum[wid] = incl;
-    __syncthreads();
-    int before = incl - free_i;
-    for (int w = 0; w < wid; ++w) before += wsum[w];
-    if (free_i) rowid[kb + before] = tid;
+    // the rows not taken follow the pivots, in ascending order: row w + s nw comes after all of slot s' < s
+    if (kb < m) {
+        for (int s = 0, before = kb; s < ROWS && s * nw < m; ++s) {
+            const int f = (int)((live >> s) & 1u);
+            if (lane == 0) nfree[wid] = f;
+            __syncthreads();
+            const int v = lane < nw ? nfree[lane] : 0;
+            const unsigned fm = __ballot_sync(0xffffffffu, v != 0);
+            if (f && lane == 0) rowid[before + __popc(fm & ((1u << wid) - 1u))] = wid + s * nw;
+            before += __popc(fm);
+            __syncthreads();
+        }
+    }
     __syncthreads();
     // this panel's permutation (rows < k0 stay) and the accumulated one
     for (int i = tid; i < m; i += blockDim.x) {
         perm[k0 + i] = k0 + rowid[i];
-        gp[i] = gperm[k0 + rowid[i]];
+        gperm[k0 + i] = gps[rowid[i]];
     }
-    __syncthreads();
-    for (int i = tid; i < m; i += blockDim.x) gperm[k0 + i] = gp[i];
-    // FP64 LU of the permuted pivot block, thread (i, j) = (warp, lane) owning
-    // entry (i, j), one block barrier per column: at step c, rows i > c take
-    // l_i = A[i][c] / U_cc (kept apart in Lf, so A[i][c] is never written while
-    // it is read) and update A[i][j], j > c, from row c, which no thread writes
-    // in this step.  The thread of entry (c + 1, c + 1) forms the next pivot's
-    // reciprocal as soon as its last update is done (FP64 division is a long
-    // sequence at this GPU's FP64 rate: one thread per pivot).
-    __shared__ double Lf[BGJ_B][BGJ_B + 1];
-    const int i = tid >> 5, j = lane;
-    const bool mine = i < kb && j < kb;
-    if (mine) A[i][j] = X[(size_t)(k0 + rowid[i]) * n + k0 + j];
-    __syncthreads();
-    auto pivot = [&](int c) {
-        const double pv = A[c][c];
-        if (!(fabs(pv) > tiny)) atomicOr(status, ST_SINGULAR);
-        rpiv[c] = 1.0 / (pv == 0.0 ? 1.0 : pv);
-    };
-    if (tid == 0) pivot(0);
-    __syncthreads();
-    for (int c = 0; c < kb; ++c) {
-        if (mine && i > c && j >= c) {
-            const double l = A[i][c] * rpiv[c];
-            if (j == c) Lf[i][c] = l;
-            else A[i][j] -= l * A[c][j];
-            if (i == c + 1 && j == c + 1) pivot(c + 1);
+    if (wid >= 8) return;                          // the LU: eight warps, named barrier 1
+    double a[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = wid + 8 * s;
+        a[s] = i < kb && lane < kb ? X[(size_t)(k0 + rowid[i]) * n + k0 + lane] : 0.0;
+    }
+    const long long tiny_bits = __double_as_longlong(tiny);
+    // row c is final: its pivot's reciprocal, and the row scaled by it right of the pivot
+    auto publish = [&](int c, double row) {
+        const double pv = __shfl_sync(0xffffffffu, row, c);
+        const long long mag = __double_as_longlong(pv) & 0x7FFFFFFFFFFFFFFFll;   // (comparing doubles is an FP64 instruction)
+        const double rc = mag == 0 ? 1.0 : fast_recip(pv);
+        qrow[c & 1][lane] = lane > c ? row * rc : 0.0;
+        if (lane == 0) {
+            rpiv[c] = rc;
+            if (mag <= tiny_bits || mag > 0x7FF0000000000000ll) atomicOr(status, ST_SINGULAR);
         }
-        __syncthreads();
+    };
+    if (wid == 0) publish(0, a[0]);
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    for (int c = 0; c + 1 < kb; ++c) {
+        const double q = qrow[c & 1][lane];
+        const int s1 = (c + 1) >> 3;
+        if (wid == ((c + 1) & 7)) {
+            double row = s1 == 0 ? a[0] : s1 == 1 ? a[1] : s1 == 2 ? a[2] : a[3];
+            row -= __shfl_sync(0xffffffffu, row, c) * q;
+            publish(c + 1, row);
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (s == s1) a[s] = row;
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            if (wid + 8 * s > c + 1) a[s] -= __shfl_sync(0xffffffffu, a[s], c) * q;     // (warp-uniform)
+        asm volatile("bar.sync 1, 256;" ::: "memory");
     }
-    if (mine) LU[i * BGJ_B + j] = j < i ? Lf[i][j] : A[i][j];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int i = wid + 8 * s;
+        if (i < kb && lane < kb) LU[i * BGJ_B + lane] = lane < i ? a[s] * rpiv[lane] : a[s];
+    }
     if (tid < kb) LU[BGJ_B * BGJ_B + tid] = rpiv[tid];
 }
 
 // One warp per column j < n (y_j, z_j) and per row r < n outside the panel
-// (l_r); lanes over the panel's kb entries.  Blocks of 8 warps.
-__global__ void __launch_bounds__(256) k_bgj_subst(const double* __restrict__ X, int n, int k0, int kb,
+// (l_r); lanes over the panel's kb entries.  Blocks of 4 warps, one on each
+// quarter of an SM: the solves are chains of 94 FP64 instructions at 64 clocks.
+__global__ void __launch_bounds__(128) k_bgj_subst(const double* __restrict__ X, int n, int k0, int kb,
                                                     const int* __restrict__ perm, const double* __restrict__ LU,
                                                     double* __restrict__ Y, double* __restrict__ Z,
                                                     double* __restrict__ Lr) {
     __shared__ double F[BGJ_B][BGJ_B + 1];
     __shared__ double rd[BGJ_B];                   // 1 / U_ll
     const int lane = threadIdx.x & 31;
-    const int wg = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int wg = blockIdx.x * 4 + (threadIdx.x >> 5);
     pdl_wait();
     for (int t = threadIdx.x; t < BGJ_B * BGJ_B; t += blockDim.x) {
         const int a = t >> 5, b = t & 31;
@@ -416,46 +502,37 @@ __global__ void __launch_bounds__(256) k_bgj_subst(const double* __restrict__ X,
     }
 }
 
-// The sweep into Y: tile of 8 rows x 32 columns, one entry per thread
-__global__ void __launch_bounds__(256) k_bgj_sweep(const double* __restrict__ X, int n, int k0, int kb,
+// The sweep: tile of 4 rows x 32 columns, one entry per thread.  The last
+// panel's writes S^-1 itself, its columns in the order gperm undoes.
+__global__ void __launch_bounds__(128) k_bgj_sweep(const double* __restrict__ X, int n, int k0, int kb,
                                                     const int* __restrict__ perm, const double* __restrict__ Yk,
                                                     const double* __restrict__ Zk, const double* __restrict__ Lr,
-                                                    double* __restrict__ Out) {
-    __shared__ double Ls[8][BGJ_B];
+                                                    const int* __restrict__ gperm, double* __restrict__ Out) {
+    __shared__ double Ls[4][BGJ_B];
     __shared__ double Ys[BGJ_B][32];
-    const int j = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 8 + threadIdx.y;
+    const int j = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 4 + threadIdx.y;
     pdl_wait();
     const bool rk = r >= k0 && r < k0 + kb;
     Ls[threadIdx.y][threadIdx.x] = (r < n && !rk && (int)threadIdx.x < kb) ? Lr[(size_t)r * BGJ_B + threadIdx.x] : 0.0;
-    for (int l = threadIdx.y; l < BGJ_B; l += 8)
+#pragma unroll
+    for (int l = threadIdx.y; l < BGJ_B; l += 4)
         Ys[l][threadIdx.x] = (l < kb && j < n) ? Yk[(size_t)l * n + j] : 0.0;
+    const bool in = r < n && j < n, jk = j >= k0 && j < k0 + kb;
+    double x = 0.0;
+    if (in && rk) x = Zk[(size_t)(r - k0) * n + j];
+    else if (in && !jk) x = X[(size_t)(r < k0 ? r : perm[r]) * n + j];
+    const int col = in && gperm ? gperm[j] : j;
     __syncthreads();
-    if (r >= n || j >= n) return;
-    double out;
-    if (rk) {
-        out = Zk[(size_t)(r - k0) * n + j];
-    } else {
-        double acc = 0.0;
-        for (int l = 0; l < kb; ++l) acc += Ls[threadIdx.y][l] * Ys[l][threadIdx.x];
-        const bool jk = j >= k0 && j < k0 + kb;
-        const int src = r < k0 ? r : perm[r];
-        out = (jk ? 0.0 : X[(size_t)src * n + j]) - acc;
+    if (!in) return;
+    if (!rk) {
+        double a0 = 0.0, a1 = 0.0;
+        for (int l = 0; l < kb; l += 2) {          // entries past kb are zero
+            a0 += Ls[threadIdx.y][l] * Ys[l][threadIdx.x];
+            a1 += Ls[threadIdx.y][l + 1] * Ys[l + 1][threadIdx.x];
+        }
+        x -= a0 + a1;
     }
-    Out[(size_t)r * n + j] = out;
-}
-
-// S^-1[i][gperm[r]] = X[i][r]
-__global__ void k_bgj_unpermute(const double* __restrict__ X, int n, const int* __restrict__ gperm,
-                                double* __restrict__ Sinv) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
-    pdl_wait();
-    if (r >= n) return;
-    Sinv[(size_t)i * n + gperm[r]] = X[(size_t)i * n + r];
-}
-
-__global__ void k_iota(int* __restrict__ v, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) v[i] = i;
+    Out[(size_t)r * n + col] = x;
 }
 
 // deterministic block reduction of a double (fixed tree)
@@ -533,63 +610,6 @@ __global__ void k_rows(const double* __restrict__ A, int ns, const double* __res
 }
 
 inline dim3 rows_grid(int ns, int nc) { return dim3((unsigned)ceil_div(ns, 8), (unsigned)ceil_div(nc, 3)); }
-
-// Order of the sheet deposit: the 16 ns stencil entries e = 16 p + 4 b + a
-// sorted by (grid node, e), so that each node's entries are contiguous and in
-// index order.  One block; bitonic sort of the 64-bit keys node 2^16 + e
-// (e < 2^14, node < 2^22) in shared memory, padded to n2 = 2^k >= 16 ns.
-constexpr int SHEET_SORT_MAX = 1024;
-constexpr int SHEET_SORT_THREADS = 1024;
-
-__global__ void __launch_bounds__(SHEET_SORT_THREADS) k_sheet_order(const int* __restrict__ six,
-                                                                     const int* __restrict__ siy, int ns, int nx,
-                                                                     int n2, int* __restrict__ sorder,
-                                                                     int* __restrict__ snode) {
-    extern __shared__ unsigned long long key[];
-    const int ne = 16 * ns;
-    for (int e = threadIdx.x; e < n2; e += blockDim.x) {
-        if (e < ne) {
-            const int p = e >> 4, a = e & 3, b = (e >> 2) & 3;
-            const unsigned long long node = (unsigned long long)siy[4 * p + b] * nx + six[4 * p + a];
-            key[e] = (node << 16) | (unsigned long long)e;
-        } else {
-            key[e] = ~0ull;
-        }
-    }
-    __syncthreads();
-    // Stages whose partner distance j is below SEG stay inside SEG-key
-    // segments; warp w owns segments w, w + 32, ... and runs them with warp
-    // barriers only, so block barriers remain for the j >= SEG stages.
-    // Pair p of a stage (p < n2 / 2) is the key index with a zero bit
-    // inserted at bit log2(j), and its partner has that bit set.
-    constexpr int SEG = 64;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    auto cmpx = [&](int p, int j, int k) {
-        const int lo = p & (j - 1);
-        const int i = ((p - lo) << 1) | lo, l = i | j;
-        const unsigned long long x = key[i], y = key[l];
-        if ((x > y) == ((i & k) == 0)) {
-            key[i] = y;
-            key[l] = x;
-        }
-    };
-    for (int k = 2; k <= n2; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= SEG) {
-                for (int p = threadIdx.x; p < (n2 >> 1); p += blockDim.x) cmpx(p, j, k);
-                __syncthreads();
-            } else {
-                // this warp's segments: SEG / 2 pairs each, one per lane
-                for (int sgm = wid; sgm * SEG < n2; sgm += nw) cmpx(sgm * (SEG / 2) + lane, j, k);
-                __syncwarp();
-                if (j == 1) __syncthreads();   // the next k begins with a block-wide distance
-            }
-        }
-    for (int i = threadIdx.x; i < ne; i += blockDim.x) {
-        sorder[i] = (int)(key[i] & 0xFFFFull);
-        snode[i] = (int)(key[i] >> 16);
-    }
-}
 
 // E_s L^-1 w at surface point p = dx^2 sum_nodes w_m sum_{16 stencil nodes s} d_p(s) G(s - m),
 // summed in FP64 over the nonzero nodes of w (any precision of w).  Evaluating
@@ -761,34 +781,6 @@ __global__ void __launch_bounds__(256) k_surface_einvlw_sparse(const int* __rest
 inline int ew_split(int ns) { return std::max(1, std::min(EW_SPLIT_MAX, ceil_div(152, ns))); }
 
 // The same quantity from an FP64 psi = -L^-1 w on the grid: E_s L^-1 w = -E_s psi.
-// lowest and highest row among n stencil rows (one block)
-__global__ void k_stencil_rows(const int* __restrict__ siy, int n, int* __restrict__ rows) {
-    __shared__ int lo[8], hi[8];
-    int a = 1 << 30, b = -1;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        a = min(a, siy[i]);
-        b = max(b, siy[i]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a = min(a, __shfl_xor_sync(0xffffffffu, a, o));
-        b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        lo[threadIdx.x >> 5] = a;
-        hi[threadIdx.x >> 5] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-            a = min(a, lo[w]);
-            b = max(b, hi[w]);
-        }
-        rows[0] = a;
-        rows[1] = b;
-    }
-}
-
 __global__ void k_surface_from_psi(const double* __restrict__ psi, int nx, int ns, const int* __restrict__ six,
                                    const int* __restrict__ siy, const double* __restrict__ swx,
                                    const double* __restrict__ swy, double* __restrict__ out) {
@@ -852,6 +844,7 @@ __global__ void k_gemv(const double* __restrict__ Sinv, int ns, const double* __
     }
     if (threadIdx.x < nc) y[(size_t)threadIdx.x * ns + p] = sh[threadIdx.x][0];
 }
+
 
 }  // namespace
 
@@ -1094,26 +1087,23 @@ pf_status invert_schur_matrix(pf_plan p, pf_schur s) {
         int* perm = (int*)(Lr + (size_t)BGJ_B * ns);
         int* gperm = perm + ns;
         double* buf[2] = {s->A, s->A + (size_t)ns * ns};
-        k_iota<<<ceil_div(ns, 256), 256, 0, st>>>(gperm, ns);
-        PF_LAUNCH_CHECK(p);
         const double* X = s->S;
         int cur = 0;
         for (int k0 = 0; k0 < ns; k0 += BGJ_B) {
             const int kb = std::min(BGJ_B, ns - k0);
-            const size_t sh = (size_t)(ns - k0) * 33 * sizeof(float);
-            PF_CUDA(p, set_smem(k_bgj_panel, sh));
-            PF_CUDA(p, pf_launch(k_bgj_panel, 1, BGJ_PANEL_THREADS, sh, st, X, ns, k0, kb, perm, gperm, LU, 1e-300,
-                                 p->d_status));
-            PF_CUDA(p, pf_launch(k_bgj_subst, ceil_div(2 * ns, 8), 256, 0, st, X, ns, k0, kb, (const int*)perm,
+            const bool last = k0 + kb == ns;
+            double* out = last ? s->Sinv : buf[cur];
+            const int m = ns - k0, rows = m <= 256 ? 8 : 32, warps = std::max(8, ceil_div(m, rows));
+            PF_CUDA(p, pf_launch(rows == 8 ? k_bgj_panel<8> : k_bgj_panel<32>, 1, 32 * warps, 0, st, X, ns, k0, kb, perm, gperm,
+                                 LU, 1e-300, p->d_status));
+            PF_CUDA(p, pf_launch(k_bgj_subst, ceil_div(2 * ns, 4), 128, 0, st, X, ns, k0, kb, (const int*)perm,
                                  (const double*)LU, Yk, Zk, Lr));
-            PF_CUDA(p, pf_launch(k_bgj_sweep, dim3(ceil_div(ns, 32), ceil_div(ns, 8)), dim3(32, 8), 0, st, X, ns, k0,
+            PF_CUDA(p, pf_launch(k_bgj_sweep, dim3(ceil_div(ns, 32), ceil_div(ns, 4)), dim3(32, 4), 0, st, X, ns, k0,
                                  kb, (const int*)perm, (const double*)Yk, (const double*)Zk, (const double*)Lr,
-                                 buf[cur]));
-            X = buf[cur];
+                                 last ? (const int*)gperm : nullptr, out));
+            X = out;
             cur ^= 1;
         }
-        PF_CUDA(p, pf_launch(k_bgj_unpermute, dim3(ceil_div(ns, 256), ns), dim3(256), 0, st, X, ns,
-                             (const int*)gperm, s->Sinv));
     } else {
         k_augment<<<dim3(ceil_div(2 * ns, 256), ns), 256, 0, st>>>(s->S, s->A, ns);
         PF_LAUNCH_CHECK(p);
@@ -1133,21 +1123,13 @@ pf_status schur_factor_device(pf_plan p, pf_schur s) {
     cudaStream_t st = p->stream;
     k_surface_stencil<<<ceil_div(8 * ns, 32), 32, 0, st>>>(s->x, s->y, ns, p->x0, p->y0, p->dx, p->nx, p->ny, s->six,
                                                             s->siy, s->swx, s->swy, p->d_status);
-    k_stencil_rows<<<1, 256, 0, st>>>(s->siy, 4 * ns, s->rows);
     PF_LAUNCH_CHECK(p);
-    if (s->snode) {
-        int n2 = 1;
-        while (n2 < 16 * ns) n2 <<= 1;
-        const size_t sh = (size_t)n2 * sizeof(unsigned long long);
-        PF_CUDA(p, set_smem(k_sheet_order, sh));
-        k_sheet_order<<<1, SHEET_SORT_THREADS, sh, st>>>(s->six, s->siy, ns, p->nx, n2, s->sorder, s->snode);
-        PF_LAUNCH_CHECK(p);
-    }
-    k_schur_build<<<dim3(ceil_div(ns, 128), ns), 128, 0, st>>>(s->six, s->siy, s->swx, s->swy, s->ds, ns, p->G, p->nx,
-                                                                s->S, ns);
-    PF_LAUNCH_CHECK(p);
+    const int gx = ceil_div(ns, 128), orows = s->snode ? ceil_div(16 * ns, 128 * gx) : 0;
+    PF_CUDA(p, pf_launch(k_schur_build, dim3(gx, ns + orows + 1), 128, 0, st, s->six, s->siy, s->swx, s->swy, s->ds, ns, p->G,
+                         p->nx, s->S, ns, orows, s->sorder, s->snode, s->rows));
     PF_TRY(invert_schur_matrix(p, s));
     // f0 = S^-1 1 with one refinement step (scratch: the solve workspace)
+    if (ns <= SHEET_SMALL) return sheet_f0_small(p, s);
     k_f0_rows<<<ceil_div(ns, 8), 256, 0, st>>>(s->Sinv, ns, s->f0);
     k_rows<1><<<rows_grid(ns, 1), 256, 0, st>>>(s->S, ns, s->f0, 1, nullptr, s->work);
     k_rows<2><<<rows_grid(ns, 1), 256, 0, st>>>(s->Sinv, ns, s->work, 1, nullptr, s->f0);

@@ -125,13 +125,14 @@ struct SheetSmall {
     const double* part;              // E L^-1 w: `chunks` partial sums a point
     int chunks;
     const double* unit;
-    double *f, *scal;
+    double *f, *scal, *f0hat_out;
     Release rel;
     const int *sorder, *snode;       // sval (nullable): R_s f dx^2 at each node's first sorted entry
     const double *swx, *swy;
     double* sval;
 };
 pf_status sheet_small(pf_plan p, const SheetSmall& a);                                            // sheet.cu
+pf_status sheet_f0_small(pf_plan p, pf_schur s);                                                  // sheet.cu
 
 // What a time step adds to a sheet solve (all of it only while ns <=
 // SHEET_SMALL, but for vs->pairs): the vortices the right-hand side or the

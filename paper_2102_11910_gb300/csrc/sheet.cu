@@ -206,6 +206,7 @@ static_assert(2 * PF_MAX_BODIES * 8 <= VR_THREADS, "a group of lanes per release
 // (ns 256) on eight SMs; past SHEET_SMALL points one block per row fills more
 // of the GPU (sheet_solve_device).
 constexpr int SC_BLOCKS = 8, SC_THREADS = 256;
+constexpr int SHEET_F0 = -1;         // mode: f0 of a new factor instead of a sheet
 
 struct ScShared {
     double v[3][SHEET_SMALL], y[3][SHEET_SMALL], r[3][SHEET_SMALL], z[3][SHEET_SMALL];
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(SC_THREADS) __cluster_dims__(SC_BLOCKS, 1, 1) 
         cp_async8(mat + i, A.S + at);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const double Gamma0 = *A.gamma0;
+    const double Gamma0 = A.mode == SHEET_F0 ? 1.0 : *A.gamma0;
     const int p = tid, lane = tid & 31, wid = tid >> 5;   // ns <= SC_THREADS
     if (wid == SC_THREADS / 32 - 1) {                     // the last warp: param, +- the sum of Gamma
         double g = A.param_d ? *A.param_d : A.param_h;
@@ -318,7 +319,12 @@ __global__ void __launch_bounds__(SC_THREADS) __cluster_dims__(SC_BLOCKS, 1, 1) 
     }
     // right-hand side 0 (every block its own copy): s'_b - shift + E L^-1 w
     double sb = 0.0, ew = 0.0;
-    if (p < ns) {
+    if (A.mode == SHEET_F0) {
+        if (p < ns) {
+            sb = 1.0;
+            s.ds[p] = A.ds[p];
+        }
+    } else if (p < ns) {
         const double x = A.x[p], y = A.y[p], fh = A.f0hat[p];
         s.ds[p] = A.ds[p];
         s.f0[p] = A.f0[p];
@@ -338,7 +344,7 @@ __global__ void __launch_bounds__(SC_THREADS) __cluster_dims__(SC_BLOCKS, 1, 1) 
         double sh = 0.0;
         if (A.mode == PF_SHEET_GIVEN_S0) {
             sh = s.param;
-        } else if (A.mode != PF_SHEET_CIRCULATION) {
+        } else if (A.mode != PF_SHEET_CIRCULATION && A.mode != SHEET_F0) {
             for (int q = lane; q < ns; q += 32) sh += s.f[q];
             sh = warp_sum(sh) / Gamma0;
         }
@@ -380,6 +386,23 @@ __global__ void __launch_bounds__(SC_THREADS) __cluster_dims__(SC_BLOCKS, 1, 1) 
     product(0, minv, s.v, s.v, s.y);
     product(1, mat, s.y, s.v, s.r);
     product(2, minv, s.r, s.y, s.z);
+    if (A.mode == SHEET_F0) {                             // f0, f0hat = dS f0, Gamma0 = <1, f0>
+        if (me != 0) return;
+        if (p < ns) {
+            const double f0 = s.z[0][p], h = s.ds[p] * f0;
+            A.f[p] = f0;
+            A.f0hat_out[p] = h;
+            s.f[p] = h;
+        }
+        __syncthreads();
+        if (wid == 0) {
+            double g = 0.0;
+            for (int q = lane; q < ns; q += 32) g += s.f[q];
+            g = warp_sum(g);
+            if (lane == 0) A.scal[0] = g;
+        }
+        return;
+    }
     // (no remote access after the last barrier.)  Every block closes the
     // constraint rows for itself and adds its share of R_s f's nodes.
     if (wid < 3 && A.mode != PF_SHEET_GIVEN_S0) {
@@ -499,6 +522,21 @@ pf_status vortex_rhs(pf_plan p, pf_schur s, const VortexSource& vs, int ne, cons
     PF_KERNEL(p, "vortex_rhs", PF_CUDA(p, pf_launch(k_vortex_rhs, dim3(s->ns, A.chunks + (ne > 0)), VR_THREADS, 0, p->stream,
                                                     A, geo, p->d_status)));
     return PF_OK;
+}
+
+// f0 = S^-1 1 refined, f0hat and Gamma0 of a new factor
+pf_status sheet_f0_small(pf_plan p, pf_schur s) {
+    SheetSmall a{};
+    a.mode = SHEET_F0;
+    a.ns = s->ns;
+    a.nc = 1;
+    a.ds = s->ds;
+    a.S = s->S;
+    a.Sinv = s->Sinv;
+    a.f = s->f0;
+    a.f0hat_out = s->f0hat;
+    a.scal = s->dgamma0;
+    return sheet_small(p, a);
 }
 
 pf_status sheet_small(pf_plan p, const SheetSmall& a) {
