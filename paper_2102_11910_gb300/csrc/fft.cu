@@ -196,14 +196,16 @@ __device__ __forceinline__ void st_pair<float2>(float2* p, float2 a, float2 b) {
     *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
 }
 
-// Row groups (one complex transform of two real rows, or of one row of u + i v)
-// per block of the inverse row pass: one for P >= 1024 (a 1024-row grid's
-// velocity then runs as 1024 blocks of 128 threads, eight an SM, in one wave),
-// two for shorter rows (a whole warp or more a block).  The forward pass keeps
-// two (four rows a block: its 32-byte sectors of T1 written whole by one
-// block measured faster than twice the blocks writing halves).
-template <int R3> struct RowGroups { static constexpr int value = R3 >= 4 ? 1 : 2; };
+// Rows a block of the forward pass: two transforms of two rows each, so that
+// its 32-byte sectors of T1 are written whole by one block (measured faster
+// than twice the blocks writing halves).
 constexpr int FWD_GROUPS = 2;
+
+// Transforms a block of the inverse row pass.  A 32-byte sector of T2 holds
+// four rows' values of one k; a block that reads it for one row makes the pass
+// wait on L2 (2048 x 1800 nodes, velocity: 84 us with one row a block, 33 with
+// two, 36 with four; 768 x 512: 7.9, 6.4; 1024^2: 10.8, 10.8, 11.0).
+constexpr int INV_GROUPS = 2;
 
 template <typename T, int R3>
 __global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const T* __restrict__ w,
@@ -223,7 +225,9 @@ __global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const T* __
     C v[16];
     const int ja = h0 ? j0 : ny - 1, jb = h1 ? j0 + 1 : ny - 1;     // clamped rows: loads never branch
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < 16; ++r) {                   // n >= P / 2 >= nx: padding
+        v[r] = cmake<C>(T(0), T(0));
+        if (r >= 8) continue;
         const int n = t + TP * r;
         const int nc = n < nx ? n : nx - 1;
         const T a = w[(size_t)ja * nx + nc], b = w[(size_t)jb * nx + nc];
@@ -253,7 +257,7 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 // copied into shared memory by cp.async as the block starts, so their loads
 // overlap the column load and the forward transform.
 template <typename T, int R3>
-__global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 ? 32 / R3 : 1) k_cols_r(
+__global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 1) k_cols_r(
     const C_t<T>* __restrict__ T1, C_t<T>* __restrict__ T2a, C_t<T>* __restrict__ T2b, int ny, int nk, int mode,
     const T* __restrict__ H, const T* __restrict__ Hu, const T* __restrict__ Hv, int Hld,
     const C_t<T>* __restrict__ tw256, const C_t<T>* __restrict__ twQ) {
@@ -278,10 +282,12 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 ? 32 / R3 : 1) k_cols_
     }
     C v[16];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {            // clamped row: loads never branch
+    for (int r = 0; r < 16; ++r) {            // clamped row: loads never branch; l >= Q / 2 >= ny: padding
+        v[r] = cmake<C>(T(0), T(0));
+        if (r >= 8) continue;
         const int l = t + TQ * r;
         const C x = T1[spec_at(l < ny ? l : ny - 1, k, nk)];
-        v[r] = l < ny ? x : cmake<C>(T(0), T(0));
+        if (l < ny) v[r] = x;
     }
     fft_strided<C, false, R3>(v, buf, t, tw256, twQ);
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -299,14 +305,14 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 ? 32 / R3 : 1) k_cols_
         }
         fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < 16; ++r) {               // rows past Q / 2 are not kept
             const int l = t + TQ * r;
-            if (l < ny) T2a[spec_at(l, k, nk)] = v[r];
+            if (r < 8 && l < ny) T2a[spec_at(l, k, nk)] = v[r];
             v[r] = keep[spad(l)];                    // written by this thread
         }
         fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
             if (l < ny) T2b[spec_at(l, k, nk)] = v[r];
         }
@@ -318,7 +324,7 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 ? 32 / R3 : 1) k_cols_
         }
         fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
             if (l < ny) T2a[spec_at(l, k, nk)] = v[r];
         }
@@ -327,49 +333,39 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 ? 32 / R3 : 1) k_cols_
 
 // Inverse row pass.  A group's complex row is u_j + i v_j (node velocity: one
 // row, half spectra from T2a and T2b) or psi_j + i psi_{j+1} (two rows of
-// T2a).  Where the block's rows start at an even row, each k's values of two
-// rows come as one 16-byte pair.  FP32 at P = 2048: one group (128 threads) a
-// block at most 64 registers, eight blocks an SM, so a 1024-row grid's 1024
-// blocks run in one wave.
+// T2a).  Two rows' values of a k come as one 16-byte load.  At most 64
+// registers a thread: 1024 threads an SM.
 template <typename T, int R3>
-__global__ void __launch_bounds__(16 * R3 * RowGroups<R3>::value,
-                                  sizeof(T) == 4 && R3 == 8 ? 8 : 1) k_rows_inv_r(const C_t<T>* __restrict__ T2a,
-                                                                             const C_t<T>* __restrict__ T2b,
-                                                                             T* __restrict__ out, int nx, int ny,
-                                                                             int mode, T Uinf, T Vinf,
-                                                                             const C_t<T>* __restrict__ tw256,
-                                                                             const C_t<T>* __restrict__ twP) {
+__global__ void __launch_bounds__(16 * R3 * INV_GROUPS, sizeof(T) == 4 && R3 >= 4 ? 1024 / (16 * R3 * INV_GROUPS) : 1)
+    k_rows_inv_r(const C_t<T>* __restrict__ T2a, const C_t<T>* __restrict__ T2b, T* __restrict__ out, int nx, int ny,
+                 int mode, T Uinf, T Vinf, const C_t<T>* __restrict__ tw256, const C_t<T>* __restrict__ twP) {
     using C = C_t<T>;
-    constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = RowGroups<R3>::value;
+    constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = INV_GROUPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* bufs = reinterpret_cast<C*>(smem_raw);
     const int g = threadIdx.x / TP, t = threadIdx.x % TP;
     const bool uv = mode == CONV_UV;
     const int rows = uv ? G : 2 * G;                 // rows of the block
-    const int r0 = rows * blockIdx.x;                // <= ny - 1: every row read lies in a stored group of four
+    const int r0 = rows * blockIdx.x;                // <= ny - 1: the rows read from it lie in stored groups of four
     const int h = P / 2;
     pdl_wait();
 #pragma unroll 2
     for (int k = threadIdx.x; k <= h; k += blockDim.x) {
-        C a[2], b[2];
-        const size_t at = spec_at(r0, k, NK);
+        C a[G], b[G];
         if (uv) {                                     // group gg takes row r0 + gg
-            if (G == 2) {
-                ld_pair(T2a + at, a[0], a[1]);
-                ld_pair(T2b + at, b[0], b[1]);
-            } else {                                  // one row a block: r0 may be odd
-                a[0] = T2a[at];
-                b[0] = T2b[at];
-            }
+            const size_t at = spec_at(r0, k, NK);       // r0 is even
+            ld_pair(T2a + at, a[0], a[1]);
+            ld_pair(T2b + at, b[0], b[1]);
 #pragma unroll
             for (int gg = 0; gg < G; ++gg)
                 if (r0 + gg >= ny) a[gg] = b[gg] = cmake<C>(T(0), T(0));
         } else {                                      // group gg takes rows r0 + 2 gg, r0 + 2 gg + 1
 #pragma unroll
             for (int gg = 0; gg < G; ++gg) {
-                ld_pair(T2a + at + 2 * gg, a[gg], b[gg]);
-                if (r0 + 2 * gg >= ny) a[gg] = cmake<C>(T(0), T(0));
-                if (r0 + 2 * gg + 1 >= ny) b[gg] = cmake<C>(T(0), T(0));
+                const int j = r0 + 2 * gg;
+                ld_pair(T2a + spec_at(j < ny ? j : r0, k, NK), a[gg], b[gg]);
+                if (j >= ny) a[gg] = cmake<C>(T(0), T(0));
+                if (j + 1 >= ny) b[gg] = cmake<C>(T(0), T(0));
             }
         }
 #pragma unroll
@@ -393,7 +389,7 @@ __global__ void __launch_bounds__(16 * R3 * RowGroups<R3>::value,
         if (j < ny) {
             C* o = reinterpret_cast<C*>(out) + (size_t)j * nx;
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
+            for (int r = 0; r < 8; ++r) {
                 const int n = t + TP * r;
                 if (n < nx) o[n] = cmake<C>(v[r].x + Uinf, v[r].y + Vinf);
             }
@@ -401,7 +397,7 @@ __global__ void __launch_bounds__(16 * R3 * RowGroups<R3>::value,
     } else {
         const int ja = r0 + 2 * g, jb = ja + 1;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < 8; ++r) {
             const int n = t + TP * r;
             if (n < nx) {
                 if (ja < ny) out[(size_t)ja * nx + n] = v[r].x;
@@ -424,12 +420,10 @@ static pf_status conv_solve_r(pf_plan p, const T* w, T* out, int mode, T Uinf, T
     using C = C_t<T>;
     constexpr int P = 256 * R3P, Q = 256 * R3Q;
     const int nx = p->nx, ny = p->ny;
-    constexpr int G = RowGroups<R3P>::value;
-    const size_t sf = FWD_GROUPS * (size_t)SBuf<P>::size * sizeof(C), sr = G * (size_t)SBuf<P>::size * sizeof(C);
+    const size_t sf = FWD_GROUPS * (size_t)SBuf<P>::size * sizeof(C);
     const size_t sc = 2 * (size_t)SBuf<Q>::size * sizeof(C) + 2 * (size_t)((Q / 2 + 1 + 3) / 4 * 4) * sizeof(T);
     PF_CUDA(p, set_smem(k_rows_fwd_r<T, R3P>, sf));
     PF_CUDA(p, set_smem(k_cols_r<T, R3Q>, sc));
-    PF_CUDA(p, set_smem(k_rows_inv_r<T, R3P>, sr));
     C* T1 = reinterpret_cast<C*>(ws.T1);
     C* T2a = reinterpret_cast<C*>(ws.T2a);
     C* T2b = reinterpret_cast<C*>(ws.T2b);
@@ -437,9 +431,11 @@ static pf_status conv_solve_r(pf_plan p, const T* w, T* out, int mode, T Uinf, T
                                                       nx, ny, tw256, twP)));
     PF_KERNEL(p, "fft_cols_conv", PF_CUDA(p, pf_launch(k_cols_r<T, R3Q>, P / 2 + 1, 16 * R3Q, sc, p->stream, T1, T2a,
                                                        T2b, ny, P / 2 + 1, mode, H, Hu, Hv, p->Hld, tw256, twQ)));
-    const int nb = mode == CONV_UV ? ceil_div(ny, G) : ceil_div(ny, 2 * G);
-    PF_KERNEL(p, "fft_rows_inv", PF_CUDA(p, pf_launch(k_rows_inv_r<T, R3P>, nb, 16 * R3P * G, sr, p->stream, T2a, T2b, out,
-                                                      nx, ny, mode, Uinf, Vinf, tw256, twP)));
+    const int nb = mode == CONV_UV ? ceil_div(ny, INV_GROUPS) : ceil_div(ny, 2 * INV_GROUPS);
+    const size_t sr = INV_GROUPS * (size_t)SBuf<P>::size * sizeof(C);
+    PF_CUDA(p, set_smem(k_rows_inv_r<T, R3P>, sr));
+    PF_KERNEL(p, "fft_rows_inv", PF_CUDA(p, pf_launch(k_rows_inv_r<T, R3P>, nb, 16 * R3P * INV_GROUPS, sr, p->stream, T2a, T2b,
+                                                      out, nx, ny, mode, Uinf, Vinf, tw256, twP)));
     return PF_OK;
 }
 
