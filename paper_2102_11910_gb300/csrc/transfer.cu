@@ -197,16 +197,16 @@ pf_status vortex_interpolate_located(pf_plan p, const void* uv, int64_t nq, void
 
 pf_status vortex_interpolate(pf_plan p, const void* uv, const double* X, const double* Y, int64_t nq, void* uq, void* vq) {
     if (nq == 0) return PF_OK;
-    const int nb = (int)std::min<int64_t>(ceil_div(nq, 256), 152 * 16);
     const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0);
-    if (p->prec == PF_FP64)
-        PF_KERNEL(p, "interpolate", k_interp_xy<double><<<nb, 256, 0, p->stream>>>((const double*)uv, X, Y, nq, geo,
-                                                                                   (double*)uq, (double*)vq,
-                                                                                   p->d_status, p->d_oob));
-    else
-        PF_KERNEL(p, "interpolate", k_interp_xy<float><<<nb, 256, 0, p->stream>>>((const float*)uv, X, Y, nq, geo,
-                                                                                  (float*)uq, (float*)vq, p->d_status,
-                                                                                  p->d_oob));
+    if (p->prec == PF_FP64) {
+        const int nb = (int)std::min<int64_t>(ceil_div(nq, 256), 152 * 16);
+        PF_KERNEL(p, "interpolate", k_interp_xy_f64<<<nb, 256, 0, p->stream>>>((const double*)uv, X, Y, nq, geo, (double*)uq,
+                                                                               (double*)vq, p->d_status, p->d_oob));
+    } else {
+        const int nb = (int)std::min<int64_t>(ceil_div(nq, XY_THREADS), 152 * 16);
+        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_xy_f32, nb, XY_THREADS, 0, p->stream, (const float2*)uv, X, Y,
+                                                         nq, geo, (float*)uq, (float*)vq, p->d_status, p->d_oob)));
+    }
     return PF_OK;
 }
 

@@ -1149,24 +1149,94 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f32(const Rec<float>* __re
     }
 }
 
-// E_v at arbitrary points
-template <typename T>
-__global__ void k_interp_xy(const T* __restrict__ uv, const double* __restrict__ X, const double* __restrict__ Y,
-                            int64_t nq, Geo geo, T* __restrict__ uq, T* __restrict__ vq, int* __restrict__ status,
-                            unsigned long long* __restrict__ oob) {
+// E_v at arbitrary points, FP64: a thread a point.
+__global__ void __launch_bounds__(256) k_interp_xy_f64(const double* __restrict__ uv, const double* __restrict__ X,
+                                                       const double* __restrict__ Y, int64_t nq, Geo geo,
+                                                       double* __restrict__ uq, double* __restrict__ vq,
+                                                       int* __restrict__ status, unsigned long long* __restrict__ oob) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nq; q += (int64_t)gridDim.x * blockDim.x) {
         int ci = 0, cj = 0;
-        T fx = 0, fy = 0;
-        T su = 0, sv = 0;
-        if (split(X[q], geo.x0, geo.dx, geo.inv_dx, geo.cx, geo.nx, geo.xlim, ci, fx) &&
-            split(Y[q], geo.y0, geo.dx, geo.inv_dx, geo.cy, geo.ny, geo.ylim, cj, fy)) {
-            gather16<T>(uv, geo.nx, ci, cj, fx, fy, su, sv);
+        double fx = 0, fy = 0, su = 0, sv = 0;
+        if (loc_split(X[q], geo, 0, ci, fx) && loc_split(Y[q], geo, 1, cj, fy)) {
+            gather16<double>(uv, geo.nx, ci, cj, fx, fy, su, sv);
         } else {
             atomicAdd(oob, 1ull);
             atomicOr(status, ST_OUT_OF_DOMAIN);
         }
         uq[q] = su;
         vq[q] = sv;
+    }
+}
+
+// FP32: a warp takes 32 points.  Cells and weights are formed by a thread a
+// point and left in shared memory; then eight lanes a point, four points at a
+// time, gather one half row of the stencil each.  The pass is bound by the L1
+// lookups of its scattered loads, one a distinct line and instruction: a
+// thread a point makes 16 a point, half rows 8 (200,003 points on 768 x 512:
+// 12.8 -> XY8 us).
+constexpr int XY_THREADS = 128;
+struct XyPoint {
+    float wx[4], wy[4];
+    int at;                    // first node of the stencil; -1: off the grid
+    float u, v;
+    int pad;
+};
+__global__ void __launch_bounds__(XY_THREADS) k_interp_xy_f32(const float2* __restrict__ uv, const double* __restrict__ X,
+                                                              const double* __restrict__ Y, int64_t nq, Geo geo,
+                                                              float* __restrict__ uq, float* __restrict__ vq,
+                                                              int* __restrict__ status, unsigned long long* __restrict__ oob) {
+    __shared__ __align__(16) XyPoint pts[XY_THREADS];
+    const int lane = threadIdx.x & 31, col = lane & 3, pair = (lane >> 2) & 1;
+    XyPoint* mine = pts + (threadIdx.x & ~31);
+    pdl_wait();
+    for (int64_t q0 = ((int64_t)blockIdx.x * XY_THREADS + threadIdx.x) - lane; q0 < nq; q0 += (int64_t)gridDim.x * XY_THREADS) {
+        const int64_t q = q0 + lane;
+        {
+            XyPoint p;
+            int ci = 0, cj = 0;
+            float fx = 0.f, fy = 0.f;
+            const bool ok = q < nq && split(X[q], geo.x0, geo.dx, geo.inv_dx, geo.cx, geo.nx, geo.xlim, ci, fx) &&
+                            split(Y[q], geo.y0, geo.dx, geo.inv_dx, geo.cy, geo.ny, geo.ylim, cj, fy);
+            if (q < nq && !ok) {
+                atomicAdd(oob, 1ull);
+                atomicOr(status, ST_OUT_OF_DOMAIN);
+            }
+            m4p_weights(ok ? fx : 0.f, p.wx);
+            m4p_weights(ok ? fy : 0.f, p.wy);
+            p.at = ok ? (cj - 1) * geo.nx + ci - 1 : -1;
+            p.u = p.v = 0.f;
+            mine[lane] = p;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const XyPoint& p = mine[4 * i + (lane >> 3)];
+            const int at = p.at;
+            float2 a = make_float2(0.f, 0.f), b = a;
+            if (at >= 0) {
+                const float2* r = uv + at + 2 * pair * geo.nx + col;
+                a = __ldg(r);
+                b = __ldg(r + geo.nx);
+            }
+            const float2 w = *reinterpret_cast<const float2*>(p.wy + 2 * pair);
+            const float wx = p.wx[col];
+            float su = wx * (w.x * a.x + w.y * b.x), sv = wx * (w.x * a.y + w.y * b.y);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                su += __shfl_xor_sync(0xffffffffu, su, o);
+                sv += __shfl_xor_sync(0xffffffffu, sv, o);
+            }
+            if ((lane & 7) == 0) {
+                mine[4 * i + (lane >> 3)].u = su;
+                mine[4 * i + (lane >> 3)].v = sv;
+            }
+        }
+        __syncwarp();
+        if (q < nq) {
+            uq[q] = mine[lane].u;
+            vq[q] = mine[lane].v;
+        }
+        __syncwarp();
     }
 }
 
