@@ -144,10 +144,9 @@ struct TuneBuffers {
     }
 };
 
+// a velocity evaluation by the route that nv vortices take
 pf_status velocity_once(pf_plan p, const TuneBuffers& tb, int64_t nv) {
-    PF_TRY(vortex_regularize(p, tb.X, tb.Y, tb.G, nv, p->w));
-    PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, 1.0, 0.0));
-    return vortex_interpolate_located(p, p->uv, nv, tb.u, tb.v);
+    return pf_vic_velocity(p, tb.X, tb.Y, tb.G, nv, 1.0, 0.0, tb.u, tb.v);
 }
 
 // median time (microseconds) of `reps` evaluations in configuration c

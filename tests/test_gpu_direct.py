@@ -55,3 +55,13 @@ def test_direct_equals_binned(prec, nx, ny, n, tile, clustered):
     for a, b in ((u, ru[:n]), (v, rv[:n])):
         assert float((a - b).double().norm()) <= tol * float(b.double().norm())
         assert torch.equal(a == 0, b == 0)                     # those off the grid
+
+
+@pytest.mark.parametrize("prec", [pf.PF_FP64, pf.PF_MIXED])
+def test_tuning_a_small_set_after_a_large_one(prec):
+    """The tuner times the route that the set takes: nothing of the larger set's bins is read."""
+    plan = pf.Plan(100, 90, 0.01, 0.0, 0.0, prec)
+    pf.pf_regularize(plan, *[torch.from_numpy(a).cuda() for a in _set(20000, 100, 90, 0.01, 3, False)])
+    _oob(plan)
+    pf.pf_autotune(plan, 300, reps=1)
+    assert pf.pf_sync(plan) == 0
