@@ -77,6 +77,17 @@ inline int bin_blocks(int64_t nv, int min_span = BIN_MIN_SPAN) {
     return nv > 0 ? (int)((nv + bin_span(nv, min_span) - 1) / bin_span(nv, min_span)) : 0;
 }
 
+// Partition of the one-pass binning (transfer.cuh), for sets of the mixed path
+// up to RUN_VORTICES: the blocks' span, 0 for sets that it does not take.
+constexpr int RUN_THREADS = 512;
+constexpr int RUN_MAX = 32;                    // blocks
+constexpr int64_t RUN_VORTICES = 65536;
+inline int run_span(int64_t nv, int min_span, int prec) {
+    if (prec == PF_FP64 || nv <= 0 || nv > RUN_VORTICES) return 0;
+    const int s = (int)((nv + RUN_MAX - 1) / RUN_MAX);
+    return s < min_span ? min_span : s;
+}
+
 // Read-only tables of one grid shape, shared by a plan and its clones.
 struct PlanTables {
     int refs = 1;
@@ -129,6 +140,7 @@ struct pf_plan_s {
     int tile_threads = 256;
     int fft_impl = 0;
     int bin_tile = BIN_TILE;           // tile edge of the last binning (its records serve E_v)
+    int bin_runs = 0, bin_span = 0;    // its blocks and their span if it was the one-pass binning; else none
     // binning
     int ntx = 0, nty = 0, ntiles = 0;  // tiles at BIN_TILE
     int tile_slots = 0;                // entries of tile_count and tile_start (tiles at the smallest offered edge)

@@ -2,7 +2,9 @@
 //   R_v (Eq. vortexregularization): w_ij = dx^-2 sum_q Gamma_q d((x_i-X_q)/dx) d((y_j-Y_q)/dx)
 //   E_v = R_v^T:                    u_q  = sum_ij d d u_ij
 //
-// Regularization is a binned scatter in four kernels:
+// Small sets take one launch each way (k_deposit_direct, k_interp_direct),
+// middling ones of the mixed path two for R_v (k_bin_runs, k_deposit).  Else
+// regularization is a binned scatter in four kernels:
 //   locate   FP64 position -> integer cell + fraction (one pass, FP64 used only
 //            for g = (X - x0)/dx), compact per-vortex record, per-block tile
 //            histogram in shared memory, written out as one row per block;
@@ -82,11 +84,39 @@ BinWork plan_binwork(pf_plan p) {
     return b;
 }
 
+RunBins run_bins(pf_plan p, const Geo& geo) {
+    return RunBins{(const unsigned*)p->bin_off, p->gmax + 1, p->bin_runs, 4 * p->bin_span, geo.ntiles};
+}
+
+// R_v by the one-pass binning: two launches.  (Its table fits the histograms'
+// room: no more blocks.)
+template <int TILE>
+pf_status regularize_runs(pf_plan p, const Geo& geo, const BinWork& bw, const double* X, const double* Y, const double* G,
+                          int64_t nv, float* w, const int64_t* dn) {
+    const int span = p->bin_span;
+    const size_t sm = (size_t)span * sizeof(Pos<float>) + (size_t)geo.ntiles * sizeof(unsigned);
+    PF_CUDA(p, set_smem(k_bin_runs<TILE>, sm));
+    PF_KERNEL(p, "bin_runs", PF_CUDA(p, pf_launch(k_bin_runs<TILE>, p->bin_runs, RUN_THREADS, sm, p->stream, X, Y, G, nv,
+                                                  span, dn, geo, (Rec<float>*)bw.recs, (unsigned*)bw.bin_off, bw.gmax + 1,
+                                                  bw.status, bw.oob, (float*)bw.zu, (float*)bw.zv)));
+    PF_KERNEL(p, "regularize", PF_CUDA(p, pf_launch(k_deposit<float, TILE, RunBins>, geo.ntiles, p->tile_threads, 0,
+                                                    p->stream, (const Rec<float>*)bw.recs, run_bins(p, geo), geo, w,
+                                                    bw.status)));
+    return PF_OK;
+}
+
 template <typename T>
 pf_status regularize_configured(pf_plan p, const BinWork& bw, const double* X, const double* Y, const double* G,
                                 int64_t nv, T* w, const int64_t* dn) {
     const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0, p->tile);
     p->bin_tile = p->tile;
+    p->bin_span = run_span(nv, p->min_span, p->prec);
+    p->bin_runs = p->bin_span ? ceil_div(nv, p->bin_span) : 0;
+    if constexpr (sizeof(T) == 4) {
+        if (p->bin_runs)
+            return p->tile == BIN_TILE_SMALL ? regularize_runs<BIN_TILE_SMALL>(p, geo, bw, X, Y, G, nv, w, dn)
+                                             : regularize_runs<BIN_TILE>(p, geo, bw, X, Y, G, nv, w, dn);
+    }
     if (p->tile == BIN_TILE_SMALL)
         return regularize_launch<T, BIN_TILE_SMALL>(p, geo, bw, X, Y, G, nv, w, p->stream, p->min_span,
                                                     p->tile_threads, dn);
@@ -120,23 +150,27 @@ pf_status interpolate_direct_t(pf_plan p, const void* uv, const double* X, const
     return PF_OK;
 }
 
+template <int TILE, typename BINS>
+pf_status interpolate_tiles_f32(pf_plan p, const Geo& geo, const BINS& bins, const void* uv, int64_t nq, void* uq, void* vq) {
+    // 256 threads whatever the plan's tile_threads: four records a thread
+    // make the sort's chunks 1024 records (128-thread blocks with eight a
+    // thread fit six blocks an SM, a second wave at 1024 tiles: 28.7 us
+    // against 24.5 us at 1024^2 / 1e6)
+    PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles_f32<TILE, 4, BINS>, geo.ntiles, 256,
+                                                     (size_t)(4 * 256 + 32) * sizeof(Rec<float>), p->stream,
+                                                     (const Rec<float>*)p->recs, bins, (const float2*)uv, geo,
+                                                     (float*)uq, (float*)vq, nq, p->d_status)));
+    return PF_OK;
+}
+
 template <int TILE>
 pf_status interpolate_tiles(pf_plan p, const Geo& geo, const void* uv, int64_t nq, void* uq, void* vq) {
-    if (p->prec == PF_FP64)
-        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles_f64<TILE>, geo.ntiles, p->tile_threads, 0,
-                                                         p->stream, (const Rec<double>*)p->recs, p->tile_start,
-                                                         p->tile_count, (const double2*)uv, geo, (double*)uq,
-                                                         (double*)vq, p->rec_cap, nq, p->d_status)));
-    else
-        // 256 threads whatever the plan's tile_threads: four records a thread
-        // make the sort's chunks 1024 records (128-thread blocks with eight a
-        // thread fit six blocks an SM, a second wave at 1024 tiles: 28.7 us
-        // against 24.5 us at 1024^2 / 1e6)
-        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles_f32<TILE, 4>, geo.ntiles, 256,
-                                                         (size_t)(4 * 256 + 32) * sizeof(Rec<float>), p->stream,
-                                                         (const Rec<float>*)p->recs, p->tile_start, p->tile_count,
-                                                         (const float2*)uv, geo, (float*)uq, (float*)vq, p->rec_cap,
-                                                         nq, p->d_status)));
+    if (p->bin_runs) return interpolate_tiles_f32<TILE>(p, geo, run_bins(p, geo), uv, nq, uq, vq);
+    const FlatBins bins{p->tile_start, p->tile_count, p->gmax, p->rec_cap};
+    if (p->prec != PF_FP64) return interpolate_tiles_f32<TILE>(p, geo, bins, uv, nq, uq, vq);
+    PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_tiles_f64<TILE>, geo.ntiles, p->tile_threads, 0,
+                                                     p->stream, (const Rec<double>*)p->recs, bins, (const double2*)uv,
+                                                     geo, (double*)uq, (double*)vq, nq, p->d_status)));
     return PF_OK;
 }
 

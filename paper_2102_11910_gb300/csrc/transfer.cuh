@@ -527,6 +527,119 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : 4) k_scatter(const Pos<T>
     }
 }
 
+// One-pass binning of the mixed path's middling sets: at most RUN_MAX blocks, each
+// of which locates its span of vortices (their cells stay in shared memory),
+// counts and scans its own tiles, and writes its records in tile order into its
+// own stretch of the record array, four slots a vortex.  table[b][t] holds the
+// run of tile t in block b: first slot | records << 16.  The deposit and E_v
+// blocks find a tile's records by a search over the runs (RunRecs).  The three
+// passes of larger sets take as many launches of 3 to 6 us whatever the count
+// (a velocity of 5,000 vortices on 1024^2 65.2 -> 58.0 us, of 20,011 on 700 x 333
+// 46.7 -> 39.5, of 65,000 on 300 x 200 46.8 -> 43.6; of 131,000, whose 32 blocks
+// bind, 57.0 -> 55.9).  More and so shorter runs lose: with 304 blocks, each
+// record's run found by a scan, 1e6 vortices on 1024^2 took 109 us against 103.
+template <int TILE>
+__global__ void __launch_bounds__(RUN_THREADS) k_bin_runs(const double* __restrict__ X, const double* __restrict__ Y,
+                                                             const double* __restrict__ G, int64_t nv, int span,
+                                                             const int64_t* __restrict__ dn, Geo geo,
+                                                             Rec<float>* __restrict__ recs, unsigned* __restrict__ table,
+                                                             double* __restrict__ gmax_blk, int* __restrict__ status,
+                                                             unsigned long long* __restrict__ oob, float* __restrict__ zu,
+                                                             float* __restrict__ zv) {
+    extern __shared__ __align__(16) unsigned char run_dyn[];
+    __shared__ float wmax[RUN_THREADS / 32];
+    __shared__ int wsum[RUN_THREADS / 32];
+    Pos<float>* cells = reinterpret_cast<Pos<float>*>(run_dyn);
+    unsigned* cnt = reinterpret_cast<unsigned*>(cells + span);
+    for (int i = threadIdx.x; i < geo.ntiles; i += RUN_THREADS) cnt[i] = 0u;
+    pdl_wait();
+    if (dn) nv = *dn < nv ? *dn : nv;
+    const int64_t lo = (int64_t)blockIdx.x * span;
+    const int n = (int)(lo >= nv ? 0 : (nv - lo < span ? nv - lo : span));
+    __syncthreads();
+    float gm = 0.f;
+    int bad = 0;
+    for (int base = 0; base < n; base += RUN_THREADS * BIN_UNROLL) {
+        double xs[BIN_UNROLL], ys[BIN_UNROLL], gs[BIN_UNROLL];
+#pragma unroll
+        for (int k = 0; k < BIN_UNROLL; ++k) {   // clamped: a thread past the end reloads the last vortex
+            int i = base + k * RUN_THREADS + threadIdx.x;
+            i = i < n ? i : n - 1;
+            xs[k] = X[lo + i];
+            ys[k] = Y[lo + i];
+            gs[k] = G[lo + i];
+        }
+#pragma unroll
+        for (int k = 0; k < BIN_UNROLL; ++k) {
+            const int i = base + k * RUN_THREADS + threadIdx.x;
+            if (i >= n) break;
+            int ci = 0, cj = 0;
+            unsigned fx = 0, fy = 0;
+            Pos<float> p;
+            if (!loc_split(xs[k], geo, 0, ci, fx) || !loc_split(ys[k], geo, 1, cj, fy)) {
+                ++bad;
+                make_pos(p, 0xFFFF, 0xFFFF, 0u, 0u, 0.0);   // marker: no record
+                cells[i] = p;
+                if (zu) {
+                    zu[lo + i] = 0.f;
+                    zv[lo + i] = 0.f;
+                }
+                continue;
+            }
+            make_pos(p, ci, cj, fx, fy, gs[k]);
+            cells[i] = p;                            // read back by this thread
+            gm = abs_max(gm, p.g);
+            const int tx0 = (ci - 1) / TILE, tx1 = (ci + 2) / TILE;
+            const int ty0 = (cj - 1) / TILE, ty1 = (cj + 2) / TILE;
+            for (int ty = ty0; ty <= ty1; ++ty)
+                for (int tx = tx0; tx <= tx1; ++tx) atomicAdd(&cnt[ty * geo.ntx + tx], 1u);
+        }
+    }
+    if (bad) {
+        atomicAdd(oob, (unsigned long long)bad);
+        atomicOr(status, ST_OUT_OF_DOMAIN);
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    if (lane == 0) wmax[wid] = gm;
+    __syncthreads();
+    // exclusive scan of the counts: a thread owns `per` tiles
+    const int per = (geo.ntiles + RUN_THREADS - 1) / RUN_THREADS, t0 = threadIdx.x * per;
+    const int t1 = t0 + per < geo.ntiles ? t0 + per : geo.ntiles;
+    int sum = 0;
+    for (int i = t0; i < t1; ++i) sum += (int)cnt[i];
+    const int incl = warp_incl_scan(sum, lane);
+    if (lane == 31) wsum[wid] = incl;
+    if (threadIdx.x == 0) {
+        float m = 0.f;
+        for (int i = 0; i < RUN_THREADS / 32; ++i) m = fmax(m, wmax[i]);
+        gmax_blk[blockIdx.x] = (double)m;
+    }
+    __syncthreads();
+    unsigned run = (unsigned)(incl - sum);
+    for (int w = 0; w < wid; ++w) run += (unsigned)wsum[w];
+    unsigned* row = table + (size_t)blockIdx.x * geo.ntiles;
+    for (int i = t0; i < t1; ++i) {
+        const unsigned c = cnt[i];
+        row[i] = run | (c << 16);
+        cnt[i] = run;
+        run += c;
+    }
+    __syncthreads();
+    Rec<float>* out = recs + 4 * lo;
+    for (int i = threadIdx.x; i < n; i += RUN_THREADS) {
+        const Pos<float> p = cells[i];
+        const int ci = pos_ci(p), cj = pos_cj(p);
+        if (ci == 0xFFFF) continue;
+        const int tx0 = (ci - 1) / TILE, tx1 = (ci + 2) / TILE;
+        const int ty0 = (cj - 1) / TILE, ty1 = (cj + 2) / TILE;
+        for (int ty = ty0; ty <= ty1; ++ty)
+            for (int tx = tx0; tx <= tx1; ++tx)
+                out[atomicAdd(&cnt[ty * geo.ntx + tx], 1u)] = make_rec(p, ci - tx * TILE, cj - ty * TILE, (int)(lo + i));
+    }
+}
+
 // fixed-point scale 2^sh as a floating-point number, sh in [-60, 100]
 template <typename T> __device__ __forceinline__ T pow2(int sh);
 template <> __device__ __forceinline__ float pow2<float>(int sh) { return __int_as_float((sh + 127) << 23); }
@@ -620,27 +733,105 @@ __device__ __forceinline__ void deposit_one(const Rec<T>& rc, T scale, unsigned 
     }
 }
 
-// U records per thread at a time, the next U loaded while these are used (a
-// thread past the end reloads the last record, which it then skips)
+// The records of one tile: load() gives a thread U of them, blockDim apart (a
+// thread past the end reloads the last record, which it then skips).  FlatRecs:
+// a stretch of one array.
 constexpr int REC_U = 4;
-template <typename T, int U>
-__device__ __forceinline__ void load_recs(const Rec<T>* __restrict__ recs, int r0, int cnt, Rec<T> (&rc)[U]) {
+template <typename T> struct FlatRecs {
+    const Rec<T>* recs;
+    int cnt;
+    template <int U> __device__ __forceinline__ void load(int r0, Rec<T> (&rc)[U]) const {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int r = r0 + u * (int)blockDim.x + (int)threadIdx.x;
-        rc[u] = recs[r < cnt ? r : cnt - 1];
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * (int)blockDim.x + (int)threadIdx.x;
+            rc[u] = recs[r < cnt ? r : cnt - 1];
+        }
     }
+};
+// The runs that k_bin_runs left for the tile: five halvings find a record's.
+struct RunRecs {
+    const Rec<float>* recs;
+    const int2* runs;        // [RUN_MAX] records of the runs before; slot of the run's first record less that
+    int cnt;
+    template <int U> __device__ __forceinline__ void load(int r0, Rec<float> (&rc)[U]) const {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = min(r0 + u * (int)blockDim.x + (int)threadIdx.x, cnt - 1);
+            int b = 0;                                   // the last run that begins at r or before
+#pragma unroll
+            for (int step = RUN_MAX / 2; step > 0; step >>= 1)
+                if (runs[b + step].x <= r) b += step;
+            rc[u] = recs[r + runs[b].y];
+        }
+    }
+};
+
+// Where a tile's records are: as k_scatter left them, or in runs
+struct FlatBins {
+    const int* tile_start;
+    const unsigned* tile_count;
+    const double* gmax;            // largest |Gamma|
+    int64_t rec_cap;
+};
+struct RunBins {
+    const unsigned* table;
+    const double* gmax;            // that of each block
+    int nb, region, ntiles;        // blocks, record slots of each
+};
+
+// The records of tile t and, with GMAX, the largest |Gamma|
+template <bool GMAX, typename T>
+__device__ __forceinline__ FlatRecs<T> open_tile(const FlatBins& bins, const Rec<T>* recs, int t, int* status,
+                                                 double& gmax) {
+    int start = bins.tile_start[t], cnt = (int)bins.tile_count[t];
+    if (cnt != 0 && (start < 0 || cnt < 0 || (int64_t)start + cnt > bins.rec_cap)) {     // block-uniform
+        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
+        cnt = 0;
+    }
+    if (cnt == 0) start = 0;
+    if (GMAX) gmax = *bins.gmax;
+    return FlatRecs<T>{recs + start, cnt};
+}
+template <bool GMAX>
+__device__ __forceinline__ RunRecs open_tile(const RunBins& bins, const Rec<float>* recs, int t, int* status,
+                                             double& gmax) {
+    static_assert(RUN_MAX == 32, "a run a lane");
+    __shared__ int2 runs[RUN_MAX];
+    __shared__ int total;
+    __shared__ float top;
+    if (threadIdx.x < 32) {
+        const int b = threadIdx.x;
+        const unsigned e = b < bins.nb ? bins.table[(size_t)b * bins.ntiles + t] : 0u;
+        float gm = GMAX && b < bins.nb ? (float)bins.gmax[b] : 0.f;        // exact: a float
+        const int slot = (int)(e & 0xFFFFu);
+        int c = (int)(e >> 16);
+        if (slot + c > bins.region) {                                    // not as the binning writes it
+            atomicOr(status, ST_INTERNAL);
+            c = 0;
+        }
+        const int incl = warp_incl_scan(c, b);
+        runs[b] = make_int2(incl - c, b * bins.region + slot - (incl - c));
+        if (b == 31) total = incl;
+        if (GMAX) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+            if (b == 0) top = gm;
+        }
+    }
+    __syncthreads();
+    if (GMAX) gmax = (double)top;
+    return RunRecs{recs, runs, total};
 }
 
-// every record of the tile, given to `one`; rc holds this thread's first REC_U (load_recs at 0)
-template <typename T, typename F>
-__device__ __forceinline__ void deposit_records(const Rec<T>* __restrict__ recs, int cnt, Rec<T> (&rc)[REC_U], F one) {
-    const int stride = REC_U * (int)blockDim.x;
+// every record of the tile, given to `one`; rc holds this thread's first REC_U (src.load at 0)
+template <typename T, typename SRC, typename F>
+__device__ __forceinline__ void deposit_records(const SRC& src, Rec<T> (&rc)[REC_U], F one) {
+    const int stride = REC_U * (int)blockDim.x, cnt = src.cnt;
     for (int r0 = 0; r0 < cnt; r0 += stride) {
         Rec<T> cur[REC_U];
 #pragma unroll
         for (int u = 0; u < REC_U; ++u) cur[u] = rc[u];
-        if (r0 + stride < cnt) load_recs(recs, r0 + stride, cnt, rc);
+        if (r0 + stride < cnt) src.load(r0 + stride, rc);
 #pragma unroll
         for (int u = 0; u < REC_U; ++u)
             if (r0 + u * (int)blockDim.x + (int)threadIdx.x < cnt) one(cur[u]);
@@ -661,11 +852,11 @@ constexpr int DEP_MAX_THREADS = 256;
 constexpr int DEP_SORT_MIN = 256;     // fewer records: too few adds for the sort's three barriers to pay
 constexpr int DEP_SORT_SLOTS = REC_U * DEP_MAX_THREADS + 32;
 
-template <int ACC_W, typename T>
-__device__ __forceinline__ void deposit_records_banked(const Rec<T>* __restrict__ recs, int cnt, T scale,
+template <int ACC_W, typename T, typename SRC>
+__device__ __forceinline__ void deposit_records_banked(const SRC& src, T scale,
                                                        unsigned long long* acc, Rec<T> (&rc)[REC_U],
                                                        Rec<T>* srt, int* bcnt, int* bstart) {
-    const int stride = REC_U * (int)blockDim.x;
+    const int stride = REC_U * (int)blockDim.x, cnt = src.cnt;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
     for (int r0 = 0; r0 < cnt; r0 += stride) {
         const int n = cnt - r0 < stride ? cnt - r0 : stride;
@@ -692,7 +883,7 @@ __device__ __forceinline__ void deposit_records_banked(const Rec<T>* __restrict_
                 srt[(idx % R) * 32 + idx / R] = rc[u];
             }
         }
-        if (r0 + stride < cnt) load_recs(recs, r0 + stride, cnt, rc);   // the next chunk in flight
+        if (r0 + stride < cnt) src.load(r0 + stride, rc);   // the next chunk in flight
         __syncthreads();
         for (int i = wid; i < R; i += nw)
             if (lane * R + i < n) deposit_one<DEP_SPLIT32, ACC_W, T>(srt[i * 32 + lane], scale, acc);
@@ -714,12 +905,13 @@ __device__ __forceinline__ void deposit_clear(DepositSmem<T, TILE, SORT>& sm) {
     if (threadIdx.x < 32) sm.bcnt[threadIdx.x] = 0;
 }
 
-// w of tile (tx, ty) from its cnt records (global or shared memory); rc holds
+// w of tile (tx, ty) from its records (global or shared memory); rc holds
 // this thread's first ones, sm is cleared (the barrier is in here)
-template <typename T, int TILE, bool SORT>
-__device__ __forceinline__ void deposit_tile(const Rec<T>* recs, int cnt, double gmax, const Geo& geo, int tx, int ty,
+template <typename T, int TILE, bool SORT, typename SRC>
+__device__ __forceinline__ void deposit_tile(const SRC& src, double gmax, const Geo& geo, int tx, int ty,
                                              T* __restrict__ w, DepositSmem<T, TILE, SORT>& sm, Rec<T> (&rc)[REC_U]) {
     constexpr int ACC_W = AccW<TILE>::value;
+    const int cnt = src.cnt;
     unsigned long long* acc = sm.acc;
     int* bstart = sm.bstart;
     if constexpr (sizeof(T) == 8) {
@@ -731,7 +923,7 @@ __device__ __forceinline__ void deposit_tile(const Rec<T>* recs, int cnt, double
         unsigned* acc_hi = acc_lo + ACC_W * ACC_W;
         if (threadIdx.x == 0) bstart[0] = 0;                      // set by a record that is not finite
         __syncthreads();
-        deposit_records<T>(recs, cnt, rc,
+        deposit_records<T>(src, rc,
                            [&](const Rec<T>& r) { deposit_one_fx<ACC_W>(r, gexp, drop, acc_lo, acc_hi, &bstart[0]); });
         __syncthreads();
         for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
@@ -750,12 +942,12 @@ __device__ __forceinline__ void deposit_tile(const Rec<T>* recs, int cnt, double
         const T scale = pow2<T>(sh);
         __syncthreads();
         if (SORT && split32 && cnt >= DEP_SORT_MIN)             // block-uniform
-            deposit_records_banked<ACC_W>(recs, cnt, scale, acc, rc, sm.srt, sm.bcnt, bstart);
+            deposit_records_banked<ACC_W, T>(src, scale, acc, rc, sm.srt, sm.bcnt, bstart);
         else if (split32)
-            deposit_records<T>(recs, cnt, rc,
+            deposit_records<T>(src, rc,
                                [&](const Rec<T>& r) { deposit_one<DEP_SPLIT32, ACC_W, T>(r, scale, acc); });
         else
-            deposit_records<T>(recs, cnt, rc,
+            deposit_records<T>(src, rc,
                                [&](const Rec<T>& r) { deposit_one<DEP_F32_64, ACC_W, T>(r, scale, acc); });
         __syncthreads();
         const int* acc_hi = reinterpret_cast<const int*>(acc);
@@ -775,23 +967,18 @@ __device__ __forceinline__ void deposit_tile(const Rec<T>* recs, int cnt, double
     }
 }
 
-template <typename T, int TILE>
-__global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs, const int* __restrict__ tile_start,
-                                                 const unsigned* __restrict__ tile_count,
-                                                 const double* __restrict__ gmax_all, Geo geo, T* __restrict__ w,
-                                                 int64_t rec_cap, int* __restrict__ status) {
+template <typename T, int TILE, typename BINS>
+__global__ void __launch_bounds__(256) k_deposit(const Rec<T>* __restrict__ recs, BINS bins, Geo geo, T* __restrict__ w,
+                                                 int* __restrict__ status) {
     __shared__ DepositSmem<T, TILE, true> sm;
     const int t = blockIdx.x;
     deposit_clear(sm);
     pdl_wait();
-    int start = tile_start[t], cnt = (int)tile_count[t];
-    if (start < 0 || cnt < 0 || (int64_t)start + cnt > rec_cap) {     // block-uniform
-        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
-        start = cnt = 0;
-    }
+    double gmax;
+    const auto src = open_tile<true>(bins, recs, t, status, gmax);
     Rec<T> rc[REC_U];
-    if (cnt > 0) load_recs(recs + start, 0, cnt, rc);               // in flight across the barrier
-    deposit_tile(recs + start, cnt, *gmax_all, geo, t % geo.ntx, t / geo.ntx, w, sm, rc);
+    if (src.cnt > 0) src.load(0, rc);                               // in flight across the barrier
+    deposit_tile(src, gmax, geo, t % geo.ntx, t / geo.ntx, w, sm, rc);
 }
 
 // A bound sheet added to w with the deposit: the grid nodes of its 16 ns
@@ -875,8 +1062,9 @@ __global__ void __launch_bounds__(256) k_deposit_direct(const double* __restrict
     for (int i = 0; i < 8; ++i) gm = fmax(gm, wmax[i]);
     const int cnt = n;
     Rec<T> rc[REC_U];
-    if (cnt > 0) load_recs(list, 0, cnt, rc);
-    deposit_tile(list, cnt, (double)gm, geo, tx, ty, w, sm, rc);
+    const FlatRecs<T> src{list, cnt};
+    if (cnt > 0) src.load(0, rc);
+    deposit_tile(src, (double)gm, geo, tx, ty, w, sm, rc);
     if (sheet.n == 0) return;
     __syncthreads();                                  // the tile's w is written
     for (int i = threadIdx.x; i < sheet.n; i += 256) {
@@ -925,25 +1113,20 @@ __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int c
 // a record are integer multiply-adds (1e6 vortices on 1024^2: 227 -> 67 us); a
 // patch with an infinity or a NaN keeps its doubles and the FP64 sums.
 template <int TILE>
-__global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __restrict__ recs,
-                                                          const int* __restrict__ tile_start,
-                                                          const unsigned* __restrict__ tile_count,
+__global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __restrict__ recs, FlatBins bins,
                                                           const double2* __restrict__ uv, Geo geo,
-                                                          double* __restrict__ uq, double* __restrict__ vq,
-                                                          int64_t rec_cap, int64_t nq, int* __restrict__ status) {
+                                                          double* __restrict__ uq, double* __restrict__ vq, int64_t nq,
+                                                          int* __restrict__ status) {
     constexpr int PATCH = TILE + 3;
     __shared__ int4 patch[PATCH * PATCH];
     __shared__ int top;
     const int t = blockIdx.x;
     if (threadIdx.x == 0) top = 1;
     pdl_wait();
-    const int cnt = (int)tile_count[t];
-    if (cnt == 0) return;
-    const int start = tile_start[t];
-    if (start < 0 || cnt < 0 || (int64_t)start + cnt > rec_cap) {     // block-uniform
-        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
-        return;
-    }
+    double unused;
+    const auto src = open_tile<false>(bins, recs, t, status, unused);
+    const int cnt = src.cnt;
+    if (cnt == 0) return;                             // block-uniform
     const int tx = t % geo.ntx, ty = t / geo.ntx;
     const int gi0 = tx * TILE - 1, gj0 = ty * TILE - 1;
     double2* patchd = reinterpret_cast<double2*>(patch);
@@ -973,12 +1156,9 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
     for (int r0 = 0; r0 < cnt; r0 += U * blockDim.x) {
         Rec<double> rc[U];
         bool ok[U];
+        src.load(r0, rc);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {           // loads first (clamped index)
-            const int r = r0 + u * blockDim.x + threadIdx.x;
-            ok[u] = r < cnt;
-            rc[u] = recs[start + (ok[u] ? r : cnt - 1)];
-        }
+        for (int u = 0; u < U; ++u) ok[u] = r0 + u * (int)blockDim.x + (int)threadIdx.x < cnt;
 #pragma unroll 1
         for (int u = 0; u < U; ++u) {
             const Rec<double> c = u == 0 ? rc[0] : rc[1];
@@ -1044,14 +1224,13 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
 // warp, whose 16-byte loads are served together, read eight different bank
 // groups; non-home records (a vortex's other tiles) drop out in the same pass.
 // U records a thread a chunk.  Dynamic shared memory: (U x blockDim + 32)
-// records.
-template <int TILE, int U>
-__global__ void __launch_bounds__(256) k_interp_tiles_f32(const Rec<float>* __restrict__ recs,
-                                                          const int* __restrict__ tile_start,
-                                                          const unsigned* __restrict__ tile_count,
+// records.  Five blocks an SM (48 registers): with 64 registers, so four, 1e6
+// vortices on 1024^2 took 22.4 us instead of 20.5.
+template <int TILE, int U, typename BINS>
+__global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* __restrict__ recs, BINS bins,
                                                           const float2* __restrict__ uv, Geo geo,
-                                                          float* __restrict__ uq, float* __restrict__ vq,
-                                                          int64_t rec_cap, int64_t nq, int* __restrict__ status) {
+                                                          float* __restrict__ uq, float* __restrict__ vq, int64_t nq,
+                                                          int* __restrict__ status) {
     constexpr int PATCH = TILE + 3, PAIRS = (PATCH + 1) / 2;   // 18 pairs per patch row at TILE 32
     __shared__ float4 pe[PATCH * PAIRS];
     __shared__ float4 po[PATCH * PAIRS];
@@ -1060,15 +1239,12 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f32(const Rec<float>* __re
     Rec<float>* srt = reinterpret_cast<Rec<float>*>(interp_dyn);
     const int t = blockIdx.x;
     pdl_wait();
-    const int cnt = (int)tile_count[t];
-    if (cnt == 0) return;
-    const int start = tile_start[t];
-    if (start < 0 || cnt < 0 || (int64_t)start + cnt > rec_cap) {     // block-uniform
-        if (threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
-        return;
-    }
+    double unused;
+    const auto src = open_tile<false>(bins, recs, t, status, unused);
+    const int cnt = src.cnt;
+    if (cnt == 0) return;                         // block-uniform
     Rec<float> rc[U];
-    load_recs(recs + start, 0, cnt, rc);          // in flight while the patch is staged
+    src.load(0, rc);                              // in flight while the patch is staged
     if (threadIdx.x < 32) bcnt[threadIdx.x] = 0;
     const int tx = t % geo.ntx, ty = t / geo.ntx;
     const int gi0 = tx * TILE - 1, gj0 = ty * TILE - 1;
@@ -1119,7 +1295,7 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f32(const Rec<float>* __re
                 srt[(idx % R) * 32 + idx / R] = rc[u];
             }
         }
-        if (r0 + stride < cnt) load_recs(recs + start, r0 + stride, cnt, rc);   // the next chunk in flight
+        if (r0 + stride < cnt) src.load(r0 + stride, rc);   // the next chunk in flight
         __syncthreads();
         for (int i = wid; i < R; i += nw) {
             if (lane * R + i >= nh) continue;
@@ -1375,8 +1551,8 @@ template <typename T, int TILE = BIN_TILE>
 pf_status deposit_launch(pf_plan p, const Geo& geo, const Rec<T>* recs, const int* tile_start,
                          const unsigned* tile_count, const double* gmax, int64_t rec_cap, int* status, T* w,
                          cudaStream_t s, int threads = 256) {
-    PF_KERNEL(p, "regularize", PF_CUDA(p, pf_launch(k_deposit<T, TILE>, geo.ntiles, threads, 0, s, recs, tile_start, tile_count,
-                                                    gmax, geo, w, rec_cap, status)));
+    PF_KERNEL(p, "regularize", PF_CUDA(p, pf_launch(k_deposit<T, TILE, FlatBins>, geo.ntiles, threads, 0, s, recs,
+                                                    FlatBins{tile_start, tile_count, gmax, rec_cap}, geo, w, status)));
     return PF_OK;
 }
 
