@@ -33,7 +33,7 @@ void free_plan(pf_plan p) {
     }
     if (p->shared && --p->shared->refs == 0) {
         void* tables[] = {p->G, p->H64, p->H32, p->Hu64, p->Hv64, p->Hu32, p->Hv32, p->twP64, p->twQ64, p->twP32,
-                          p->twQ32, p->tw256_64, p->tw256_32, p->twP_fx};
+                          p->twQ32, p->twP32_r, p->twP_fx};
         for (void* q : tables)
             if (q) cudaFree(q);
         delete p->shared;
@@ -54,6 +54,17 @@ void twiddles(std::vector<C>& v, int N) {
         v[m].x = (decltype(v[m].x))c;
         v[m].y = (decltype(v[m].y))s;
     }
+}
+
+// the register passes' table of length N (fft_reg.cuh), appended to v
+void pass_twiddles(std::vector<float2>& v, int N) {
+    std::vector<float2> t256, tN;
+    twiddles(t256, 256);
+    twiddles(tN, N);
+    for (int r = 1; r < 16; ++r)
+        for (int k = 0; k < 16; ++k) v.push_back(t256[r * k]);
+    for (int r = 1; r < N / 256; ++r)
+        for (int j = 0; j < 256; ++j) v.push_back(tN[r * j]);
 }
 
 template <typename T>
@@ -88,12 +99,12 @@ pf_status plan_init(pf_plan p) {
     PF_TRY(upload(p, &p->twQ64, tqd));
     PF_TRY(upload(p, &p->twP32, tpf));
     PF_TRY(upload(p, &p->twQ32, tqf));
-    std::vector<double2> t256d;
-    std::vector<float2> t256f;
-    twiddles(t256d, 256);
-    twiddles(t256f, 256);
-    PF_TRY(upload(p, &p->tw256_64, t256d));
-    PF_TRY(upload(p, &p->tw256_32, t256f));
+    std::vector<float2> pass;              // both in one allocation (one copy if P = Q)
+    pass_twiddles(pass, P);
+    const size_t np = pass.size();
+    if (Q != P) pass_twiddles(pass, Q);
+    PF_TRY(upload(p, &p->twP32_r, pass));
+    p->twQ32_r = p->twP32_r + (Q != P ? np : 0);
     std::vector<int4> fx;                  // both in one allocation (one copy if P = Q)
     fx_twiddles(fx, P);
     if (Q != P) fx_twiddles(fx, Q);
@@ -202,7 +213,7 @@ pf_status pf_plan_clone(pf_plan src, int32_t precision, void* stream, pf_plan* o
     p->shared->refs++;
     p->G = src->G; p->H64 = src->H64; p->H32 = src->H32; p->Hu64 = src->Hu64; p->Hv64 = src->Hv64;
     p->Hu32 = src->Hu32; p->Hv32 = src->Hv32; p->twP64 = src->twP64; p->twQ64 = src->twQ64; p->twP32 = src->twP32;
-    p->twQ32 = src->twQ32; p->tw256_64 = src->tw256_64; p->tw256_32 = src->tw256_32;
+    p->twQ32 = src->twQ32; p->twP32_r = src->twP32_r; p->twQ32_r = src->twQ32_r;
     p->twP_fx = src->twP_fx; p->twQ_fx = src->twQ_fx;
     // make sure the source's tables are complete before another stream reads them
     if (cudaStreamSynchronize(src->stream) != cudaSuccess) {

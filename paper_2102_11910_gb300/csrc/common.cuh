@@ -118,8 +118,8 @@ struct pf_plan_s {
     double2* twQ64 = nullptr;
     float2* twP32 = nullptr;
     float2* twQ32 = nullptr;
-    double2* tw256_64 = nullptr;   // exp(-2 pi i m / 256), m in [0, 256)
-    float2* tw256_32 = nullptr;
+    float2* twP32_r = nullptr;     // in the order of the register passes (fft_reg.cuh); twQ32_r is part of it
+    float2* twQ32_r = nullptr;
     int4* twP_fx = nullptr;        // twP, twQ in Q62 halves (fixfft.cu)
     int4* twQ_fx = nullptr;
     int* fx_exp = nullptr;         // exponents of the fixed-point passes: FXE_* below (per plan)

@@ -203,15 +203,14 @@ constexpr int FWD_GROUPS = 2;
 
 // Transforms a block of the inverse row pass.  A 32-byte sector of T2 holds
 // four rows' values of one k; a block that reads it for one row makes the pass
-// wait on L2 (2048 x 1800 nodes, velocity: 84 us with one row a block, 33 with
-// two, 36 with four; 768 x 512: 7.9, 6.4; 1024^2: 10.8, 10.8, 11.0).
+// wait on L2 (2048 x 1800 nodes, velocity: 84 us with one row a block, 28 with
+// two, a tenth more with four; at 1024^2 all three the same, 9.2).
 constexpr int INV_GROUPS = 2;
 
 template <typename T, int R3>
 __global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const T* __restrict__ w,
                                                                                 C_t<T>* __restrict__ T1, int nx,
-                                                                                int ny, const C_t<T>* __restrict__ tw256,
-                                                                                const C_t<T>* __restrict__ twP) {
+                                                                                int ny, const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = FWD_GROUPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -233,7 +232,7 @@ __global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const T* __
         const T a = w[(size_t)ja * nx + nc], b = w[(size_t)jb * nx + nc];
         v[r] = cmake<C>(n < nx && h0 ? a : T(0), n < nx && h1 ? b : T(0));
     }
-    fft_strided<C, false, R3>(v, buf, t, tw256, twP);
+    fft_strided<C, false, R3>(v, buf, t, tw);
 #pragma unroll
     for (int r = 0; r < 16; ++r) buf[spad(t + TP * r)] = v[r];
     __syncthreads();
@@ -255,12 +254,15 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 
 // Column pass.  The block's rows of the kernel spectra (Hu and Hv, or H) are
 // copied into shared memory by cp.async as the block starts, so their loads
-// overlap the column load and the forward transform.
+// overlap the column load and the forward transform.  128 registers a thread
+// hold the twiddles of all three transforms; loading them again in each (96
+// registers, five blocks an SM instead of four) measured 18.3 us against 16.0 at
+// 1024^2, 80 registers and six blocks 21.7, 168 and three 18.6.
 template <typename T, int R3>
 __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 1) k_cols_r(
     const C_t<T>* __restrict__ T1, C_t<T>* __restrict__ T2a, C_t<T>* __restrict__ T2b, int ny, int nk, int mode,
     const T* __restrict__ H, const T* __restrict__ Hu, const T* __restrict__ Hv, int Hld,
-    const C_t<T>* __restrict__ tw256, const C_t<T>* __restrict__ twQ) {
+    const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     constexpr int Q = 256 * R3, TQ = Q / 16, SB = SBuf<Q>::size;
     constexpr int NH = (Q / 2 + 1 + 3) / 4 * 4, PER = 16 / sizeof(T);   // spectrum row length, elements per copy
@@ -289,7 +291,7 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
         const C x = T1[spec_at(l < ny ? l : ny - 1, k, nk)];
         if (l < ny) v[r] = x;
     }
-    fft_strided<C, false, R3>(v, buf, t, tw256, twQ);
+    fft_strided<C, false, R3>(v, buf, t, tw);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (mode == CONV_UV) {
@@ -303,14 +305,14 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
             keep[spad(l)] = iw * hs1[lq];          // even in l
             v[r] = iw * (lo ? hu : -hu);            // odd in l
         }
-        fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
+        fft_strided<C, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 16; ++r) {               // rows past Q / 2 are not kept
             const int l = t + TQ * r;
             if (r < 8 && l < ny) T2a[spec_at(l, k, nk)] = v[r];
             v[r] = keep[spad(l)];                    // written by this thread
         }
-        fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
+        fft_strided<C, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
             const int l = t + TQ * r;
             v[r] = v[r] * hs0[l <= Q / 2 ? l : Q - l];
         }
-        fft_strided<C, true, R3>(v, buf, t, tw256, twQ);
+        fft_strided<C, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
 template <typename T, int R3>
 __global__ void __launch_bounds__(16 * R3 * INV_GROUPS, sizeof(T) == 4 && R3 >= 4 ? 1024 / (16 * R3 * INV_GROUPS) : 1)
     k_rows_inv_r(const C_t<T>* __restrict__ T2a, const C_t<T>* __restrict__ T2b, T* __restrict__ out, int nx, int ny,
-                 int mode, T Uinf, T Vinf, const C_t<T>* __restrict__ tw256, const C_t<T>* __restrict__ twP) {
+                 int mode, T Uinf, T Vinf, const C_t<T>* __restrict__ tw) {
     using C = C_t<T>;
     constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = INV_GROUPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -383,7 +385,7 @@ __global__ void __launch_bounds__(16 * R3 * INV_GROUPS, sizeof(T) == 4 && R3 >= 
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = buf[spad(t + TP * r)];
     __syncthreads();
-    fft_strided<C, true, R3>(v, buf, t, tw256, twP);
+    fft_strided<C, true, R3>(v, buf, t, tw);
     if (uv) {
         const int j = r0 + g;
         if (j < ny) {
@@ -416,7 +418,7 @@ struct ConvWs {
 
 template <typename T, int R3P, int R3Q>
 static pf_status conv_solve_r(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                              const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, const C_t<T>* tw256, ConvWs ws) {
+                              const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
     using C = C_t<T>;
     constexpr int P = 256 * R3P, Q = 256 * R3Q;
     const int nx = p->nx, ny = p->ny;
@@ -428,39 +430,39 @@ static pf_status conv_solve_r(pf_plan p, const T* w, T* out, int mode, T Uinf, T
     C* T2a = reinterpret_cast<C*>(ws.T2a);
     C* T2b = reinterpret_cast<C*>(ws.T2b);
     PF_KERNEL(p, "fft_rows_fwd", PF_CUDA(p, pf_launch(k_rows_fwd_r<T, R3P>, ceil_div(ny, 2 * FWD_GROUPS), 16 * R3P * FWD_GROUPS, sf, p->stream, w, T1,
-                                                      nx, ny, tw256, twP)));
+                                                      nx, ny, twP)));
     PF_KERNEL(p, "fft_cols_conv", PF_CUDA(p, pf_launch(k_cols_r<T, R3Q>, P / 2 + 1, 16 * R3Q, sc, p->stream, T1, T2a,
-                                                       T2b, ny, P / 2 + 1, mode, H, Hu, Hv, p->Hld, tw256, twQ)));
+                                                       T2b, ny, P / 2 + 1, mode, H, Hu, Hv, p->Hld, twQ)));
     const int nb = mode == CONV_UV ? ceil_div(ny, INV_GROUPS) : ceil_div(ny, 2 * INV_GROUPS);
     const size_t sr = INV_GROUPS * (size_t)SBuf<P>::size * sizeof(C);
     PF_CUDA(p, set_smem(k_rows_inv_r<T, R3P>, sr));
     PF_KERNEL(p, "fft_rows_inv", PF_CUDA(p, pf_launch(k_rows_inv_r<T, R3P>, nb, 16 * R3P * INV_GROUPS, sr, p->stream, T2a, T2b,
-                                                      out, nx, ny, mode, Uinf, Vinf, tw256, twP)));
+                                                      out, nx, ny, mode, Uinf, Vinf, twP)));
     return PF_OK;
 }
 
 template <typename T, int R3P>
 static pf_status conv_dispatch_q(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                                 const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, const C_t<T>* tw256, ConvWs ws) {
+                                 const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
     switch (p->Q) {
-        case 256: return conv_solve_r<T, R3P, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 512: return conv_solve_r<T, R3P, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 1024: return conv_solve_r<T, R3P, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 2048: return conv_solve_r<T, R3P, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 4096: return conv_solve_r<T, R3P, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
+        case 256: return conv_solve_r<T, R3P, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 512: return conv_solve_r<T, R3P, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 1024: return conv_solve_r<T, R3P, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 2048: return conv_solve_r<T, R3P, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 4096: return conv_solve_r<T, R3P, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
     }
     return PF_ERR_ARG;
 }
 
 template <typename T>
 static pf_status conv_dispatch(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                               const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, const C_t<T>* tw256, ConvWs ws) {
+                               const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
     switch (p->P) {
-        case 256: return conv_dispatch_q<T, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 512: return conv_dispatch_q<T, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 1024: return conv_dispatch_q<T, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 2048: return conv_dispatch_q<T, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
-        case 4096: return conv_dispatch_q<T, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, tw256, ws);
+        case 256: return conv_dispatch_q<T, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 512: return conv_dispatch_q<T, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 1024: return conv_dispatch_q<T, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 2048: return conv_dispatch_q<T, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 4096: return conv_dispatch_q<T, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
     }
     return PF_ERR_ARG;
 }
@@ -497,7 +499,7 @@ pf_status conv_solve(pf_plan p, const void* w, void* out, int mode, double Uinf,
     }
     if (reg)
         return conv_dispatch<float>(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
-                                    p->Hv32, p->twP32, p->twQ32, p->tw256_32, ws);
+                                    p->Hv32, p->twP32_r, p->twQ32_r, ws);
     return conv_solve_t<float>(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
                                p->Hv32, p->twP32, p->twQ32, ws);
 }

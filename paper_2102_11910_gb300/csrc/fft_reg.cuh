@@ -6,7 +6,15 @@
 // without leaving registers.  Stockham autosort passes of radix 16, 16, R3;
 // data cross between threads through one shared buffer of N complex values,
 // twice.  Forward: X(k) = sum_n x(n) exp(-2 pi i k n / N); inverse: +i,
-// unnormalised.  tw256[m] = exp(-2 pi i m / 256), twN[m] = exp(-2 pi i m / N).
+// unnormalised.
+//
+// Twiddles come from a table in the order in which the passes read it, a
+// multiplier r at a time, so that a warp's load is one or two lines at a fixed
+// distance: tw[(r - 1) 16 + k] = exp(-2 pi i r k / 256), r = 1 .. 15, k < 16, then
+// [(r - 1) 256 + j] = exp(-2 pi i r j / N), r = 1 .. R3 - 1, j < 256.  Gathered from
+// one table of powers by r k and r j, a load took up to 16 lines and an address
+// of its own (2048 x 1800 nodes, velocity: rows 16.4, columns 68, rows 32.9 us
+// became 14.5, 62.8, 28.1; 1024^2: 6.4, 17.9, 10.7 became 5.9, 16.0, 9.2).
 #pragma once
 #include <type_traits>
 
@@ -118,6 +126,7 @@ __device__ __forceinline__ void dft_r(C* v) {
     else if constexpr (R == 2) dft2<C, INV>(v[0], v[1]);
 }
 
+constexpr int TW_PASS3 = 15 * 16;        // where the second part begins
 template <typename C, bool INV>
 __device__ __forceinline__ C twiddle(const C* __restrict__ tw, int m) {
     C w = tw[m];
@@ -134,8 +143,7 @@ template <int N> struct SBuf { static constexpr int size = N + N / 16; };
 // is the group's shared buffer (SBuf<N>::size complex).  All threads of the
 // block must call this the same number of times (it contains __syncthreads).
 template <typename C, bool INV, int R3>
-__device__ __forceinline__ void fft_strided(C (&v)[16], C* buf, int t, const C* __restrict__ tw256,
-                                            const C* __restrict__ twN) {
+__device__ __forceinline__ void fft_strided(C (&v)[16], C* buf, int t, const C* __restrict__ tw) {
     constexpr int N = 256 * R3;
     constexpr int T = N / 16;
     // pass 1: radix 16, Ns = 1; inputs v[r] = x[t + T r]; outputs to 16 t + r
@@ -149,7 +157,7 @@ __device__ __forceinline__ void fft_strided(C (&v)[16], C* buf, int t, const C* 
 #pragma unroll
         for (int r = 0; r < 16; ++r) v[r] = buf[spad(t + T * r)];
 #pragma unroll
-        for (int r = 1; r < 16; ++r) v[r] = v[r] * twiddle<C, INV>(tw256, r * k);
+        for (int r = 1; r < 16; ++r) v[r] = v[r] * twiddle<C, INV>(tw + k, (r - 1) * 16);
         dft16<C, INV>(v);
         __syncthreads();
         if (R3 == 1) return;          // N = 256: outputs t + 16 r already in place
@@ -170,7 +178,7 @@ __device__ __forceinline__ void fft_strided(C (&v)[16], C* buf, int t, const C* 
 #pragma unroll
             for (int r = 0; r < R3; ++r) u[r] = buf[spad(j + 256 * r)];
 #pragma unroll
-            for (int r = 1; r < R3; ++r) u[r] = u[r] * twiddle<C, INV>(twN, r * j);
+            for (int r = 1; r < R3; ++r) u[r] = u[r] * twiddle<C, INV>(tw + TW_PASS3 + j, (r - 1) * 256);
             dft_r<C, INV, R3>(u);
 #pragma unroll
             for (int r = 0; r < R3; ++r) v[m + r * M] = u[r];
