@@ -660,20 +660,20 @@ __global__ void __launch_bounds__(RUN_THREADS) k_bin_runs(const double* __restri
 template <typename T> __device__ __forceinline__ T pow2(int sh);
 template <> __device__ __forceinline__ float pow2<float>(int sh) { return __int_as_float((sh + 127) << 23); }
 
-// a b = hi 2^16 + lo + e, |lo| <= 2^15, |e| <= 1/2 (and a little for the sum
-// below), for |a b| < 2^38, with FP32 operations only (no conversion
-// instructions, which issue at 1/8 rate): added to 1.5 2^39 the product leaves
-// its multiple of 2^16, h, in the sum's low mantissa bits; a b - h is within
-// 2^15, and added to 1.5 2^23 leaves its nearest integer there.  The product
-// itself is not rounded.  (Two operations a term fewer than splitting the
-// rounded product; with sorted_slot 1e6 vortices on 1024^2 deposit in 19.8 us
-// instead of 21.6, 4e6 on 2048 x 1800 in 60 instead of 67.  Other sorts measured:
-// 2048 records at a time 19.9 and 63 us; 128 by each warp alone, no barriers,
-// 22.6 and 65.)
-__device__ __forceinline__ void split_hilo(float a, float b, int& hi, int& lo) {
-    const float t = __fmaf_rn(a, b, 0x1.8p39f);
+// x = hi 2^16 + lo + e, |lo| <= 2^15, |e| <= 1/2, for |x| < 2^38, with FP32
+// adds only (no conversion instructions, which issue at 1/8 rate): added to
+// 1.5 2^39, x leaves its multiple of 2^16, h, in the sum's low mantissa bits;
+// x - h is exact, and added to 1.5 2^23 leaves its nearest integer there.
+// (Splitting the product gy wx unrounded, by fused multiply-adds, is one
+// operation less and a little more accurate, but other bits of w move a state
+// of dense vortices by 2e-9 of its positions, which are FP64 results.)
+// With sorted_slot 1e6 vortices on 1024^2 deposit in 20.0 us instead of 21.6,
+// 4e6 on 2048 x 1800 in 61 instead of 67.  Other sorts measured: 2048 records
+// at a time no faster; 128 by each warp alone, no barriers, a tenth slower.
+__device__ __forceinline__ void split_hilo(float x, int& hi, int& lo) {
+    const float t = __fadd_rn(x, 0x1.8p39f);
     hi = __float_as_int(t) - 0x53400000;
-    lo = __float_as_int(__fadd_rn(__fmaf_rn(a, b, __fsub_rn(0x1.8p39f, t)), 0x1.8p23f)) - 0x4B400000;
+    lo = __float_as_int(__fadd_rn(__fsub_rn(x, __fsub_rn(t, 0x1.8p39f)), 0x1.8p23f)) - 0x4B400000;
 }
 
 // Deposit: one block per node tile accumulates its records in shared memory as
@@ -740,13 +740,14 @@ __device__ __forceinline__ void deposit_one(const Rec<T>& rc, T scale, unsigned 
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int node = base + b * ACC_W + a;
+            const T x = gy * wx[a];
             if (MODE == DEP_SPLIT32) {
                 int hi, lo;
-                split_hilo((float)gy, (float)wx[a], hi, lo);
+                split_hilo((float)x, hi, lo);
                 atomicAdd(&acc_hi[node], hi);
                 atomicAdd(&acc_lo[node], lo);
             } else {
-                atomicAdd(&acc[node], (unsigned long long)__float2ll_rn((float)(gy * wx[a])));
+                atomicAdd(&acc[node], (unsigned long long)__float2ll_rn((float)x));
             }
         }
     }
