@@ -1263,27 +1263,19 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
 // U records a thread a chunk.  Dynamic shared memory: (U x blockDim + 32)
 // records.  Five blocks an SM (48 registers): with 64 registers, so four, 1e6
 // vortices on 1024^2 took 22.4 us instead of 20.5.
-template <int TILE, int U, typename BINS>
-__global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* __restrict__ recs, BINS bins,
-                                                          const float2* __restrict__ uv, Geo geo,
-                                                          float* __restrict__ uq, float* __restrict__ vq, int64_t nq,
-                                                          int* __restrict__ status) {
-    constexpr int PATCH = TILE + 3, PAIRS = (PATCH + 1) / 2;   // 18 pairs per patch row at TILE 32
-    __shared__ float4 pe[PATCH * PAIRS];
-    __shared__ float4 po[PATCH * PAIRS];
-    __shared__ int bcnt[32], bstart[32], nhome;
-    extern __shared__ __align__(16) unsigned char interp_dyn[];
-    Rec<float>* srt = reinterpret_cast<Rec<float>*>(interp_dyn);
-    const int t = blockIdx.x;
-    pdl_wait();
-    double unused;
-    const auto src = open_tile<false>(bins, recs, t, status, unused);
-    const int cnt = src.cnt;
-    if (cnt == 0) return;                         // block-uniform
-    Rec<float> rc[U];
-    src.load(0, rc);                              // in flight while the patch is staged
-    if (threadIdx.x < 32) bcnt[threadIdx.x] = 0;
-    const int tx = t % geo.ntx, ty = t / geo.ntx;
+template <int TILE> struct InterpSmem {
+    static constexpr int PATCH = TILE + 3, PAIRS = (PATCH + 1) / 2;   // 18 pairs per patch row at TILE 32
+    float4 pe[PATCH * PAIRS];
+    float4 po[PATCH * PAIRS];
+    int bcnt[32], bstart[32], nhome;
+};
+
+// The tile's patch; a barrier follows it
+template <int TILE>
+__device__ __forceinline__ void stage_patch(InterpSmem<TILE>& sm, const float2* __restrict__ uv, const Geo& geo, int tx,
+                                            int ty) {
+    constexpr int PATCH = InterpSmem<TILE>::PATCH, PAIRS = InterpSmem<TILE>::PAIRS;
+    if (threadIdx.x < 32) sm.bcnt[threadIdx.x] = 0;
     const int gi0 = tx * TILE - 1, gj0 = ty * TILE - 1;
     // patch nodes px, py in [0, 2 PAIRS) x [0, PATCH); px = 2 PAIRS - 1 only pads
     for (int i = threadIdx.x; i < PATCH * 2 * PAIRS; i += blockDim.x) {
@@ -1291,18 +1283,28 @@ __global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* _
         const int gi = gi0 + px, gj = gj0 + py;
         float2 v = make_float2(0.f, 0.f);
         if (px < PATCH && gi >= 0 && gi < geo.nx && gj >= 0 && gj < geo.ny) v = uv[(size_t)gj * geo.nx + gi];
-        float* e = reinterpret_cast<float*>(&pe[py * PAIRS + px / 2]) + 2 * (px & 1);
+        float* e = reinterpret_cast<float*>(&sm.pe[py * PAIRS + px / 2]) + 2 * (px & 1);
         e[0] = v.x;
         e[1] = v.y;
         if (px >= 1) {
-            float* o = reinterpret_cast<float*>(&po[py * PAIRS + (px - 1) / 2]) + 2 * ((px - 1) & 1);
+            float* o = reinterpret_cast<float*>(&sm.po[py * PAIRS + (px - 1) / 2]) + 2 * ((px - 1) & 1);
             o[0] = v.x;
             o[1] = v.y;
         }
     }
-    __syncthreads();
+}
+
+// one(record, u, v, place) for each home record: place counts them up without
+// gaps, a row of lanes on end.  rc: the thread's first U; srt: U x blockDim + 32.
+// Returns their number.  CHAIN: a row's four terms added from the left, fused;
+// a state's FP64 positions follow these bits.
+template <int TILE, bool CHAIN, int U, typename SRC, typename F>
+__device__ __forceinline__ int interp_home_records(InterpSmem<TILE>& sm, const SRC& src, Rec<float> (&rc)[U],
+                                                   Rec<float>* srt, F one) {
+    constexpr int PAIRS = InterpSmem<TILE>::PAIRS;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
-    const int stride = U * (int)blockDim.x;
+    const int stride = U * (int)blockDim.x, cnt = src.cnt;
+    int seen = 0;
     for (int r0 = 0; r0 < cnt; r0 += stride) {
         const int n = cnt - r0 < stride ? cnt - r0 : stride;
         int key[U], pos[U];
@@ -1311,25 +1313,27 @@ __global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* _
             const int lx = rec_lx(rc[u]), ly = rec_ly(rc[u]);
             const bool home = u * (int)blockDim.x + (int)threadIdx.x < n && lx >= 0 && lx < TILE && ly >= 0 &&
                               ly < TILE;
-            const float4* row = ((lx & 1) ? po + (lx - 1) / 2 : pe + lx / 2) + ly * PAIRS;
+            const float4* row = ((lx & 1) ? sm.po + (lx - 1) / 2 : sm.pe + lx / 2) + ly * PAIRS;
             key[u] = home ? (int)((__cvta_generic_to_shared(row) >> 4) & 31) : -1;
-            pos[u] = home ? atomicAdd(&bcnt[key[u]], 1) : 0;
+            pos[u] = home ? atomicAdd(&sm.bcnt[key[u]], 1) : 0;
         }
         __syncthreads();
         if (wid == 0) {                               // bucket starts; counters cleared for the next chunk
-            const int c = bcnt[lane];
+            const int c = sm.bcnt[lane];
             const int incl = warp_incl_scan(c, lane);
-            bstart[lane] = incl - c;
-            bcnt[lane] = 0;
-            if (lane == 31) nhome = incl;
+            sm.bstart[lane] = incl - c;
+            sm.bcnt[lane] = 0;
+            if (lane == 31) sm.nhome = incl;
         }
         __syncthreads();
-        const int nh = nhome, R = (nh + 31) >> 5;
+        const int nh = sm.nhome, R = (nh + 31) >> 5;
         const unsigned inv = SLOT_INV.m[R];
+        // row i holds full + (i < more) records, from lane 0 on
+        const int full = (int)(((unsigned)nh * inv) >> 20), more = nh - full * R;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (key[u] >= 0) {
-                srt[sorted_slot(bstart[key[u]] + pos[u], R, inv)] = rc[u];
+                srt[sorted_slot(sm.bstart[key[u]] + pos[u], R, inv)] = rc[u];
             }
         }
         if (r0 + stride < cnt) src.load(r0 + stride, rc);   // the next chunk in flight
@@ -1341,25 +1345,55 @@ __global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* _
             float wx[4], wy[4];
             m4p_weights(rec_fx(rcu), wx);
             m4p_weights(rec_fy(rcu), wy);
-            const float4* rows = (lx & 1) ? po + (lx - 1) / 2 : pe + lx / 2;   // node px = lx is the first
+            const float4* rows = (lx & 1) ? sm.po + (lx - 1) / 2 : sm.pe + lx / 2;   // node px = lx is the first
             float su = 0.f, sv = 0.f;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 const float4 p0 = rows[(ly + b) * PAIRS], p1 = rows[(ly + b) * PAIRS + 1];
-                const float ru = wx[0] * p0.x + wx[1] * p0.z + wx[2] * p1.x + wx[3] * p1.z;
-                const float rv = wx[0] * p0.y + wx[1] * p0.w + wx[2] * p1.y + wx[3] * p1.w;
+                float ru, rv;
+                if (CHAIN) {
+                    ru = __fmaf_rn(wx[3], p1.z, __fmaf_rn(wx[2], p1.x, __fmaf_rn(wx[1], p0.z, __fmul_rn(wx[0], p0.x))));
+                    rv = __fmaf_rn(wx[3], p1.w, __fmaf_rn(wx[2], p1.y, __fmaf_rn(wx[1], p0.w, __fmul_rn(wx[0], p0.y))));
+                } else {
+                    ru = wx[0] * p0.x + wx[1] * p0.z + wx[2] * p1.x + wx[3] * p1.z;
+                    rv = wx[0] * p0.y + wx[1] * p0.w + wx[2] * p1.y + wx[3] * p1.w;
+                }
                 su += wy[b] * ru;
                 sv += wy[b] * rv;
             }
-            if (rcu.q < 0 || rcu.q >= nq) {
-                atomicOr(status, ST_INTERNAL);
-                continue;
-            }
-            uq[rcu.q] = su;
-            vq[rcu.q] = sv;
+            one(rcu, su, sv, seen + i * full + min(i, more) + lane);
         }
+        seen += nh;
         __syncthreads();                              // srt and the counters are reused
     }
+    return seen;
+}
+
+template <int TILE, int U, typename BINS>
+__global__ void __launch_bounds__(256, 5) k_interp_tiles_f32(const Rec<float>* __restrict__ recs, BINS bins,
+                                                          const float2* __restrict__ uv, Geo geo,
+                                                          float* __restrict__ uq, float* __restrict__ vq, int64_t nq,
+                                                          int* __restrict__ status) {
+    __shared__ InterpSmem<TILE> sm;
+    extern __shared__ __align__(16) unsigned char interp_dyn[];
+    const int t = blockIdx.x;
+    pdl_wait();
+    double unused;
+    const auto src = open_tile<false>(bins, recs, t, status, unused);
+    if (src.cnt == 0) return;                     // block-uniform
+    Rec<float> rc[U];
+    src.load(0, rc);                              // in flight while the patch is staged
+    stage_patch<TILE>(sm, uv, geo, t % geo.ntx, t / geo.ntx);
+    __syncthreads();
+    interp_home_records<TILE, false>(sm, src, rc, reinterpret_cast<Rec<float>*>(interp_dyn),
+                              [&](const Rec<float>& r, float su, float sv, int) {
+                                  if (r.q < 0 || r.q >= nq) {
+                                      atomicOr(status, ST_INTERNAL);
+                                      return;
+                                  }
+                                  uq[r.q] = su;
+                                  vq[r.q] = sv;
+                              });
 }
 
 // E_v at arbitrary points, FP64: a thread a point.

@@ -13,7 +13,9 @@
 //              patch, the position moved by dt (u, v) in fixed point, the new
 //              record kept at the old slot, the number of records bound for
 //              each tile of the 5 x 5 block around it, added into the new
-//              tile counts;
+//              tile counts (zero before: each step's scatter clears the counts
+//              it was the last to read, so that no memset stands between the
+//              launches, which breaks their overlap: 3 us a step);
 //   offsets    one block: the new tile starts (a scan of the counts);
 //   scatter    per source tile: a slice of every destination tile claimed with
 //              one atomic add, records copied to their new tiles (home and
@@ -135,24 +137,72 @@ __device__ __forceinline__ bool moved_dest(int ci, int cj, int tx, int ty, const
     return true;
 }
 
-// E_v and the Euler move of every home record of a tile.  The tile's velocity
-// patch (nodes -1 .. 33 in each direction) is staged in shared memory; the
-// advected record goes to moved[slot]; the block counts its records per
-// destination tile (a vortex whose new stencil straddles tiles is counted in
-// each of them).  Optionally writes the velocity at the vortex's original
-// index.
+// The Euler move of a home record with velocity (su, sv): its new cell and
+// fraction relative to the source tile, and its destination tiles counted in
+// lcnt (counting the source tile itself, nearly every one's, in a register and
+// adding it at the end made the pass slower: 801 against 794 us for eight
+// steps).  Optionally writes the velocity at the vortex's original index.
 template <typename T>
-__global__ void __launch_bounds__(256) k_vic_advect(const Rec<T>* __restrict__ recs, const int* __restrict__ tile_start,
-                                                    const unsigned* __restrict__ tile_count,
-                                                    const C_t<T>* __restrict__ uv, Geo geo, T dt_dx,
-                                                    Moved<T>* __restrict__ moved, int* __restrict__ dcount,
-                                                    unsigned* __restrict__ tcount_next,
-                                                    T* __restrict__ uq, T* __restrict__ vq, int64_t rec_cap,
-                                                    int64_t nq, int* __restrict__ status,
-                                                    unsigned long long* __restrict__ oob) {
+struct Advance {
+    const Geo& geo;
+    T dt_dx;
+    int tx, ty;
+    int* lcnt;
+    T *uq, *vq;
+    int64_t nq;
+    int* status;
+    unsigned long long* oob;
+    __device__ __forceinline__ Moved<T> operator()(const Rec<T>& rc, T su, T sv) {
+        if (uq != nullptr && rc.q >= 0 && rc.q < nq) {
+            uq[rc.q] = su;
+            vq[rc.q] = sv;
+        }
+        int ci = rec_lx(rc), cj = rec_ly(rc);
+        Moved<T> m = {};
+        if constexpr (sizeof(T) == 4) {
+            move_axis(rc.xw, su * dt_dx, ci, m.xw);
+            move_axis(rc.yw, sv * dt_dx, cj, m.yw);
+        } else {
+            move_axis(rc.fx, su * dt_dx, ci, m.fx);
+            move_axis(rc.fy, sv * dt_dx, cj, m.fy);
+        }
+        int x0, x1, y0, y1;
+        if (!moved_dest(ci, cj, tx, ty, geo, x0, x1, y0, y1, status, oob)) {
+            m = {};
+            m.q = -1;
+            return m;
+        }
+        if constexpr (sizeof(T) == 4) {
+            m.xw = (m.xw & ~0xFFu) | (unsigned)(ci + MOVE_BIAS);
+            m.yw = (m.yw & ~0xFFu) | (unsigned)(cj + MOVE_BIAS);
+        } else {
+            m.lx = (short)ci;
+            m.ly = (short)cj;
+        }
+        m.g = rc.g;
+        m.q = rc.q;
+        for (int dy = y0; dy <= y1; ++dy)
+            for (int dx = x0; dx <= x1; ++dx) atomicAdd(&lcnt[dir_of(dx, dy)], 1);
+        return m;
+    }
+};
+
+// E_v and the move of every home record of a tile; the moved records go to the
+// tile's slots in `moved`.  FP64: a thread a record, from the staged patch
+// (nodes -1 .. 33 in each direction).  FP32: as k_interp_tiles_f32, the records
+// in bank order, moved ones packed and the slots left marked empty (1e6
+// vortices on 1024^2, eight steps with set and get: 794 -> 775 us against a
+// thread a record there too).
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_vic_advect(
+    const Rec<T>* __restrict__ recs, const int* __restrict__ tile_start, const unsigned* __restrict__ tile_count,
+    const C_t<T>* __restrict__ uv, Geo geo, T dt_dx, Moved<T>* __restrict__ moved, int* __restrict__ dcount,
+    unsigned* __restrict__ tcount_next, T* __restrict__ uq, T* __restrict__ vq, int64_t rec_cap, int64_t nq,
+    int* __restrict__ status, unsigned long long* __restrict__ oob) {
     using C = C_t<T>;
-    __shared__ C patch[PATCH * PATCH];
+    __shared__ typename std::conditional<sizeof(T) == 4, InterpSmem<BIN_TILE>, C[PATCH * PATCH]>::type sm;
     __shared__ int lcnt[NDIR];
+    extern __shared__ __align__(16) unsigned char advect_dyn[];
     const int t = blockIdx.x;
     const int tx = t % geo.ntx, ty = t / geo.ntx;
     if (threadIdx.x < NDIR) lcnt[threadIdx.x] = 0;
@@ -162,81 +212,71 @@ __global__ void __launch_bounds__(256) k_vic_advect(const Rec<T>* __restrict__ r
     const bool ok = start >= 0 && cnt >= 0 && (int64_t)start + cnt <= rec_cap;     // block-uniform
     if (!ok && threadIdx.x == 0) atomicOr(status, ST_INTERNAL);
     const int n = ok ? cnt : 0;
-    if (n > 0) {
-        const int gi0 = tx * BIN_TILE - 1, gj0 = ty * BIN_TILE - 1;
-        for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {
-            const int gi = gi0 + i % PATCH, gj = gj0 + i / PATCH;
-            C v = cmake<C>(T(0), T(0));
-            if (gi >= 0 && gi < geo.nx && gj >= 0 && gj < geo.ny) v = uv[(size_t)gj * geo.nx + gi];
-            patch[i] = v;
+    Advance<T> advance{geo, dt_dx, tx, ty, lcnt, uq, vq, nq, status, oob};
+    if constexpr (sizeof(T) == 4) {
+        if (n > 0) {
+            const FlatRecs<float> src{recs + start, n};
+            Rec<float> rc[REC_U];
+            src.load(0, rc);
+            stage_patch<BIN_TILE>(sm, uv, geo, tx, ty);
+            __syncthreads();
+            const int homes = interp_home_records<BIN_TILE, true>(
+                sm, src, rc, reinterpret_cast<Rec<float>*>(advect_dyn),
+                [&](const Rec<float>& r, float su, float sv, int place) { moved[start + place] = advance(r, su, sv); });
+            Moved<float> none = {};
+            none.q = -1;
+            for (int r = homes + threadIdx.x; r < n; r += 256) moved[start + r] = none;
         }
-    }
-    __syncthreads();
-    constexpr int U = 4;
-    for (int r0 = 0; r0 < n; r0 += U * 256) {
-      Rec<T> rcs[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {          // clamped: a thread past the end reloads the last record
-          const int r = r0 + u * 256 + (int)threadIdx.x;
-          rcs[u] = recs[start + (r < n ? r : n - 1)];
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int r = r0 + u * 256 + threadIdx.x;
-        if (r >= n) break;
-        const Rec<T> rc = rcs[u];
-        const int lx = rec_lx(rc), ly = rec_ly(rc);
-        Moved<T> m = {};
-        m.q = -1;
-        if (lx >= 0 && lx < BIN_TILE && ly >= 0 && ly < BIN_TILE) {
-            T wx[4], wy[4];
-            m4p_weights(rec_fx(rc), wx);
-            m4p_weights(rec_fy(rc), wy);
-            T su = 0, sv = 0;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const C* row = patch + (ly + b) * PATCH + lx;    // node (lx - 1 + a, ly - 1 + b)
-                T ru = 0, rv = 0;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const C c = row[a];
-                    ru += wx[a] * c.x;
-                    rv += wx[a] * c.y;
-                }
-                su += wy[b] * ru;
-                sv += wy[b] * rv;
-            }
-            if (uq != nullptr && rc.q >= 0 && rc.q < nq) {
-                uq[rc.q] = su;
-                vq[rc.q] = sv;
-            }
-            int ci = lx, cj = ly;
-            Moved<T> mv = {};
-            if constexpr (sizeof(T) == 4) {
-                move_axis(rc.xw, su * dt_dx, ci, mv.xw);
-                move_axis(rc.yw, sv * dt_dx, cj, mv.yw);
-            } else {
-                move_axis(rc.fx, su * dt_dx, ci, mv.fx);
-                move_axis(rc.fy, sv * dt_dx, cj, mv.fy);
-            }
-            int x0, x1, y0, y1;
-            if (moved_dest(ci, cj, tx, ty, geo, x0, x1, y0, y1, status, oob)) {
-                if constexpr (sizeof(T) == 4) {
-                    mv.xw = (mv.xw & ~0xFFu) | (unsigned)(ci + MOVE_BIAS);
-                    mv.yw = (mv.yw & ~0xFFu) | (unsigned)(cj + MOVE_BIAS);
-                } else {
-                    mv.lx = (short)ci;
-                    mv.ly = (short)cj;
-                }
-                mv.g = rc.g;
-                mv.q = rc.q;
-                m = mv;
-                for (int dy = y0; dy <= y1; ++dy)
-                    for (int dx = x0; dx <= x1; ++dx) atomicAdd(&lcnt[dir_of(dx, dy)], 1);
+    } else {
+        if (n > 0) {
+            const int gi0 = tx * BIN_TILE - 1, gj0 = ty * BIN_TILE - 1;
+            for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {
+                const int gi = gi0 + i % PATCH, gj = gj0 + i / PATCH;
+                C v = cmake<C>(T(0), T(0));
+                if (gi >= 0 && gi < geo.nx && gj >= 0 && gj < geo.ny) v = uv[(size_t)gj * geo.nx + gi];
+                sm[i] = v;
             }
         }
-        moved[start + r] = m;
-      }
+        __syncthreads();
+        constexpr int U = 4;
+        for (int r0 = 0; r0 < n; r0 += U * 256) {
+            Rec<T> rcs[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {          // clamped: a thread past the end reloads the last record
+                const int r = r0 + u * 256 + (int)threadIdx.x;
+                rcs[u] = recs[start + (r < n ? r : n - 1)];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int r = r0 + u * 256 + threadIdx.x;
+                if (r >= n) break;
+                const Rec<T> rc = rcs[u];
+                const int lx = rec_lx(rc), ly = rec_ly(rc);
+                Moved<T> m = {};
+                m.q = -1;
+                if (lx >= 0 && lx < BIN_TILE && ly >= 0 && ly < BIN_TILE) {
+                    T wx[4], wy[4];
+                    m4p_weights(rec_fx(rc), wx);
+                    m4p_weights(rec_fy(rc), wy);
+                    T su = 0, sv = 0;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const C* row = sm + (ly + b) * PATCH + lx;    // node (lx - 1 + a, ly - 1 + b)
+                        T ru = 0, rv = 0;
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) {
+                            const C c = row[a];
+                            ru += wx[a] * c.x;
+                            rv += wx[a] * c.y;
+                        }
+                        su += wy[b] * ru;
+                        sv += wy[b] * rv;
+                    }
+                    m = advance(rc, su, sv);
+                }
+                moved[start + r] = m;
+            }
+        }
     }
     __syncthreads();
     if (threadIdx.x < NDIR) {
@@ -346,7 +386,7 @@ __device__ __forceinline__ void scatter_one(const Moved<T>& m, bool live, const 
 template <typename T>
 __global__ void __launch_bounds__(256) k_vic_scatter(const Moved<T>* __restrict__ moved,
                                                      const int* __restrict__ tile_start,
-                                                     const unsigned* __restrict__ tile_count,
+                                                     unsigned* __restrict__ tile_count,
                                                      const int* __restrict__ dcount, int ntx,
                                                      int* __restrict__ fill, int64_t rec_cap,
                                                      Rec<T>* __restrict__ out, long long* __restrict__ nrec,
@@ -362,8 +402,9 @@ __global__ void __launch_bounds__(256) k_vic_scatter(const Moved<T>* __restrict_
         base[threadIdx.x] = c ? atomicAdd(&fill[t + (threadIdx.x / 5 - 2) * ntx + (threadIdx.x % 5 - 2)], c) : 0;
     }
     if (threadIdx.x == 0) nhome = 0;
-    __syncthreads();
     const int cnt = (int)tile_count[t];
+    __syncthreads();
+    if (threadIdx.x == 0) tile_count[t] = 0;         // read for the last time: the next step counts into it
     const int start = tile_start[t];
     if (!(start >= 0 && cnt >= 0 && (int64_t)start + cnt <= rec_cap)) return;   // reported by the advect pass
     constexpr int U = 4;
@@ -404,9 +445,13 @@ __global__ void k_vic_get(const Rec<T>* __restrict__ recs, const int* __restrict
     }
 }
 
-__global__ void k_fill_nan(double* a, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = __longlong_as_double(0x7FF8000000000000ll);
+__global__ void k_fill_nan(double* __restrict__ X, double* __restrict__ Y, double* __restrict__ G, int64_t n) {
+    const double nan = __longlong_as_double(0x7FF8000000000000ll);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        X[i] = nan;
+        Y[i] = nan;
+        G[i] = nan;
+    }
 }
 
 void free_state(pf_vic_state s) {
@@ -425,8 +470,8 @@ pf_status vic_step_t(pf_vic_state s, double dt, double Uinf, double Vinf, T* uq,
     PF_TRY((deposit_launch<T, BIN_TILE>(p, geo, rc, s->tstart[c], s->tcount[c], s->gmax, s->rec_cap, p->d_status,
                                         (T*)p->w, p->stream)));
     PF_TRY(conv_solve(p, p->w, p->uv, CONV_UV, Uinf, Vinf));
-    PF_CUDA(p, cudaMemsetAsync(s->tcount[n], 0, (size_t)geo.ntiles * sizeof(unsigned), p->stream));
-    PF_KERNEL(p, "vic_advect", PF_CUDA(p, pf_launch(k_vic_advect<T>, geo.ntiles, 256, 0, p->stream, rc, s->tstart[c],
+    const size_t adv_smem = sizeof(T) == 4 ? (size_t)(REC_U * 256 + 32) * sizeof(Rec<T>) : 0;
+    PF_KERNEL(p, "vic_advect", PF_CUDA(p, pf_launch(k_vic_advect<T>, geo.ntiles, 256, adv_smem, p->stream, rc, s->tstart[c],
                                                    s->tcount[c], (const C_t<T>*)p->uv, geo, (T)(dt / p->dx),
                                                    (Moved<T>*)s->moved, s->dcount, s->tcount[n], uq, vq, s->rec_cap,
                                                    s->nv0, p->d_status, p->d_oob)));
@@ -475,7 +520,8 @@ pf_status pf_vic_state_create(pf_plan p, int64_t capacity, pf_vic_state* out) {
     if (e == cudaSuccess) e = cudaMalloc(&s->fill, nt * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&s->gmax, (BIN_MAX_BLOCKS + 1) * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&s->nrec, 2 * sizeof(long long));
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->tcount[0], 0, nt * sizeof(unsigned), p->stream);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+        e = cudaMemsetAsync(s->tcount[i], 0, nt * sizeof(unsigned), p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->tstart[0], 0, nt * sizeof(int), p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->gmax, 0, sizeof(double), p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->nrec, 0, 2 * sizeof(long long), p->stream);
@@ -504,6 +550,8 @@ pf_status pf_vic_state_set(pf_vic_state s, const double* X, const double* Y, con
     bw.tile_start = s->tstart[0];
     bw.gmax = s->gmax;
     const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0);
+    // the first step counts into the other one
+    PF_CUDA(p, cudaMemsetAsync(s->tcount[1], 0, (size_t)geo.ntiles * sizeof(unsigned), p->stream));
     if (p->prec == PF_FP64) PF_TRY(bin_launch<double>(p, geo, bw, X, Y, G, nv, p->stream));
     else PF_TRY(bin_launch<float>(p, geo, bw, X, Y, G, nv, p->stream));
     const long long cnt[2] = {0, (long long)nv};
@@ -522,10 +570,8 @@ pf_status pf_vic_state_get(pf_vic_state s, double* X, double* Y, double* G, int6
         if (!X || !Y || !G) return PF_ERR_ARG;
         const Geo geo = make_geo(p->nx, p->ny, p->dx, p->x0, p->y0);
         const int nb = (int)std::min<int64_t>(ceil_div(s->nv0, 256), 1024);
-        for (double* a : {X, Y, G}) {
-            k_fill_nan<<<nb, 256, 0, p->stream>>>(a, s->nv0);
-            PF_LAUNCH_CHECK(p);
-        }
+        k_fill_nan<<<nb, 256, 0, p->stream>>>(X, Y, G, s->nv0);
+        PF_LAUNCH_CHECK(p);
         if (p->prec == PF_FP64)
             k_vic_get<double><<<geo.ntiles, 256, 0, p->stream>>>((const Rec<double>*)s->recs[s->cur], s->tstart[s->cur],
                                                                   s->tcount[s->cur], geo, X, Y, G, s->nv0);
