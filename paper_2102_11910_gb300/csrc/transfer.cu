@@ -201,6 +201,7 @@ pf_status regularize_direct(pf_plan p, const double* X, const double* Y, const d
 // E_v at n vortices from their positions, with a step's position update
 pf_status interpolate_direct(pf_plan p, const void* uv, const double* X, const double* Y, int64_t n, const int64_t* dn,
                              void* uq, void* vq, const AdvanceArgs& adv) {
+    if (n == 0) return PF_OK;
     if (p->prec == PF_FP64) return interpolate_direct_t<double>(p, uv, X, Y, n, dn, (double*)uq, (double*)vq, adv);
     return interpolate_direct_t<float>(p, uv, X, Y, n, dn, (float*)uq, (float*)vq, adv);
 }
