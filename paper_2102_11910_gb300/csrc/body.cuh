@@ -77,6 +77,7 @@ struct VortexSource {
     const int64_t* dn = nullptr;
     int64_t cap = 0;           // the most n or *dn can be
     int pairs = 0;
+    unsigned long long* oob = nullptr;   // with pairs: counts the vortices off the grid, as the R_v it replaces
 };
 // Steps take the vortex sum while ns x capacity is at most this: 2000 vortices
 // x 64 points cost 10 us, the FFT of a 768 x 512 field and the R_v it needs 75.

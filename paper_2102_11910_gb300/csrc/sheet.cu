@@ -57,6 +57,7 @@ struct VortexRhs {
     int ns, ne, chunks, place; // place: released positions from e, written to newx, newy; else read there
     EdgeGeo e;
     double *newx, *newy;
+    unsigned long long* oob;       // if not null: += the vortices off the grid
     double *part, *gpart, *unit;   // part[p * chunks + c], gpart[c], unit[j * ns + p]
 };
 
@@ -173,6 +174,11 @@ __global__ void __launch_bounds__(VR_THREADS) k_vortex_rhs(VortexRhs A, Geo geo,
                 if (axis == 0) s.g[v] = q < q1 ? A.G[q] : 0.0;
             }
             __syncthreads();
+            if (p == 0 && A.oob && tid < VR_ROUND && r0 + tid < q1 &&
+                (s.base[tid][0] >= 1 << 20 || s.base[tid][1] >= 1 << 20)) {
+                atomicAdd(A.oob, 1ull);
+                atomicOr(status, ST_OUT_OF_DOMAIN);
+            }
 #pragma unroll 1
             for (int v = tid >> 3; v < VR_ROUND; v += VR_THREADS / 8)
                 if (s.base[v][0] < 1 << 20 && s.base[v][1] < 1 << 20)
@@ -503,6 +509,7 @@ pf_status vortex_rhs(pf_plan p, pf_schur s, const VortexSource& vs, int ne, cons
     A.nv = vs.n;
     A.dn = vs.dn;
     A.pairs = vs.pairs;
+    A.oob = vs.oob;
     A.six = s->six;
     A.siy = s->siy;
     A.swx = s->swx;

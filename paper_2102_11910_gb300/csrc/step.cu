@@ -393,6 +393,7 @@ VortexSource vortex_source(pf_plan p, pf_state s, int ns, const double* X, const
     v.dn = c.dn;
     v.cap = s->cap;
     v.pairs = p->rhs_route == PF_RHS_AUTO && (int64_t)ns * s->cap <= VORTEX_PAIRS;
+    v.oob = p->d_oob;
     return v;
 }
 

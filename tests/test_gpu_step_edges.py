@@ -33,3 +33,24 @@ def test_a_step_without_vortices(prec, scheme, body):
     assert pf.pf_sync(plan) == 0
     X, _, _, t = pf.pf_state_get(state)
     assert len(X) == 0 and t == 0.01
+
+
+# capacities: the vortex sum with the one-launch transfers, the field's right-hand side with them (ns x
+# capacity past 2^19), the same with binned ones
+@pytest.mark.parametrize("prec", [pf.PF_FP64, pf.PF_MIXED])
+@pytest.mark.parametrize("multi", [False, True])
+@pytest.mark.parametrize("capacity", [256, 2048, 1 << 14, 1 << 17])
+def test_vortices_off_the_grid_are_counted_alike(prec, multi, capacity):
+    plan = _plan(prec)
+    rng = np.random.default_rng(8)
+    a = rng.uniform(0, 2 * np.pi, 130)
+    X, Y = 0.7 * np.cos(a), 0.7 * np.sin(a)
+    X[[3, 64, 129]], Y[70] = 5.0, -7.0                             # four of them
+    state = pf.State(plan, capacity)
+    pf.pf_state_set(state, X, Y, rng.normal(0.0, 0.02, 130), 0.0)
+    if multi:
+        pf.pf_step_multi(plan, state, 0.01, [_ellipse()], 1)
+    else:
+        pf.pf_step(plan, state, 0.01, _ellipse(), 1)
+    with pytest.raises(pf.GridPfError, match=" 16 points"):        # R_v twice in each of two stages
+        pf.pf_sync(plan)
