@@ -24,13 +24,13 @@ PF_MIXED = 1
 def _ptr(t, dtype=None, name="tensor"):
     if t is None:
         return None
+    if t.is_cuda and t.is_contiguous() and (dtype is None or t.dtype == dtype):
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError("%s must be a CUDA tensor" % name)
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
-    if dtype is not None and t.dtype != dtype:
-        raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
-    return ctypes.c_void_p(t.data_ptr())
+    raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
 
 
 class Plan:
