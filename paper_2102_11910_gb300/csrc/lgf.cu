@@ -25,42 +25,67 @@ constexpr int DE_STEPS_PER_UNIT = 64;
 constexpr double DE_S_MIN = -5.0;
 constexpr int DE_NODES = 532;   // s_k = -5 + k/64, k = 0..531
 
-__global__ void k_lgf_table(double* __restrict__ G, int nx, int ny, const double* __restrict__ node_t,
-                            const double* __restrict__ node_u, const double* __restrict__ node_c, int nn) {
+// One entry a thread, a warp a block (32 entries of a row): a warp's FP64
+// instruction holds its quarter of the SM for 64 clocks, so a small table has to
+// spread its few warps over all SMs (a plan of 8 x 8 nodes 1.1 ms, of 128^2 1.3;
+// with blocks of eight rows 1.8 and 2.0).  Bound by the FP64 pipe: exp and
+// sin are some 50 operations a quadrature node, at two lanes a clock and SM, and
+// most nodes need neither.  x = -2 M u falls along the nodes.  While |x| < 2^-54
+// (and the sine's argument N t/2 below it, as u = t/2 there), expm1(x) = x,
+// exp(x) = 1 and sin(N t/2) = N t/2 to the last bit; once x < -40, exp(x) < 2^-57 and the
+// numerator is 1 to the last bit.  G(m, n) = G(n, m) is formed once where the
+// table holds both.  The sums are the same, bitwise, as with every term in full.
+// Whole plan creation, with every term in full and so: 128^2 2.3 -> 1.3 ms,
+// 768 x 512 21 -> 7.0, 1024^2 51 -> 12, 2048 x 1800 176 -> 42.
+constexpr int LGF_TX = 32;
+constexpr double LGF_TINY = 0x1p-54, LGF_GONE = -40.0;
+
+__global__ void __launch_bounds__(LGF_TX) k_lgf_table(double* __restrict__ G, int nx, int ny,
+                                                      const double* __restrict__ node_t,
+                                                      const double* __restrict__ node_u,
+                                                      const double* __restrict__ node_c, int nn) {
+    const int m = blockIdx.x * LGF_TX + threadIdx.x, n = blockIdx.y;
+    if ((int)blockIdx.x * LGF_TX + LGF_TX - 1 < n && n <= nx) return;   // all of them mirrors
     extern __shared__ double sh[];
     double* st = sh;
     double* su = sh + nn;
     double* sc = sh + 2 * nn;
-    for (int k = threadIdx.x; k < nn; k += blockDim.x) {
+    for (int k = threadIdx.x; k < nn; k += LGF_TX) {
         st[k] = node_t[k];
         su[k] = node_u[k];
         sc[k] = node_c[k];
     }
     __syncthreads();
-    const int64_t total = (int64_t)(nx + 1) * (ny + 1);
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int m = (int)(e % (nx + 1));
-        const int n = (int)(e / (nx + 1));
-        const int M = m > n ? m : n;
-        const int N = m > n ? n : m;
-        double acc = 0.0;
-        if (M > 0) {
-            for (int k = 0; k < nn; ++k) {
-                const double x = -2.0 * M * su[k];
-                double ex, em1;
-                if (x > -0.5) {
-                    em1 = expm1(x);
-                    ex = 1.0 + em1;
-                } else {
-                    ex = exp(x);
-                    em1 = ex - 1.0;
-                }
-                const double sn = sin(0.5 * N * st[k]);
-                acc += sc[k] * (-em1 + ex * 2.0 * sn * sn);
-            }
+    if (m > nx || n > ny || (m < n && n <= nx)) return;
+    const int M = m > n ? m : n;
+    const int N = m > n ? n : m;
+    double acc = 0.0;
+    if (M > 0) {
+        int k = 0;
+        for (; k < nn; ++k) {
+            const double x = -2.0 * M * su[k];
+            if (!(x > -LGF_TINY)) break;
+            const double sn = 0.5 * N * st[k];
+            acc += sc[k] * (-x + 2.0 * sn * sn);
         }
-        G[e] = acc;
+        for (; k < nn; ++k) {
+            const double x = -2.0 * M * su[k];
+            if (x < LGF_GONE) break;
+            double ex, em1;
+            if (x > -0.5) {
+                em1 = expm1(x);
+                ex = 1.0 + em1;
+            } else {
+                ex = exp(x);
+                em1 = ex - 1.0;
+            }
+            const double sn = sin(0.5 * N * st[k]);
+            acc += sc[k] * (-em1 + ex * 2.0 * sn * sn);
+        }
+        for (; k < nn; ++k) acc += sc[k];
     }
+    G[(size_t)n * (nx + 1) + m] = acc;
+    if (n < m && m <= ny) G[(size_t)m * (nx + 1) + n] = acc;
 }
 
 __device__ __forceinline__ double lgf_at(const double* __restrict__ G, int nx, int m, int n) {
@@ -132,7 +157,8 @@ pf_status lgf_build(pf_plan p) {
     PF_CUDA(p, cudaMemcpyAsync(dn + DE_NODES, u.data(), DE_NODES * sizeof(double), cudaMemcpyHostToDevice, p->stream));
     PF_CUDA(p, cudaMemcpyAsync(dn + 2 * DE_NODES, c.data(), DE_NODES * sizeof(double), cudaMemcpyHostToDevice, p->stream));
     const size_t sh = 3 * DE_NODES * sizeof(double);
-    k_lgf_table<<<4 * 152, 256, sh, p->stream>>>(p->G, nx, ny, dn, dn + DE_NODES, dn + 2 * DE_NODES, DE_NODES);
+    const dim3 grid(ceil_div(nx + 1, LGF_TX), ny + 1);
+    k_lgf_table<<<grid, LGF_TX, sh, p->stream>>>(p->G, nx, ny, dn, dn + DE_NODES, dn + 2 * DE_NODES, DE_NODES);
     PF_LAUNCH_CHECK(p);
 
     double2* g = nullptr;
