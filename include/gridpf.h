@@ -88,7 +88,7 @@ pf_status pf_plan_fft_size(pf_plan plan, int32_t* P, int32_t* Q);
  *   PF_RHS_SPARSE  the direct sum over a list of the nonzero nodes built once
  *                  per solve (16 ns nnz multiply-adds);
  *   PF_RHS_AUTO    (default) in time stepping, while ns x capacity is at most
- *                  2^19 (capacity: the state's, so that a step's route does
+ *                  180000 + P Q / 10 (capacity: the state's, so that a step's route does
  *                  not change as vortices are shed), no field at all: the sum
  *                  from the vortices themselves, as pf_sheet_solve_vortices
  *                  forms it; otherwise the FFT when P, Q >= 256 and, for FP64

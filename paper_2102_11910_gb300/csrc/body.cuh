@@ -79,9 +79,13 @@ struct VortexSource {
     int pairs = 0;
     unsigned long long* oob = nullptr;   // with pairs: counts the vortices off the grid, as the R_v it replaces
 };
-// Steps take the vortex sum while ns x capacity is at most this: 2000 vortices
-// x 64 points cost 10 us, the FFT of a 768 x 512 field and the R_v it needs 75.
-constexpr int64_t VORTEX_PAIRS = (int64_t)1 << 19;
+// Steps take the vortex sum while ns x capacity is at most this.  The sum costs
+// 0.19 us a thousand pairs; the field's right-hand side (R_v and the 64-bit
+// streamfunction) 35 us and 20 more for every 2^20 nodes of the padded torus.
+// A stage by field and by sum just below the line: 256^2 96 and 95.7 us, 512^2
+// 114.3 and 112.1, 768 x 512 190.6 and 183.3, 1000^2 223 and 193; at 1.3 times
+// it 98 and 109, 115.7 and 131.2, 191.8 and 209.8, 222.7 and 231.2 (mixed).
+inline int64_t vortex_pairs_max(pf_plan p) { return 180000 + (int64_t)p->P * p->Q / 10; }
 
 // E_s L^-1 R_v Gamma into s->ewpart (vortex_rhs_chunks partial sums a
 // point), sums of Gamma into s->gpart (as many), E_s L^-1 d_j of ne released

@@ -392,7 +392,7 @@ VortexSource vortex_source(pf_plan p, pf_state s, int ns, const double* X, const
     v.n = c.n;
     v.dn = c.dn;
     v.cap = s->cap;
-    v.pairs = p->rhs_route == PF_RHS_AUTO && (int64_t)ns * s->cap <= VORTEX_PAIRS;
+    v.pairs = p->rhs_route == PF_RHS_AUTO && (int64_t)ns * s->cap <= vortex_pairs_max(p);
     v.oob = p->d_oob;
     return v;
 }

@@ -36,7 +36,7 @@ def test_a_step_without_vortices(prec, scheme, body):
 
 
 # capacities: the vortex sum with the one-launch transfers, the field's right-hand side with them (ns x
-# capacity past 2^19), the same with binned ones
+# capacity past the sum's limit), the same with binned ones
 @pytest.mark.parametrize("prec", [pf.PF_FP64, pf.PF_MIXED])
 @pytest.mark.parametrize("multi", [False, True])
 @pytest.mark.parametrize("capacity", [256, 2048, 1 << 14, 1 << 17])
