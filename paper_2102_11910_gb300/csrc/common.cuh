@@ -77,6 +77,11 @@ inline int bin_blocks(int64_t nv, int min_span = BIN_MIN_SPAN) {
     return nv > 0 ? (int)((nv + bin_span(nv, min_span) - 1) / bin_span(nv, min_span)) : 0;
 }
 
+// ints of the histograms of a binning pass of nv vortices: a row of tiles for each block
+inline int64_t bin_off_ints(int nx, int ny, int tile, int64_t nv, int min_span) {
+    return (int64_t)bin_blocks(nv, min_span) * ((nx + tile - 1) / tile) * ((ny + tile - 1) / tile);
+}
+
 // Partition of the one-pass binning (transfer.cuh), for sets of the mixed path
 // up to RUN_VORTICES: the blocks' span, 0 for sets that it does not take.
 constexpr int RUN_THREADS = 512;
@@ -311,6 +316,7 @@ pf_status regularize_direct(pf_plan p, const double* X, const double* Y, const d
                             const int64_t* dn, pf_schur_s* sch);
 pf_status interpolate_direct(pf_plan p, const void* uv, const double* X, const double* Y, int64_t n, const int64_t* dn,
                              void* uq, void* vq, const AdvanceArgs& adv);
-pf_status plan_reserve_vortices(pf_plan p, int64_t nv);   // transfer.cu: vortex buffers for nv ahead of time
+// transfer.cu: vortex buffers for a binning of nv vortices in tiles of `tile` nodes, min_span or more a block
+pf_status plan_reserve_vortices(pf_plan p, int64_t nv, int tile, int min_span);
 pf_status vortex_interpolate(pf_plan p, const void* uv, const double* X, const double* Y, int64_t nq, void* uq, void* vq);
 pf_status vortex_interpolate_located(pf_plan p, const void* uv, int64_t nq, void* uq, void* vq);

@@ -174,7 +174,7 @@ pf_status new_slot(pf_server s, int shape, int64_t cap, int ns, Slot** out) {
     if (e != cudaSuccess) st = e == cudaErrorMemoryAllocation ? PF_ERR_OOM : PF_ERR_CUDA;
     if (st == PF_OK) st = pf_plan_clone(h.base, s->cfg.precision, sl->stream, &sl->plan);
     if (st == PF_OK) st = pf_state_create(sl->plan, cap, &sl->state);
-    if (st == PF_OK) st = plan_reserve_vortices(sl->plan, cap);
+    if (st == PF_OK) st = plan_reserve_vortices(sl->plan, cap, sl->plan->tile, sl->plan->min_span);
     if (st != PF_OK) {
         destroy_slot(s, sl);
         return st;

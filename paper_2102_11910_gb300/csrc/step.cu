@@ -583,7 +583,7 @@ bool fixed_in_time(const pf_body_kinematics& k) { return k.ns == 0 || k.amp == 0
 // what a captured step of the full capacity needs ready: the vortex buffers,
 // the factor at the (fixed) pose and the buffers of the sheet's route
 pf_status prepare_capture(pf_plan p, pf_state s, const pf_body_kinematics& k) {
-    PF_TRY(plan_reserve_vortices(p, s->cap));
+    PF_TRY(plan_reserve_vortices(p, s->cap, p->tile, p->min_span));
     if (k.ns > 0) {
         PF_TRY(ensure_schur(p, s, surface_of(&k, 1, std::vector<Pose>{body_pose(k, s->t)})));
         PF_TRY(sheet_solve_reserve(p, s->fac[0].f, 16 * s->cap));

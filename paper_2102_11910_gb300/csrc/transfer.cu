@@ -29,7 +29,7 @@
 
 namespace {
 
-pf_status plan_bin_reserve(pf_plan p, int64_t nv) {
+pf_status plan_bin_reserve(pf_plan p, int64_t nv, int tile, int min_span) {
     const size_t psz = p->prec == PF_FP64 ? sizeof(Pos<double>) : sizeof(Pos<float>);
     const size_t rsz = p->prec == PF_FP64 ? sizeof(Rec<double>) : sizeof(Rec<float>);
     if (nv > (int64_t)1 << 29) {   // record slots are 32-bit
@@ -56,10 +56,9 @@ pf_status plan_bin_reserve(pf_plan p, int64_t nv) {
         PF_CUDA(p, cudaMalloc(&p->recs, (size_t)cap * rsz));
         p->rec_cap = cap;
     }
-    const int64_t ntiles = (int64_t)ceil_div(p->nx, p->tile) * ceil_div(p->ny, p->tile);
-    const int64_t need = (int64_t)bin_blocks(nv, p->min_span) * ntiles;
+    const int64_t need = bin_off_ints(p->nx, p->ny, tile, nv, min_span);
     if (need > p->bin_off_cap) {
-        const int64_t cap = std::max<int64_t>(need, (int64_t)bin_blocks(p->pos_cap, p->min_span) * ntiles);
+        const int64_t cap = std::max<int64_t>(need, bin_off_ints(p->nx, p->ny, tile, p->pos_cap, min_span));
         PF_CUDA(p, cudaStreamSynchronize(p->stream));
         if (p->bin_off) cudaFree(p->bin_off);
         p->bin_off = nullptr;
@@ -78,6 +77,7 @@ BinWork plan_binwork(pf_plan p) {
     b.gmax = p->gmax;
     b.tile_start = p->tile_start;
     b.bin_off = p->bin_off;
+    b.off_cap = p->bin_off_cap;
     b.pos = p->pos;
     b.recs = p->recs;
     b.rec_cap = p->rec_cap;
@@ -94,6 +94,7 @@ template <int TILE>
 pf_status regularize_runs(pf_plan p, const Geo& geo, const BinWork& bw, const double* X, const double* Y, const double* G,
                           int64_t nv, float* w, const int64_t* dn) {
     const int span = p->bin_span;
+    if ((int64_t)p->bin_runs * geo.ntiles > bw.off_cap) return PF_ERR_INTERNAL;
     const size_t sm = (size_t)span * sizeof(Pos<float>) + (size_t)geo.ntiles * sizeof(unsigned);
     PF_CUDA(p, set_smem(k_bin_runs<TILE>, sm));
     PF_KERNEL(p, "bin_runs", PF_CUDA(p, pf_launch(k_bin_runs<TILE>, p->bin_runs, RUN_THREADS, sm, p->stream, X, Y, G, nv,
@@ -179,8 +180,9 @@ pf_status interpolate_tiles(pf_plan p, const Geo& geo, const void* uv, int64_t n
 // the plan's binning scratch (cell records, histograms, status words)
 BinWork plan_binwork_for(pf_plan p) { return plan_binwork(p); }
 
-// size the plan's vortex buffers for nv vortices ahead of time
-pf_status plan_reserve_vortices(pf_plan p, int64_t nv) { return plan_bin_reserve(p, nv); }
+pf_status plan_reserve_vortices(pf_plan p, int64_t nv, int tile, int min_span) {
+    return plan_bin_reserve(p, nv, tile, min_span);
+}
 
 bool vortices_direct(pf_plan p, int64_t n) { return plan_direct(p, n); }
 
@@ -213,7 +215,7 @@ pf_status interpolate_direct(pf_plan p, const void* uv, const double* X, const d
 pf_status vortex_regularize(pf_plan p, const double* X, const double* Y, const double* G, int64_t nv, void* w,
                             const int64_t* dn, void* zu, void* zv) {
     if (!zu && plan_direct(p, nv)) return regularize_direct(p, X, Y, G, nv, w, dn, nullptr);
-    pf_status st = plan_bin_reserve(p, nv);
+    pf_status st = plan_bin_reserve(p, nv, p->tile, p->min_span);
     if (st != PF_OK) return st;
     BinWork bw = plan_binwork(p);
     bw.zu = zu;
@@ -305,6 +307,7 @@ BinWork noalloc_binwork(unsigned char* base) {
     b.tile_start = (int*)(t + NOALLOC_MAX_TILES);
     b.gmax = (double*)(t + 2 * NOALLOC_MAX_TILES);
     b.bin_off = (int*)(base + NOALLOC_HEADER + NOALLOC_TILE_BYTES);
+    b.off_cap = (int64_t)NOALLOC_MAX_BLOCKS * NOALLOC_MAX_TILES;
     b.pos = base + NOALLOC_HEADER + NOALLOC_TILE_BYTES + NOALLOC_OFF_BYTES;
     b.recs = base + NOALLOC_HEADER + NOALLOC_TILE_BYTES + NOALLOC_OFF_BYTES + NOALLOC_POS_BYTES;
     b.rec_cap = 4 * NOALLOC_MAX_VORTICES;

@@ -1551,7 +1551,8 @@ struct BinWork {
     unsigned* tile_count;     // written by k_offsets
     double* gmax;             // [0]: largest |Gamma| (k_offsets); [1 + b]: that of locate block b
     int* tile_start;
-    int* bin_off;             // bin_blocks(nv) * ntiles
+    int* bin_off;             // a histogram row of ntiles a block
+    int64_t off_cap;          // ints in bin_off
     void* pos;
     void* recs;
     int64_t rec_cap;          // record slots in recs
@@ -1584,6 +1585,10 @@ pf_status bin_launch_nt(pf_plan p, const Geo& geo, const BinWork& bw, const doub
     const int nb = bin_blocks(nv, min_span);
     const int64_t span = bin_span(nv, min_span);
     const int mb = bin_max_blocks(nv);
+    if ((int64_t)nb * geo.ntiles > bw.off_cap) {
+        if (p) snprintf(p->err, sizeof(p->err), "binning of %lld vortices: histograms reserved for fewer blocks", (long long)nv);
+        return PF_ERR_INTERNAL;
+    }
     const size_t sh_loc = (size_t)geo.ntiles * sizeof(unsigned);
     const size_t sh_sc = 2 * (size_t)geo.ntiles * sizeof(unsigned);
     if (set_smem(k_locate<T, TILE, NT>, sh_loc) != cudaSuccess || set_smem(k_scatter<T, TILE, NT>, sh_sc) != cudaSuccess)

@@ -542,7 +542,8 @@ pf_status pf_vic_state_destroy(pf_vic_state s) {
 pf_status pf_vic_state_set(pf_vic_state s, const double* X, const double* Y, const double* G, int64_t nv) {
     if (!s || nv < 0 || nv > s->cap || (nv > 0 && (!X || !Y || !G))) return PF_ERR_ARG;
     pf_plan p = s->plan;
-    PF_TRY(plan_reserve_vortices(p, nv));        // the plan's per-vortex cell records and histograms
+    // the plan's cell records and histograms, for the binning below: in a state's own tiles and partition, whatever the plan's
+    PF_TRY(plan_reserve_vortices(p, nv, BIN_TILE, BIN_MIN_SPAN));
     BinWork bw = plan_binwork_for(p);
     bw.recs = s->recs[0];
     bw.rec_cap = s->rec_cap;
