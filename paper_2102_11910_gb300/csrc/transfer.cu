@@ -241,8 +241,10 @@ pf_status vortex_interpolate(pf_plan p, const void* uv, const double* X, const d
                                                                                (double*)vq, p->d_status, p->d_oob));
     } else {
         const int nb = (int)std::min<int64_t>(ceil_div(nq, XY_THREADS), 152 * 16);
-        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(k_interp_xy_f32, nb, XY_THREADS, 0, p->stream, (const float2*)uv, X, Y,
-                                                         nq, geo, (float*)uq, (float*)vq, p->d_status, p->d_oob)));
+        const bool pairs = (uintptr_t)uv % sizeof(float2) == 0;
+        PF_KERNEL(p, "interpolate", PF_CUDA(p, pf_launch(pairs ? k_interp_xy_f32<true> : k_interp_xy_f32<false>, nb, XY_THREADS,
+                                                         0, p->stream, (const float*)uv, X, Y, nq, geo, (float*)uq, (float*)vq,
+                                                         p->d_status, p->d_oob)));
     }
     return PF_OK;
 }

@@ -1428,7 +1428,13 @@ struct XyPoint {
     float u, v;
     int pad;
 };
-__global__ void __launch_bounds__(XY_THREADS) k_interp_xy_f32(const float2* __restrict__ uv, const double* __restrict__ X,
+// PAIRS: uv lies on 8-byte boundaries and a node is one load; a caller's field that starts on an odd word is read by words.
+template <bool PAIRS> __device__ __forceinline__ float2 load_node(const float* __restrict__ p) {
+    if constexpr (PAIRS) return __ldg(reinterpret_cast<const float2*>(p));
+    else return make_float2(__ldg(p), __ldg(p + 1));
+}
+template <bool PAIRS>
+__global__ void __launch_bounds__(XY_THREADS) k_interp_xy_f32(const float* __restrict__ uv, const double* __restrict__ X,
                                                               const double* __restrict__ Y, int64_t nq, Geo geo,
                                                               float* __restrict__ uq, float* __restrict__ vq,
                                                               int* __restrict__ status, unsigned long long* __restrict__ oob) {
@@ -1461,9 +1467,9 @@ __global__ void __launch_bounds__(XY_THREADS) k_interp_xy_f32(const float2* __re
             const int at = p.at;
             float2 a = make_float2(0.f, 0.f), b = a;
             if (at >= 0) {
-                const float2* r = uv + at + 2 * pair * geo.nx + col;
-                a = __ldg(r);
-                b = __ldg(r + geo.nx);
+                const float* r = uv + 2 * ((size_t)at + 2 * pair * geo.nx + col);
+                a = load_node<PAIRS>(r);
+                b = load_node<PAIRS>(r + 2 * geo.nx);
             }
             const float2 w = *reinterpret_cast<const float2*>(p.wy + 2 * pair);
             const float wx = p.wx[col];
