@@ -329,7 +329,11 @@ pf_status pf_poisson_solve(pf_plan p, const void* w, void* psi) {
 
 pf_status pf_velocity_solve(pf_plan p, const void* w, double Uinf, double Vinf, void* uv) {
     if (!p || !w || !uv) return PF_ERR_ARG;
-    return conv_solve(p, w, uv, CONV_UV, Uinf, Vinf);
+    // the passes write a node's (u, v) in one store: a field that starts off such a pair's boundary is copied out
+    if ((uintptr_t)uv % (2 * p->esz) == 0) return conv_solve(p, w, uv, CONV_UV, Uinf, Vinf);
+    PF_TRY(conv_solve(p, w, p->uv, CONV_UV, Uinf, Vinf));
+    PF_CUDA(p, cudaMemcpyAsync(uv, p->uv, 2 * (size_t)p->nx * p->ny * p->esz, cudaMemcpyDeviceToDevice, p->stream));
+    return PF_OK;
 }
 
 pf_status pf_interpolate(pf_plan p, const void* uv, const double* Xq, const double* Yq, int64_t nq, void* uq, void* vq) {
