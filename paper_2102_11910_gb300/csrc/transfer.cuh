@@ -1145,10 +1145,11 @@ __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int c
 // record whose cell lies in the tile (each vortex has exactly one such record)
 // gathers its 4x4 stencil there and writes its result at its original index.
 //
-// FP64: the patch is held in fixed point below 2^58 of its largest value, as
-// centred halves (16 bytes a node, as the doubles), and the forty products of
-// a record are integer multiply-adds (1e6 vortices on 1024^2: 227 -> 67 us); a
-// patch with an infinity or a NaN keeps its doubles and the FP64 sums.
+// FP64: the patch is held in fixed point, each component below 2^58 of its own
+// largest value (a stream along x leaves v its digits), as centred halves (16
+// bytes a node, as the doubles), and the forty products of a record are integer
+// multiply-adds (1e6 vortices on 1024^2: 227 -> 67 us); a patch with an infinity
+// or a NaN keeps its doubles and the FP64 sums.
 template <int TILE>
 __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __restrict__ recs, FlatBins bins,
                                                           const double2* __restrict__ uv, Geo geo,
@@ -1156,9 +1157,9 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
                                                           int* __restrict__ status) {
     constexpr int PATCH = TILE + 3;
     __shared__ int4 patch[PATCH * PATCH];
-    __shared__ int top;
+    __shared__ int top[2];
     const int t = blockIdx.x;
-    if (threadIdx.x == 0) top = 1;
+    if (threadIdx.x < 2) top[threadIdx.x] = 1;
     pdl_wait();
     double unused;
     const auto src = open_tile<false>(bins, recs, t, status, unused);
@@ -1167,24 +1168,30 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
     const int tx = t % geo.ntx, ty = t / geo.ntx;
     const int gi0 = tx * TILE - 1, gj0 = ty * TILE - 1;
     double2* patchd = reinterpret_cast<double2*>(patch);
-    int ef = 1;
+    int eu = 1, ev = 1;
     for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {
         const int gi = gi0 + i % PATCH, gj = gj0 + i / PATCH;
         double2 v = make_double2(0.0, 0.0);
         if (gi >= 0 && gi < geo.nx && gj >= 0 && gj < geo.ny) v = uv[(size_t)gj * geo.nx + gi];
         patchd[i] = v;
-        ef = max(ef, max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF));
+        eu = max(eu, (__double2hiint(v.x) >> 20) & 0x7FF);
+        ev = max(ev, (__double2hiint(v.y) >> 20) & 0x7FF);
     }
     __syncthreads();                                  // top is initialised
-    ef = __reduce_max_sync(0xffffffffu, ef);
-    if ((threadIdx.x & 31) == 0) atomicMax(&top, ef);
+    eu = __reduce_max_sync(0xffffffffu, eu);
+    ev = __reduce_max_sync(0xffffffffu, ev);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&top[0], eu);
+        atomicMax(&top[1], ev);
+    }
     __syncthreads();
-    const int emax = top;
-    const bool finite = emax < 2047;                  // block-uniform
+    eu = top[0];
+    ev = top[1];
+    const bool finite = max(eu, ev) < 2047;           // block-uniform
     if (finite) {
         for (int i = threadIdx.x; i < PATCH * PATCH; i += blockDim.x) {       // each thread its own nodes, in place
             const double2 v = patchd[i];
-            const FxSplit a = fx_split(fx_from_double(v.x, emax)), b = fx_split(fx_from_double(v.y, emax));
+            const FxSplit a = fx_split(fx_from_double(v.x, eu)), b = fx_split(fx_from_double(v.y, ev));
             patch[i] = make_int4(a.h, a.l, b.h, b.l);
         }
         __syncthreads();
@@ -1222,8 +1229,8 @@ __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __r
                     su += fx_weigh(fx_split((hu << 1) + (tu >> 30)), wy[b]);
                     sv += fx_weigh(fx_split((hv << 1) + (tv >> 30)), wy[b]);
                 }
-                ou = fx_to_double(su, fx_exp(emax));
-                ov = fx_to_double(sv, fx_exp(emax));
+                ou = fx_to_double(su, fx_exp(eu));
+                ov = fx_to_double(sv, fx_exp(ev));
             } else {
                 double wx[4], wy[4];
                 m4p_weights(c.fx, wx);
