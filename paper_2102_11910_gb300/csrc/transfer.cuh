@@ -252,11 +252,16 @@ __device__ __forceinline__ bool split_rec(double X, const Geo& g, int axis, int&
 __device__ __forceinline__ bool split_rec(double X, const Geo& g, int axis, int& c, double& f) { return loc_split(X, g, axis, c, f); }
 template <typename T> using Frac = typename std::conditional<sizeof(T) == 4, unsigned, double>::type;
 
-// max(m, |g|), a NaN ignored; the doubles compared as integers
-__device__ __forceinline__ float abs_max(float m, float g) { return fmaxf(m, fabsf(g)); }
+// max(m, |g|), compared as integers, so that a NaN is above all; NaNs as infinities
+__device__ __forceinline__ float abs_max(float m, float g) {
+    return __int_as_float(max(__float_as_int(m), __float_as_int(g) & 0x7FFFFFFF));
+}
 __device__ __forceinline__ double abs_max(double m, double g) {
-    const long long a = __double_as_longlong(g) & 0x7FFFFFFFFFFFFFFFll;
-    return a <= 0x7FF0000000000000ll && a > __double_as_longlong(m) ? __longlong_as_double(a) : m;
+    return __longlong_as_double(max(__double_as_longlong(m), __double_as_longlong(g) & 0x7FFFFFFFFFFFFFFFll));
+}
+__device__ __forceinline__ float no_nan(float m) { return m <= INFINITY ? m : INFINITY; }
+__device__ __forceinline__ double no_nan(double m) {
+    return __longlong_as_double(min(__double_as_longlong(m), 0x7FF0000000000000ll));
 }
 
 // The vortex count and block span of a binning pass: the launch's own, or,
@@ -336,6 +341,7 @@ __global__ void __launch_bounds__(NT) k_locate(const double* __restrict__ X, con
         atomicAdd(oob, (unsigned long long)bad);
         atomicOr(status, ST_OUT_OF_DOMAIN);
     }
+    gm = no_nan(gm);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
     if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = gm;
@@ -616,6 +622,7 @@ __global__ void __launch_bounds__(RUN_THREADS) k_bin_runs(const double* __restri
         atomicOr(status, ST_OUT_OF_DOMAIN);
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    gm = no_nan(gm);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
     if (lane == 0) wmax[wid] = gm;
@@ -683,7 +690,9 @@ __device__ __forceinline__ void split_hilo(float x, int& hi, int& lo) {
 // 64-bit add.  Integer sums are exact, so the result does not depend on the
 // order of the adds.  The scale bounds every node sum by the tile's record
 // count times the largest |Gamma| of the whole regularization (reduced by
-// k_offsets from the locate blocks' maxima).  (A one-add variant with a
+// k_offsets from the locate blocks' maxima).  If that is not finite, each tile
+// looks through its records (tile_gmax): one that holds such a strength becomes NaN,
+// the others go by their own largest.  (A one-add variant with a
 // node-window bound measured no faster and lost seven bits on clustered
 // vortices; shared adds are not what bounds this kernel.)
 //
@@ -704,8 +713,7 @@ enum { DEP_SPLIT32 = 0, DEP_F32_64 = 1 };
 // us with FP64 products and 64-bit adds, 53 us.
 template <int ACC_W>
 __device__ __forceinline__ void deposit_one_fx(const Rec<double>& rc, int gexp, int drop, unsigned* acc_lo,
-                                               unsigned* acc_hi, int* bad) {
-    if (((__double2hiint(rc.g) >> 20) & 0x7FF) == 0x7FF) *bad = 1;      // not finite: the tile becomes NaN
+                                               unsigned* acc_hi) {
     FxSplit wx[4], wy[4];
     fx_m4p(rc.fx, wx);
     fx_m4p(rc.fy, wy);
@@ -934,12 +942,33 @@ struct DepositSmem {
     unsigned long long acc[AccW<TILE>::value * AccW<TILE>::value];
     Rec<T> srt[SORT && sizeof(T) == 4 ? DEP_SORT_SLOTS : 1];
     int bcnt[32], bstart[32];
+    unsigned long long top;    // tile_gmax: the largest finite |Gamma|'s bits, and whether there are others
+    int bad;
 };
 
 template <typename T, int TILE, bool SORT>
 __device__ __forceinline__ void deposit_clear(DepositSmem<T, TILE, SORT>& sm) {
     for (int i = threadIdx.x; i < AccW<TILE>::value * AccW<TILE>::value; i += blockDim.x) sm.acc[i] = 0ull;
     if (threadIdx.x < 32) sm.bcnt[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        sm.top = 0ull;
+        sm.bad = 0;
+    }
+}
+
+// the tile's largest finite |Gamma|; sm.bad is set if one of its strengths is not finite
+template <typename T, int TILE, bool SORT, typename SRC>
+__device__ __noinline__ double tile_gmax(const SRC src, DepositSmem<T, TILE, SORT>& sm) {
+    __syncthreads();
+    for (int r0 = 0; r0 < src.cnt; r0 += (int)blockDim.x) {
+        Rec<T> rc[1];
+        src.load(r0, rc);
+        const double g = fabs((double)rc[0].g);
+        if (g < INFINITY) atomicMax(&sm.top, (unsigned long long)__double_as_longlong(g));
+        else sm.bad = 1;
+    }
+    __syncthreads();
+    return __longlong_as_double((long long)sm.top);
 }
 
 // w of tile (tx, ty) from its records (global or shared memory); rc holds
@@ -950,7 +979,7 @@ __device__ __forceinline__ void deposit_tile(const SRC& src, double gmax, const 
     constexpr int ACC_W = AccW<TILE>::value;
     const int cnt = src.cnt;
     unsigned long long* acc = sm.acc;
-    int* bstart = sm.bstart;
+    if (__double2hiint(gmax) == 0x7FF00000) gmax = tile_gmax<T, TILE, SORT, SRC>(src, sm);     // an infinity; block-uniform
     if constexpr (sizeof(T) == 8) {
         // terms below 2^58 come drop bits finer than the sums, which stay below 2^63
         const int gf = (int)(__double_as_longlong(gmax) >> 52) & 0x7FF, gexp = gf ? gf : 1;
@@ -958,19 +987,17 @@ __device__ __forceinline__ void deposit_tile(const SRC& src, double gmax, const 
         const int sh = -(fx_exp(gexp) + drop);
         unsigned* acc_lo = reinterpret_cast<unsigned*>(acc);
         unsigned* acc_hi = acc_lo + ACC_W * ACC_W;
-        if (threadIdx.x == 0) bstart[0] = 0;                      // set by a record that is not finite
         __syncthreads();
-        deposit_records<T>(src, rc,
-                           [&](const Rec<T>& r) { deposit_one_fx<ACC_W>(r, gexp, drop, acc_lo, acc_hi, &bstart[0]); });
+        deposit_records<T>(src, rc, [&](const Rec<T>& r) { deposit_one_fx<ACC_W>(r, gexp, drop, acc_lo, acc_hi); });
         __syncthreads();
+        const double inv_dx2 = sm.bad ? (double)NAN : geo.inv_dx2;
         for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
             const int lx = i % TILE, ly = i / TILE;
             const int gi = tx * TILE + lx, gj = ty * TILE + ly;
             const int node = (ly + ACC_HALO) * ACC_W + lx + ACC_HALO;
             if (gi < geo.nx && gj < geo.ny) {
                 const long long a = (long long)(((unsigned long long)acc_hi[node] << 32) | acc_lo[node]);
-                w[(size_t)gj * geo.nx + gi] = bstart[0] ? __longlong_as_double(0x7FF8000000000000ll)
-                                                        : fx_to_double(a, -sh) * geo.inv_dx2;
+                w[(size_t)gj * geo.nx + gi] = fx_to_double(a, -sh) * inv_dx2;
             }
         }
     } else {
@@ -979,7 +1006,7 @@ __device__ __forceinline__ void deposit_tile(const SRC& src, double gmax, const 
         const T scale = pow2<T>(sh);
         __syncthreads();
         if (SORT && split32 && cnt >= DEP_SORT_MIN)             // block-uniform
-            deposit_records_banked<ACC_W, T>(src, scale, acc, rc, sm.srt, sm.bcnt, bstart);
+            deposit_records_banked<ACC_W, T>(src, scale, acc, rc, sm.srt, sm.bcnt, sm.bstart);
         else if (split32)
             deposit_records<T>(src, rc,
                                [&](const Rec<T>& r) { deposit_one<DEP_SPLIT32, ACC_W, T>(r, scale, acc); });
@@ -989,7 +1016,7 @@ __device__ __forceinline__ void deposit_tile(const SRC& src, double gmax, const 
         __syncthreads();
         const int* acc_hi = reinterpret_cast<const int*>(acc);
         const int* acc_lo = reinterpret_cast<const int*>(acc) + ACC_W * ACC_W;
-        const float inv_dx2f = (float)geo.inv_dx2;
+        const float inv_dx2f = sm.bad ? NAN : (float)geo.inv_dx2;
         for (int i = threadIdx.x; i < TILE * TILE; i += blockDim.x) {
             const int lx = i % TILE, ly = i / TILE;
             const int gi = tx * TILE + lx, gj = ty * TILE + ly;
@@ -1092,6 +1119,7 @@ __global__ void __launch_bounds__(256) k_deposit_direct(const double* __restrict
         atomicAdd(oob, (unsigned long long)bad);
         atomicOr(status, ST_OUT_OF_DOMAIN);
     }
+    gm = no_nan(gm);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
     if (lane == 0) wmax[wid] = gm;
