@@ -310,18 +310,6 @@ __global__ void k_extract_inverse(const double* __restrict__ A, double* __restri
 constexpr int BGJ_B = 32;              // panel width
 constexpr int BGJ_MAX = 1024;          // ns handled by one panel block (panel rows in shared memory)
 
-// 1 / p within an ulp (Newton's iteration in its cubic form, r (1 + e + e^2)
-// with e = 1 - p r, from the hardware's 20-bit estimate: 2^-60 and one
-// rounding); p normal and away from the ends of the range, else a division
-__device__ __forceinline__ double fast_recip(double p) {
-    const int ef = (__double2hiint(p) >> 20) & 0x7FF;
-    if (ef < 64 || ef > 1982) return 1.0 / p;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
-    const double e = fma(-p, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // One block of (n - k0) / ROWS warps, at least eight.  Pivot rows by partial
 // pivoting on an FP32 copy of the panel held in registers (warp w has rows w, w
 // + nw, .., a lane a column): each warp offers its largest |entry| of column c

@@ -46,6 +46,21 @@ struct pf_schur_s {
 };
 constexpr int EW_SPLIT_MAX = 16;
 
+// 1 / p within one unit in the last place of the division
+// (tests/host/recip_check.cu): one step of the hyperpower (Schulz) iteration of order three,
+// r (1 + e + e^2) with e = 1 - p r, from the hardware's 20-bit estimate r: e^3
+// is about 2^-60, and one rounding; p normal and away from the ends of the
+// range, else the division itself.  (Three dependent FP64 instructions of 64
+// clocks; it stands in the serial chain of k_bgj_panel.)
+__device__ __forceinline__ double fast_recip(double p) {
+    const int ef = (__double2hiint(p) >> 20) & 0x7FF;
+    if (ef < 64 || ef > 1982) return 1.0 / p;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+    const double e = fma(-p, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 pf_status schur_create(pf_plan p, int ns, pf_schur* out);
 void schur_free(pf_schur s);
 pf_status schur_factor_device(pf_plan p, pf_schur s);
