@@ -1178,29 +1178,21 @@ void schur_free(pf_schur s) {
     delete s;
 }
 
-// Full sheet solve on device.  psi_w: real field; vx, vy: device positions of
-// the new vortices (mode KUTTA_SHED).  Results: f (device, ns) and scal[0..2] =
-// (s0, Gamma1, Gamma2) on the device.
 // E_s L^-1 w into ew (ns doubles): the FP64 sum with the LGF, over all nodes
 // or over a list of the nonzero ones, or a 64-bit FFT solve psi = -L^-1 w
 // (fixfft.cu) read at the stencils.
-// Route from the field w (no vortex source): the sparse sum when the caller
-// bounds the nonzero nodes and the sum is small (below 2^24 multiply-adds its
-// few blocks finish sooner than an FFT's passes), else the FFT solve where the
-// padded torus allows it, else the direct sum.  The sums run on the FP64 pipe
-// (two multiply-adds a clock and SM), the FFT on the integer pipe, so an FP64
-// plan keeps the direct sum only below ns nx ny = 2^18, where it takes about
-// as long as the FFT's three launches (128^2: 72 us at ns 64, 2^20, against 25).
+// The automatic route from the field w: the FFT solve where the padded torus
+// allows it, else the direct sum.  The sums run on the FP64 pipe (two
+// multiply-adds a clock and SM), the FFT on the integer pipe, so an FP64 plan
+// keeps the direct sum only below ns nx ny = 2^18, where it takes about as long
+// as the FFT's three launches (128^2: 72 us at ns 64, 2^20, against 25).
 enum FieldRoute { ROUTE_SPARSE, ROUTE_DIRECT, ROUTE_FFT };
 
-FieldRoute field_route(pf_plan p, int ns, int64_t nnz_bound) {
+FieldRoute field_route(pf_plan p, int ns) {
     const int64_t M = (int64_t)p->nx * p->ny;
     const bool fft_ok = p->P >= 256 && p->Q >= 256;
     const bool mixed = p->prec != PF_FP64;
-    const int64_t sparse_max = (int64_t)1 << 24;
-    if (p->rhs_route == PF_RHS_SPARSE ||
-        (p->rhs_route == PF_RHS_AUTO && nnz_bound >= 0 && 16 * (int64_t)ns * nnz_bound < sparse_max))
-        return ROUTE_SPARSE;
+    if (p->rhs_route == PF_RHS_SPARSE) return ROUTE_SPARSE;
     if (fft_ok && (p->rhs_route == PF_RHS_FFT ||
                    (p->rhs_route == PF_RHS_AUTO && (mixed || (int64_t)ns * M > ((int64_t)1 << 18)))))
         return ROUTE_FFT;
@@ -1226,11 +1218,11 @@ pf_status field_route_buffers(pf_plan p, FieldRoute r) {
     return PF_OK;
 }
 
-pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew, int64_t nnz_bound) {
+pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew) {
     const int ns = s->ns;
     cudaStream_t st = p->stream;
     const int64_t M = (int64_t)p->nx * p->ny;
-    const FieldRoute route = field_route(p, ns, nnz_bound);
+    const FieldRoute route = field_route(p, ns);
     PF_TRY(field_route_buffers(p, route));
     if (route == ROUTE_SPARSE) {
         int* counts = p->nz_idx + M;
@@ -1282,8 +1274,8 @@ pf_status surface_rhs(pf_plan p, pf_schur s, const void* w, double* ew, int64_t 
 
 // allocate ahead of time what a sheet solve with this nonzero bound would
 // allocate on first use (a step captured for replay may not allocate)
-pf_status sheet_solve_reserve(pf_plan p, pf_schur s, int64_t nnz_bound) {
-    return field_route_buffers(p, field_route(p, s->ns, nnz_bound));
+pf_status sheet_solve_reserve(pf_plan p, pf_schur s, int64_t cap) {
+    return vortices_summed(p, s->ns, cap) ? PF_OK : field_route_buffers(p, field_route(p, s->ns));
 }
 
 // Several bodies (Sec. 2.7, Eq. kuttasystem4), one block of 256.  y holds
@@ -1379,7 +1371,7 @@ __global__ void __launch_bounds__(256) k_constraints_multi(int ns, pf_multibody 
 // Gamma1, Gamma2) on the device.
 pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_motion& m, int mode, double param,
                              const double* param_dev, int n_edges, const int* edges, double* vx, double* vy, double* f,
-                             const EdgeBounds& eb, int64_t nnz_bound, const SheetStep& step) {
+                             const EdgeBounds& eb, const SheetStep& step) {
     const int ns = s->ns;
     cudaStream_t st = p->stream;
     double* sb = s->work;
@@ -1391,7 +1383,7 @@ pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_moti
     const int ne = mode == PF_SHEET_KUTTA_SHED ? n_edges : 0, nc = 1 + ne;
     if (step.vs || ne > 0)
         PF_TRY(vortex_rhs(p, s, step.vs ? *step.vs : VortexSource(), ne, step.place, vx, vy, rhs + ns));
-    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew, nnz_bound));
+    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew));
     const double* part = pairs ? s->ewpart : ew;
     const int chunks = pairs ? vortex_rhs_chunks(ns, step.vs->cap) : 1;
     const int k1 = n_edges > 0 ? edges[0] : 0, k2 = n_edges > 1 ? edges[1] : 0;
@@ -1708,7 +1700,7 @@ double* multibody_newpos(pf_schur s) { return s->mwork + (2 + 3 * (size_t)MB_COL
 
 pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const pf_multibody& mb, int ne,
                                    double* vx, double* vy, double* f, const double* gw_dev,
-                                   double** out_dev, int64_t nnz_bound, const VortexSource* vs) {
+                                   double** out_dev, const VortexSource* vs) {
     const int nb = mb.n_bodies, ns = s->ns, nc = 1 + ne + nb;
     cudaStream_t st = p->stream;
     PF_TRY(multibody_scratch(p, s));
@@ -1722,7 +1714,7 @@ pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const p
     PF_LAUNCH_CHECK(p);
     const bool pairs = vs && vs->pairs;
     if (pairs || ne > 0) PF_TRY(vortex_rhs(p, s, pairs ? *vs : VortexSource(), ne, nullptr, vx, vy, rhs + ns));
-    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew, nnz_bound));
+    if (!pairs) PF_TRY(surface_rhs(p, s, w, ew));
     k_rhs0<<<1, 256, 0, st>>>(PF_SHEET_KUTTA_SHED, ns, 0.0, nullptr, sb, pairs ? s->ewpart : ew,
                               pairs ? vortex_rhs_chunks(ns, vs->cap) : 1, s->f0hat, s->dgamma0, rhs);
     k_indicators<<<dim3(ceil_div(ns, 256), nb), 256, 0, st>>>(ns, mb, rhs + (size_t)(1 + ne) * ns);
@@ -1850,8 +1842,7 @@ pf_status pf_sheet_solve_vortices(pf_plan p, pf_schur s, const double* X, const 
     vs.pairs = 1;
     SheetStep step;
     step.vs = &vs;
-    pf_status st = sheet_solve_device(p, s, nullptr, *m, mode, param, nullptr, n_edges, edges, vxy, vxy + 2, f, EdgeBounds(), -1,
-                                      step);
+    pf_status st = sheet_solve_device(p, s, nullptr, *m, mode, param, nullptr, n_edges, edges, vxy, vxy + 2, f, EdgeBounds(), step);
     if (st != PF_OK) return st;
     double sc[3];
     PF_CUDA(p, cudaMemcpyAsync(sc, s->scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, p->stream));

@@ -100,7 +100,11 @@ struct VortexSource {
 // A stage by field and by sum just below the line: 256^2 96 and 95.7 us, 512^2
 // 114.3 and 112.1, 768 x 512 190.6 and 183.3, 1000^2 223 and 193; at 1.3 times
 // it 98 and 109, 115.7 and 131.2, 191.8 and 209.8, 222.7 and 231.2 (mixed).
-inline int64_t vortex_pairs_max(pf_plan p) { return 180000 + (int64_t)p->P * p->Q / 10; }
+inline int64_t vortex_pairs_max(int P, int Q) { return 180000 + (int64_t)P * Q / 10; }
+// (a rule on the state's capacity: a captured step takes the route of the step it stands for)
+inline bool vortices_summed(pf_plan p, int ns, int64_t cap) {
+    return p->rhs_route == PF_RHS_AUTO && (int64_t)ns * cap <= vortex_pairs_max(p->P, p->Q);
+}
 
 // E_s L^-1 R_v Gamma into s->ewpart (vortex_rhs_chunks partial sums a
 // point), sums of Gamma into s->gpart (as many), E_s L^-1 d_j of ne released
@@ -111,7 +115,7 @@ pf_status vortex_rhs(pf_plan p, pf_schur s, const VortexSource& vs, int ne, cons
                      double* unit);                                                               // sheet.cu
 pf_status sheet_solve_multi_device(pf_plan p, pf_schur s, const void* w, const pf_multibody& mb, int ne,
                                    double* vx, double* vy, double* f, const double* gw_dev,
-                                   double** out_dev, int64_t nnz_bound = -1, const VortexSource* vs = nullptr);
+                                   double** out_dev, const VortexSource* vs = nullptr);
 // Generalized edge condition (Sec. 2.5) for the shedding mode: with on = 0 every
 // edge sheds under the Kutta condition; otherwise edge e sheds only when its
 // intermediate value lies outside [lo[e], hi[e]], and ends at the bound crossed.
@@ -165,17 +169,14 @@ struct SheetStep {
     Release rel;
     bool nodes = false;
 };
-// param_dev (nullable): device copy of `param` read by the kernels instead;
-// nnz_bound >= 0: at most that many nodes of w are nonzero (lets the surface
-// right-hand side take the sparse route), -1: unknown
+// param_dev (nullable): device copy of `param` read by the kernels instead
 pf_status sheet_solve_device(pf_plan p, pf_schur s, const void* w, const pf_motion& m, int mode, double param,
                              const double* param_dev, int n_edges, const int* edges, double* vx, double* vy, double* f,
-                             const EdgeBounds& eb = EdgeBounds(), int64_t nnz_bound = -1,
-                             const SheetStep& step = SheetStep());
+                             const EdgeBounds& eb = EdgeBounds(), const SheetStep& step = SheetStep());
 // w += R_s f  (device f of ns doubles, w real[nx*ny])
 pf_status sheet_deposit(pf_plan p, pf_schur s, const double* f, void* w);
-// allocate what a sheet solve with this nonzero bound allocates on first use
-pf_status sheet_solve_reserve(pf_plan p, pf_schur s, int64_t nnz_bound);
+// allocate what the sheet solves of steps of a state of this capacity allocate on first use
+pf_status sheet_solve_reserve(pf_plan p, pf_schur s, int64_t cap);
 
 // step.cu: asynchronous state transfers used by the request server
 pf_status state_load_async(pf_state s, const double* X, const double* Y, const double* G, int64_t nv, double t);

@@ -91,12 +91,11 @@ int64_t slot_bytes(const Shape& s, int prec, int64_t cap, int ns) {
     // two Schur factors (a moving body keeps the last two poses), each S, the
     // ns x 2 ns Gauss-Jordan workspace, S^-1, and O(ns) vectors and orderings
     const int64_t schur = 2 * ((int64_t)ns * ns * 8 * 4 + (int64_t)ns * 328);
-    // FP64 buffers of the FFT route of the surface right-hand side (mixed plans)
-    const int64_t M = (int64_t)s.nx * s.ny;
+    // 64-bit streamfunction and spectra of the surface right-hand side where it
+    // comes from the field (mixed plans)
     const int Q = 1 << (32 - __builtin_clz(2 * s.ny - 1));
-    const bool fft = P >= 256 && Q >= 256 && (int64_t)ns * M > ((int64_t)1 << 22);
-    const int64_t rhs = ((fft && prec != PF_FP64) ? 2 * M * 8 + 2 * (int64_t)ldK * ldT * 16 : 0) +
-                        M * 12;    // node list of the sparse route
+    const bool field = prec != PF_FP64 && P >= 256 && Q >= 256 && (int64_t)ns * cap > vortex_pairs_max(P, Q);
+    const int64_t rhs = field ? (int64_t)s.nx * s.ny * 8 + 2 * (int64_t)ldK * ldT * 16 : 0;
     return grid + bins + state + schur + rhs;
 }
 

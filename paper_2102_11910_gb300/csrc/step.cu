@@ -392,7 +392,7 @@ VortexSource vortex_source(pf_plan p, pf_state s, int ns, const double* X, const
     v.n = c.n;
     v.dn = c.dn;
     v.cap = s->cap;
-    v.pairs = p->rhs_route == PF_RHS_AUTO && (int64_t)ns * s->cap <= vortex_pairs_max(p);
+    v.pairs = vortices_summed(p, ns, s->cap);
     v.oob = p->d_oob;
     return v;
 }
@@ -447,7 +447,7 @@ pf_status body_stage(pf_plan p, pf_state s, const pf_body_kinematics& k, double 
                 PF_LAUNCH_CHECK(p);
             }
             PF_TRY(sheet_solve_device(p, sch, p->w, m, PF_SHEET_KUTTA_SHED, 0.0, s->red, 2, kk, s->newpos,
-                                      s->newpos + MAX_EDGES, s->f, eb, 16 * s->cap, step));
+                                      s->newpos + MAX_EDGES, s->f, eb, step));
             if (!small) {
                 k_append<<<1, 32, 0, p->stream>>>(const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->newpos,
                                                   sch->scal + 1, 2, s->dn, c.dn != nullptr, s->cap, p->d_status);
@@ -457,7 +457,7 @@ pf_status body_stage(pf_plan p, pf_state s, const pf_body_kinematics& k, double 
         } else {
             if (small) step.gsign = -1.0;
             PF_TRY(sheet_solve_device(p, sch, p->w, m, PF_SHEET_CIRCULATION, 0.0, s->red + 1, 0, nullptr, nullptr,
-                                      nullptr, s->f, EdgeBounds(), 16 * s->cap, step));
+                                      nullptr, s->f, EdgeBounds(), step));
         }
     }
     PhaseSpan ph(p, "phase_velocity");
@@ -500,8 +500,7 @@ pf_status bodies_stage(pf_plan p, pf_state s, const pf_body_kinematics* k, int n
     if (ne > 0) k_place<<<1, 32, 0, p->stream>>>(X, Y, e, c.dn, s->newpos);
     PF_LAUNCH_CHECK(p);
     double* out = nullptr;
-    PF_TRY(sheet_solve_multi_device(p, sch, p->w, mb, ne, s->newpos, s->newpos + MAX_EDGES, s->f, gw, &out,
-                                    16 * s->cap, &vs));
+    PF_TRY(sheet_solve_multi_device(p, sch, p->w, mb, ne, s->newpos, s->newpos + MAX_EDGES, s->f, gw, &out, &vs));
     if (ne > 0) {
         k_append<<<1, 32, 0, p->stream>>>(const_cast<double*>(X), const_cast<double*>(Y), s->G, c.n, s->newpos,
                                           out + nb, ne, s->dn, c.dn != nullptr, s->cap, p->d_status);
@@ -586,7 +585,7 @@ pf_status prepare_capture(pf_plan p, pf_state s, const pf_body_kinematics& k) {
     PF_TRY(plan_reserve_vortices(p, s->cap, p->tile, p->min_span));
     if (k.ns > 0) {
         PF_TRY(ensure_schur(p, s, surface_of(&k, 1, std::vector<Pose>{body_pose(k, s->t)})));
-        PF_TRY(sheet_solve_reserve(p, s->fac[0].f, 16 * s->cap));
+        PF_TRY(sheet_solve_reserve(p, s->fac[0].f, s->cap));
     }
     return PF_OK;
 }
