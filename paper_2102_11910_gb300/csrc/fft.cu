@@ -180,19 +180,13 @@ __device__ __forceinline__ size_t spec_at(int j, int k, int nk) {
 }
 
 // Two consecutive rows j, j + 1 (j even) of a half spectrum are adjacent in
-// this layout: one 16-byte access in FP32, two in FP64.
-template <typename C>
-__device__ __forceinline__ void ld_pair(const C* p, C& a, C& b) { a = p[0]; b = p[1]; }
-template <>
-__device__ __forceinline__ void ld_pair<float2>(const float2* p, float2& a, float2& b) {
+// this layout: one 16-byte access.
+__device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     a = make_float2(q.x, q.y);
     b = make_float2(q.z, q.w);
 }
-template <typename C>
-__device__ __forceinline__ void st_pair(C* p, C a, C b) { p[0] = a; p[1] = b; }
-template <>
-__device__ __forceinline__ void st_pair<float2>(float2* p, float2 a, float2 b) {
+__device__ __forceinline__ void st_pair(float2* p, float2 a, float2 b) {
     *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
 }
 
@@ -207,43 +201,42 @@ constexpr int FWD_GROUPS = 2;
 // two, a tenth more with four; at 1024^2 all three the same, 9.2).
 constexpr int INV_GROUPS = 2;
 
-template <typename T, int R3>
-__global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const T* __restrict__ w,
-                                                                                C_t<T>* __restrict__ T1, int nx,
-                                                                                int ny, const C_t<T>* __restrict__ tw) {
-    using C = C_t<T>;
+template <int R3>
+__global__ void __launch_bounds__(16 * R3 * FWD_GROUPS) k_rows_fwd_r(const float* __restrict__ w,
+                                                                                float2* __restrict__ T1, int nx,
+                                                                                int ny, const float2* __restrict__ tw) {
     constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = FWD_GROUPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* bufs = reinterpret_cast<C*>(smem_raw);
+    float2* bufs = reinterpret_cast<float2*>(smem_raw);
     const int g = threadIdx.x / TP, t = threadIdx.x % TP;
-    C* buf = bufs + g * SB;
+    float2* buf = bufs + g * SB;
     const int r0 = 2 * G * blockIdx.x;          // the block's first row (even)
     const int j0 = r0 + 2 * g;
     const bool h0 = j0 < ny, h1 = j0 + 1 < ny;
     pdl_wait();
-    C v[16];
+    float2 v[16];
     const int ja = h0 ? j0 : ny - 1, jb = h1 ? j0 + 1 : ny - 1;     // clamped rows: loads never branch
 #pragma unroll
     for (int r = 0; r < 16; ++r) {                   // n >= P / 2 >= nx: padding
-        v[r] = cmake<C>(T(0), T(0));
+        v[r] = make_float2(0.f, 0.f);
         if (r >= 8) continue;
         const int n = t + TP * r;
         const int nc = n < nx ? n : nx - 1;
-        const T a = w[(size_t)ja * nx + nc], b = w[(size_t)jb * nx + nc];
-        v[r] = cmake<C>(n < nx && h0 ? a : T(0), n < nx && h1 ? b : T(0));
+        const float a = w[(size_t)ja * nx + nc], b = w[(size_t)jb * nx + nc];
+        v[r] = make_float2(n < nx && h0 ? a : 0.f, n < nx && h1 ? b : 0.f);
     }
-    fft_strided<C, false, R3>(v, buf, t, tw);
+    fft_strided<float2, false, R3>(v, buf, t, tw);
 #pragma unroll
     for (int r = 0; r < 16; ++r) buf[spad(t + TP * r)] = v[r];
     __syncthreads();
     // per k, the half spectra of the rows j0, j0 + 1 of each group are adjacent
     // (rows past ny get the zero spectrum of their zero input)
-    C* dst = T1 + (size_t)(r0 >> 2) * NK * 4 + (r0 & 3);
+    float2* dst = T1 + (size_t)(r0 >> 2) * NK * 4 + (r0 & 3);
     for (int e = threadIdx.x; e < NK * G; e += blockDim.x) {
         const int k = e / G, gg = e % G;
-        const C* bz = bufs + gg * SB;
-        const C z1 = bz[spad(k)], z2 = conjc(bz[spad((P - k) & (P - 1))]);
-        st_pair(dst + 4 * k + 2 * gg, (z1 + z2) * T(0.5), mul_mi(z1 - z2) * T(0.5));
+        const float2* bz = bufs + gg * SB;
+        const float2 z1 = bz[spad(k)], z2 = conjc(bz[spad((P - k) & (P - 1))]);
+        st_pair(dst + 4 * k + 2 * gg, (z1 + z2) * 0.5f, mul_mi(z1 - z2) * 0.5f);
     }
 }
 
@@ -258,40 +251,39 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 // hold the twiddles of all three transforms; loading them again in each (96
 // registers, five blocks an SM instead of four) measured 18.3 us against 16.0 at
 // 1024^2, 80 registers and six blocks 21.7, 168 and three 18.6.
-template <typename T, int R3>
-__global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 1) k_cols_r(
-    const C_t<T>* __restrict__ T1, C_t<T>* __restrict__ T2a, C_t<T>* __restrict__ T2b, int ny, int nk, int mode,
-    const T* __restrict__ H, const T* __restrict__ Hu, const T* __restrict__ Hv, int Hld,
-    const C_t<T>* __restrict__ tw) {
-    using C = C_t<T>;
+template <int R3>
+__global__ void __launch_bounds__(16 * R3, R3 > 1 ? 32 / R3 : 1) k_cols_r(
+    const float2* __restrict__ T1, float2* __restrict__ T2a, float2* __restrict__ T2b, int ny, int nk, int mode,
+    const float* __restrict__ H, const float* __restrict__ Hu, const float* __restrict__ Hv, int Hld,
+    const float2* __restrict__ tw) {
     constexpr int Q = 256 * R3, TQ = Q / 16, SB = SBuf<Q>::size;
-    constexpr int NH = (Q / 2 + 1 + 3) / 4 * 4, PER = 16 / sizeof(T);   // spectrum row length, elements per copy
+    constexpr int NH = (Q / 2 + 1 + 3) / 4 * 4, PER = 16 / sizeof(float);   // spectrum row length, elements per copy
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);
-    C* keep = buf + SB;
-    T* hs0 = reinterpret_cast<T*>(keep + SB);
-    T* hs1 = hs0 + NH;
+    float2* buf = reinterpret_cast<float2*>(smem_raw);
+    float2* keep = buf + SB;
+    float* hs0 = reinterpret_cast<float*>(keep + SB);
+    float* hs1 = hs0 + NH;
     const int k = blockIdx.x, t = threadIdx.x;
     const size_t row = (size_t)k * Hld;
     pdl_wait();
     {
-        const T* s0 = mode == CONV_UV ? Hu : H;
+        const float* s0 = mode == CONV_UV ? Hu : H;
         for (int i = PER * t; i < NH; i += PER * TQ) {
             cp_async16(hs0 + i, s0 + row + i);
             if (mode == CONV_UV) cp_async16(hs1 + i, Hv + row + i);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    C v[16];
+    float2 v[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {            // clamped row: loads never branch; l >= Q / 2 >= ny: padding
-        v[r] = cmake<C>(T(0), T(0));
+        v[r] = make_float2(0.f, 0.f);
         if (r >= 8) continue;
         const int l = t + TQ * r;
-        const C x = T1[spec_at(l < ny ? l : ny - 1, k, nk)];
+        const float2 x = T1[spec_at(l < ny ? l : ny - 1, k, nk)];
         if (l < ny) v[r] = x;
     }
-    fft_strided<C, false, R3>(v, buf, t, tw);
+    fft_strided<float2, false, R3>(v, buf, t, tw);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (mode == CONV_UV) {
@@ -300,19 +292,19 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
             const int l = t + TQ * r;
             const bool lo = l <= Q / 2;
             const int lq = lo ? l : Q - l;
-            const C iw = mul_i(v[r]);
-            const T hu = hs0[lq];
+            const float2 iw = mul_i(v[r]);
+            const float hu = hs0[lq];
             keep[spad(l)] = iw * hs1[lq];          // even in l
             v[r] = iw * (lo ? hu : -hu);            // odd in l
         }
-        fft_strided<C, true, R3>(v, buf, t, tw);
+        fft_strided<float2, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 16; ++r) {               // rows past Q / 2 are not kept
             const int l = t + TQ * r;
             if (r < 8 && l < ny) T2a[spec_at(l, k, nk)] = v[r];
             v[r] = keep[spad(l)];                    // written by this thread
         }
-        fft_strided<C, true, R3>(v, buf, t, tw);
+        fft_strided<float2, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
@@ -324,7 +316,7 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
             const int l = t + TQ * r;
             v[r] = v[r] * hs0[l <= Q / 2 ? l : Q - l];
         }
-        fft_strided<C, true, R3>(v, buf, t, tw);
+        fft_strided<float2, true, R3>(v, buf, t, tw);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int l = t + TQ * r;
@@ -337,14 +329,13 @@ __global__ void __launch_bounds__(16 * R3, sizeof(T) == 4 && R3 > 1 ? 32 / R3 : 
 // row, half spectra from T2a and T2b) or psi_j + i psi_{j+1} (two rows of
 // T2a).  Two rows' values of a k come as one 16-byte load.  At most 64
 // registers a thread: 1024 threads an SM.
-template <typename T, int R3>
-__global__ void __launch_bounds__(16 * R3 * INV_GROUPS, sizeof(T) == 4 && R3 >= 4 ? 1024 / (16 * R3 * INV_GROUPS) : 1)
-    k_rows_inv_r(const C_t<T>* __restrict__ T2a, const C_t<T>* __restrict__ T2b, T* __restrict__ out, int nx, int ny,
-                 int mode, T Uinf, T Vinf, const C_t<T>* __restrict__ tw) {
-    using C = C_t<T>;
+template <int R3>
+__global__ void __launch_bounds__(16 * R3 * INV_GROUPS, R3 >= 4 ? 1024 / (16 * R3 * INV_GROUPS) : 1)
+    k_rows_inv_r(const float2* __restrict__ T2a, const float2* __restrict__ T2b, float* __restrict__ out, int nx, int ny,
+                 int mode, float Uinf, float Vinf, const float2* __restrict__ tw) {
     constexpr int P = 256 * R3, TP = P / 16, SB = SBuf<P>::size, NK = P / 2 + 1, G = INV_GROUPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* bufs = reinterpret_cast<C*>(smem_raw);
+    float2* bufs = reinterpret_cast<float2*>(smem_raw);
     const int g = threadIdx.x / TP, t = threadIdx.x % TP;
     const bool uv = mode == CONV_UV;
     const int rows = uv ? G : 2 * G;                 // rows of the block
@@ -353,47 +344,47 @@ __global__ void __launch_bounds__(16 * R3 * INV_GROUPS, sizeof(T) == 4 && R3 >= 
     pdl_wait();
 #pragma unroll 2
     for (int k = threadIdx.x; k <= h; k += blockDim.x) {
-        C a[G], b[G];
+        float2 a[G], b[G];
         if (uv) {                                     // group gg takes row r0 + gg
             const size_t at = spec_at(r0, k, NK);       // r0 is even
             ld_pair(T2a + at, a[0], a[1]);
             ld_pair(T2b + at, b[0], b[1]);
 #pragma unroll
             for (int gg = 0; gg < G; ++gg)
-                if (r0 + gg >= ny) a[gg] = b[gg] = cmake<C>(T(0), T(0));
+                if (r0 + gg >= ny) a[gg] = b[gg] = make_float2(0.f, 0.f);
         } else {                                      // group gg takes rows r0 + 2 gg, r0 + 2 gg + 1
 #pragma unroll
             for (int gg = 0; gg < G; ++gg) {
                 const int j = r0 + 2 * gg;
                 ld_pair(T2a + spec_at(j < ny ? j : r0, k, NK), a[gg], b[gg]);
-                if (j >= ny) a[gg] = cmake<C>(T(0), T(0));
-                if (j + 1 >= ny) b[gg] = cmake<C>(T(0), T(0));
+                if (j >= ny) a[gg] = make_float2(0.f, 0.f);
+                if (j + 1 >= ny) b[gg] = make_float2(0.f, 0.f);
             }
         }
 #pragma unroll
         for (int gg = 0; gg < G; ++gg) {
-            C x = a[gg], y = b[gg];
+            float2 x = a[gg], y = b[gg];
             if (k == 0 || k == h) { x.y = 0; y.y = 0; }
-            C* buf = bufs + gg * SB;
+            float2* buf = bufs + gg * SB;
             buf[spad(k)] = x + mul_i(y);
             if (k > 0 && k < h) buf[spad(P - k)] = conjc(x) + mul_i(conjc(y));
         }
     }
     __syncthreads();
-    C* buf = bufs + g * SB;
-    C v[16];
+    float2* buf = bufs + g * SB;
+    float2 v[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = buf[spad(t + TP * r)];
     __syncthreads();
-    fft_strided<C, true, R3>(v, buf, t, tw);
+    fft_strided<float2, true, R3>(v, buf, t, tw);
     if (uv) {
         const int j = r0 + g;
         if (j < ny) {
-            C* o = reinterpret_cast<C*>(out) + (size_t)j * nx;
+            float2* o = reinterpret_cast<float2*>(out) + (size_t)j * nx;
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 const int n = t + TP * r;
-                if (n < nx) o[n] = cmake<C>(v[r].x + Uinf, v[r].y + Vinf);
+                if (n < nx) o[n] = make_float2(v[r].x + Uinf, v[r].y + Vinf);
             }
         }
     } else {
@@ -416,53 +407,51 @@ struct ConvWs {
     void* T2b;
 };
 
-template <typename T, int R3P, int R3Q>
-static pf_status conv_solve_r(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                              const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
-    using C = C_t<T>;
+template <int R3P, int R3Q>
+static pf_status conv_solve_r(pf_plan p, const float* w, float* out, int mode, float Uinf, float Vinf, const float* H, const float* Hu,
+                              const float* Hv, const float2* twP, const float2* twQ, ConvWs ws) {
     constexpr int P = 256 * R3P, Q = 256 * R3Q;
     const int nx = p->nx, ny = p->ny;
-    const size_t sf = FWD_GROUPS * (size_t)SBuf<P>::size * sizeof(C);
-    const size_t sc = 2 * (size_t)SBuf<Q>::size * sizeof(C) + 2 * (size_t)((Q / 2 + 1 + 3) / 4 * 4) * sizeof(T);
-    PF_CUDA(p, set_smem(k_rows_fwd_r<T, R3P>, sf));
-    PF_CUDA(p, set_smem(k_cols_r<T, R3Q>, sc));
-    C* T1 = reinterpret_cast<C*>(ws.T1);
-    C* T2a = reinterpret_cast<C*>(ws.T2a);
-    C* T2b = reinterpret_cast<C*>(ws.T2b);
-    PF_KERNEL(p, "fft_rows_fwd", PF_CUDA(p, pf_launch(k_rows_fwd_r<T, R3P>, ceil_div(ny, 2 * FWD_GROUPS), 16 * R3P * FWD_GROUPS, sf, p->stream, w, T1,
+    const size_t sf = FWD_GROUPS * (size_t)SBuf<P>::size * sizeof(float2);
+    const size_t sc = 2 * (size_t)SBuf<Q>::size * sizeof(float2) + 2 * (size_t)((Q / 2 + 1 + 3) / 4 * 4) * sizeof(float);
+    PF_CUDA(p, set_smem(k_rows_fwd_r<R3P>, sf));
+    PF_CUDA(p, set_smem(k_cols_r<R3Q>, sc));
+    float2* T1 = reinterpret_cast<float2*>(ws.T1);
+    float2* T2a = reinterpret_cast<float2*>(ws.T2a);
+    float2* T2b = reinterpret_cast<float2*>(ws.T2b);
+    PF_KERNEL(p, "fft_rows_fwd", PF_CUDA(p, pf_launch(k_rows_fwd_r<R3P>, ceil_div(ny, 2 * FWD_GROUPS), 16 * R3P * FWD_GROUPS, sf, p->stream, w, T1,
                                                       nx, ny, twP)));
-    PF_KERNEL(p, "fft_cols_conv", PF_CUDA(p, pf_launch(k_cols_r<T, R3Q>, P / 2 + 1, 16 * R3Q, sc, p->stream, T1, T2a,
+    PF_KERNEL(p, "fft_cols_conv", PF_CUDA(p, pf_launch(k_cols_r<R3Q>, P / 2 + 1, 16 * R3Q, sc, p->stream, T1, T2a,
                                                        T2b, ny, P / 2 + 1, mode, H, Hu, Hv, p->Hld, twQ)));
     const int nb = mode == CONV_UV ? ceil_div(ny, INV_GROUPS) : ceil_div(ny, 2 * INV_GROUPS);
-    const size_t sr = INV_GROUPS * (size_t)SBuf<P>::size * sizeof(C);
-    PF_CUDA(p, set_smem(k_rows_inv_r<T, R3P>, sr));
-    PF_KERNEL(p, "fft_rows_inv", PF_CUDA(p, pf_launch(k_rows_inv_r<T, R3P>, nb, 16 * R3P * INV_GROUPS, sr, p->stream, T2a, T2b,
+    const size_t sr = INV_GROUPS * (size_t)SBuf<P>::size * sizeof(float2);
+    PF_CUDA(p, set_smem(k_rows_inv_r<R3P>, sr));
+    PF_KERNEL(p, "fft_rows_inv", PF_CUDA(p, pf_launch(k_rows_inv_r<R3P>, nb, 16 * R3P * INV_GROUPS, sr, p->stream, T2a, T2b,
                                                       out, nx, ny, mode, Uinf, Vinf, twP)));
     return PF_OK;
 }
 
-template <typename T, int R3P>
-static pf_status conv_dispatch_q(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                                 const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
+template <int R3P>
+static pf_status conv_dispatch_q(pf_plan p, const float* w, float* out, int mode, float Uinf, float Vinf, const float* H, const float* Hu,
+                                 const float* Hv, const float2* twP, const float2* twQ, ConvWs ws) {
     switch (p->Q) {
-        case 256: return conv_solve_r<T, R3P, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 512: return conv_solve_r<T, R3P, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 1024: return conv_solve_r<T, R3P, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 2048: return conv_solve_r<T, R3P, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 4096: return conv_solve_r<T, R3P, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 256: return conv_solve_r<R3P, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 512: return conv_solve_r<R3P, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 1024: return conv_solve_r<R3P, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 2048: return conv_solve_r<R3P, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 4096: return conv_solve_r<R3P, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
     }
     return PF_ERR_ARG;
 }
 
-template <typename T>
-static pf_status conv_dispatch(pf_plan p, const T* w, T* out, int mode, T Uinf, T Vinf, const T* H, const T* Hu,
-                               const T* Hv, const C_t<T>* twP, const C_t<T>* twQ, ConvWs ws) {
+static pf_status conv_dispatch(pf_plan p, const float* w, float* out, int mode, float Uinf, float Vinf, const float* H, const float* Hu,
+                               const float* Hv, const float2* twP, const float2* twQ, ConvWs ws) {
     switch (p->P) {
-        case 256: return conv_dispatch_q<T, 1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 512: return conv_dispatch_q<T, 2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 1024: return conv_dispatch_q<T, 4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 2048: return conv_dispatch_q<T, 8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
-        case 4096: return conv_dispatch_q<T, 16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 256: return conv_dispatch_q<1>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 512: return conv_dispatch_q<2>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 1024: return conv_dispatch_q<4>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 2048: return conv_dispatch_q<8>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
+        case 4096: return conv_dispatch_q<16>(p, w, out, mode, Uinf, Vinf, H, Hu, Hv, twP, twQ, ws);
     }
     return PF_ERR_ARG;
 }
@@ -498,7 +487,7 @@ pf_status conv_solve(pf_plan p, const void* w, void* out, int mode, double Uinf,
                                     p->twP64, p->twQ64, ws);
     }
     if (reg)
-        return conv_dispatch<float>(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
+        return conv_dispatch(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
                                     p->Hv32, p->twP32_r, p->twQ32_r, ws);
     return conv_solve_t<float>(p, (const float*)w, (float*)out, mode, (float)Uinf, (float)Vinf, p->H32, p->Hu32,
                                p->Hv32, p->twP32, p->twQ32, ws);

@@ -23,7 +23,6 @@
 
 template <typename C> struct real_of;
 template <> struct real_of<float2> { using type = float; };
-template <> struct real_of<double2> { using type = double; };
 
 // cos(2 pi m / 16) for a compile-time m
 template <int M>
