@@ -134,10 +134,11 @@ pf_status pf_timing_report(pf_plan plan, char* buf, int64_t buflen);
  *   tile_threads  threads per tile block of the deposit (and of E_v in FP64
  *                 plans; mixed plans' E_v always runs 256): 128 or 256.
  *                 Results are bitwise the same for both.
- *   fft           0: register-resident radix-16 Stockham passes (grids whose
- *                 padded torus is at least 256 x 256; smaller ones always take
- *                 the shared-memory passes); 1: shared-memory passes.  Results
- *                 differ by rounding.
+ *   fft           0: Stockham passes in registers, radix 16 in FP32 for mixed
+ *                 plans, radix 8 in 64-bit block fixed point for FP64 plans
+ *                 (grids whose padded torus is at least 256 x 256; smaller ones
+ *                 always take the shared-memory passes); 1: shared-memory passes
+ *                 in the plan's precision.  Results differ by rounding.
  * A new plan has {32, 1024, 256, 0}; clones copy their source's. */
 typedef struct {
     int32_t tile;

@@ -315,8 +315,11 @@ constexpr int BGJ_MAX = 1024;          // ns handled by one panel block (panel r
 // + nw, .., a lane a column): each warp offers its largest |entry| of column c
 // (to 2^-18: the low bits of the key hold the row) with the whole row it sits
 // in, so that after one block barrier every warp knows the pivot and has its
-// row.  Then the FP64 LU of the permuted pivot block, four rows a warp in eight
-// warps: the warp that owns row c + 1 updates it first, forms its pivot's
+// row.  (The copy, its short keys and its approximate division choose the rows'
+// order, nothing else.  With u / pv there a pitching plate's step of two stages
+// takes 289 us instead of 277, and its error against 64 bits is the same,
+// 2.8e-8.)  Then the FP64 LU of the permuted pivot block, four rows a warp in
+// eight warps: the warp that owns row c + 1 updates it first, forms its pivot's
 // reciprocal and publishes the scaled row, the others meanwhile update theirs,
 // one barrier a step.  The kernel runs on one SM and is two chains of 32 steps:
 // reductions and a barrier (about 500 clocks), and six dependent FP64

@@ -99,7 +99,10 @@ struct VortexSource {
 // streamfunction) 35 us and 20 more for every 2^20 nodes of the padded torus.
 // A stage by field and by sum just below the line: 256^2 96 and 95.7 us, 512^2
 // 114.3 and 112.1, 768 x 512 190.6 and 183.3, 1000^2 223 and 193; at 1.3 times
-// it 98 and 109, 115.7 and 131.2, 191.8 and 209.8, 222.7 and 231.2 (mixed).
+// it 98 and 109, 115.7 and 131.2, 191.8 and 209.8, 222.7 and 231.2 (mixed).  On
+// larger grids the sum is the faster one at the line in either precision: 1024^2
+// 241 and 198 (FP64 447 and 392), 1500 x 1024 386 and 302 (778 and 680), 2048 x
+// 1800 749 and 512 (1582 and 1319), and by up to 18 % at 1.3 times the line still.
 inline int64_t vortex_pairs_max(int P, int Q) { return 180000 + (int64_t)P * Q / 10; }
 // (a rule on the state's capacity: a captured step takes the route of the step it stands for)
 inline bool vortices_summed(pf_plan p, int ns, int64_t cap) {

@@ -139,7 +139,7 @@ struct pf_plan_s {
     void* uv = nullptr;            // 2*nx*ny real
     // launch configuration of the transfer and Poisson passes (pf_launch_config_set,
     // pf_autotune): tile edge, fewest vortices per binning block, threads per
-    // tile block, FFT kernels (0 register-resident radix-16, 1 shared-memory)
+    // tile block, FFT kernels (0 in registers: FP32 radix 16, FP64 block fixed point; 1 shared-memory)
     int tile = BIN_TILE;
     int min_span = BIN_MIN_SPAN;
     int tile_threads = 256;

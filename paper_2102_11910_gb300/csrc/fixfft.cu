@@ -16,7 +16,9 @@
 // 28 us, columns 417 -> 134 us, inverse rows 157 -> 45 us; streamfunction of
 // 512 x 384: 120 -> 44 us; and against double-float passes on the FP32 pipe
 // (48 bits) for the surface right-hand side of 768 x 512: 102 -> 66 us.  The
-// error against FP64 sums is that of the FP64 passes or below.
+// error is below that of the FP64 passes: against transforms in 80 bits, five grids of
+// 128^2 to 1024^2 and three random fields each, psi 1.3e-16 to 4.3e-15 of its norm
+// (FP64 passes 2.2e-16 to 6.9e-15, larger in each case), u and v 1.4 to 2.3e-16 (3.0 to 5.1e-16).
 //
 // A thread holds eight points (radix 8, T = N / 8 threads a transform), and
 // every kernel has one copy of the transform's code, its passes and its

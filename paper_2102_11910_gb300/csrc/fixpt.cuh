@@ -126,7 +126,7 @@ __device__ __forceinline__ double fx_to_double(long long x, int e) {
     const long long s = x >> 63;
     unsigned long long a = (unsigned long long)((x ^ s) - s);
     if (a == 0) return 0.0;
-    const int sh = __clzll((long long)a) - 1;             // |x| < 2^62: to [2^62, 2^63)
+    const int sh = __clzll((long long)a) - 1;             // |x| < 2^63: to [2^62, 2^63)
     a <<= sh;
     const int ef = e - sh + 62 + 1023;
     if (ef < 1 || ef > 2045) return ldexp((double)x, e);

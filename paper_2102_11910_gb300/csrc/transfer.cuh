@@ -1176,8 +1176,9 @@ __device__ __forceinline__ void gather16(const T* __restrict__ uv, int nx, int c
 // FP64: the patch is held in fixed point, each component below 2^58 of its own
 // largest value (a stream along x leaves v its digits), as centred halves (16
 // bytes a node, as the doubles), and the forty products of a record are integer
-// multiply-adds (1e6 vortices on 1024^2: 227 -> 67 us); a patch with an infinity
-// or a NaN keeps its doubles and the FP64 sums.
+// multiply-adds (1e6 vortices on 1024^2: 227 -> 70 us, of which the second
+// exponent is 3); a patch with an infinity or a NaN keeps its doubles and the FP64
+// sums.
 template <int TILE>
 __global__ void __launch_bounds__(256) k_interp_tiles_f64(const Rec<double>* __restrict__ recs, FlatBins bins,
                                                           const double2* __restrict__ uv, Geo geo,
@@ -1455,7 +1456,7 @@ __global__ void __launch_bounds__(256) k_interp_xy_f64(const double* __restrict_
 // time, gather one half row of the stencil each.  The pass is bound by the L1
 // lookups of its scattered loads, one a distinct line and instruction: a
 // thread a point makes 16 a point, half rows 8 (200,003 points on 768 x 512:
-// 12.8 -> XY8 us).
+// 16.6 -> 12.3 us between events).
 constexpr int XY_THREADS = 128;
 struct XyPoint {
     float wx[4], wy[4];
