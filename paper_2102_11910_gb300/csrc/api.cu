@@ -26,6 +26,7 @@ void free_plan(pf_plan p) {
                    p->d_status, p->d_oob, p->fx_exp};
     for (void* q : own)
         if (q) cudaFree(q);
+    for (void* q : p->retired) cudaFree(q);
     if (p->pscr) cudaFree(p->pscr);
     if (p->centres) {
         free_plan(p->centres);

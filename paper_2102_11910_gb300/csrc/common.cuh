@@ -154,6 +154,8 @@ struct pf_plan_s {
     int* tile_start = nullptr;
     int* bin_off = nullptr;            // per (block, tile): histogram, then first record slot
     int64_t bin_off_cap = 0;           // entries
+    bool captured = false;             // a captured step holds the addresses of the binning buffers:
+    std::vector<void*> retired;        // outgrown ones are kept here until the plan is destroyed
     void* pos = nullptr;               // per-vortex cell records of the last located set
     int64_t pos_cap = 0;
     void* recs = nullptr;              // records binned by tile (with each vortex's original index)

@@ -597,6 +597,7 @@ pf_status step_captured(pf_plan p, pf_state s, const pf_body_kinematics& k, doub
     int64_t last[2 * PF_MAX_BODIES];
     std::copy(std::begin(s->last), std::end(s->last), last);
     s->capture = true;
+    p->captured = true;
     const pf_status st = pf_step(p, s, &k, dt, scheme);
     s->capture = false;
     s->nv = nv;

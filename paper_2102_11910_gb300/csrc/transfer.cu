@@ -29,6 +29,13 @@
 
 namespace {
 
+// a binning buffer that was outgrown (the plan's stream is idle)
+void retire(pf_plan p, void* q) {
+    if (!q) return;
+    if (p->captured) p->retired.push_back(q);
+    else cudaFree(q);
+}
+
 pf_status plan_bin_reserve(pf_plan p, int64_t nv, int tile, int min_span) {
     const size_t psz = p->prec == PF_FP64 ? sizeof(Pos<double>) : sizeof(Pos<float>);
     const size_t rsz = p->prec == PF_FP64 ? sizeof(Rec<double>) : sizeof(Rec<float>);
@@ -41,7 +48,7 @@ pf_status plan_bin_reserve(pf_plan p, int64_t nv, int tile, int min_span) {
     if (nv > p->pos_cap) {
         const int64_t cap = std::max<int64_t>(std::max<int64_t>(nv, 2 * p->pos_cap), 4096);
         PF_CUDA(p, cudaStreamSynchronize(p->stream));
-        if (p->pos) cudaFree(p->pos);
+        retire(p, p->pos);
         p->pos = nullptr;
         p->pos_cap = 0;
         PF_CUDA(p, cudaMalloc(&p->pos, (size_t)cap * psz));
@@ -50,7 +57,7 @@ pf_status plan_bin_reserve(pf_plan p, int64_t nv, int tile, int min_span) {
     if (4 * nv > p->rec_cap) {   // a vortex is entered in at most four tiles
         const int64_t cap = 4 * p->pos_cap;
         PF_CUDA(p, cudaStreamSynchronize(p->stream));
-        if (p->recs) cudaFree(p->recs);
+        retire(p, p->recs);
         p->recs = nullptr;
         p->rec_cap = 0;
         PF_CUDA(p, cudaMalloc(&p->recs, (size_t)cap * rsz));
@@ -60,7 +67,7 @@ pf_status plan_bin_reserve(pf_plan p, int64_t nv, int tile, int min_span) {
     if (need > p->bin_off_cap) {
         const int64_t cap = std::max<int64_t>(need, bin_off_ints(p->nx, p->ny, tile, p->pos_cap, min_span));
         PF_CUDA(p, cudaStreamSynchronize(p->stream));
-        if (p->bin_off) cudaFree(p->bin_off);
+        retire(p, p->bin_off);
         p->bin_off = nullptr;
         p->bin_off_cap = 0;
         PF_CUDA(p, cudaMalloc(&p->bin_off, (size_t)cap * sizeof(int)));
