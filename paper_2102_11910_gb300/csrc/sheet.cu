@@ -27,11 +27,11 @@ __device__ __forceinline__ long long fx_q61(double w) {
     const long long v = fx_align1(m, 1014 - ef);                // m 2^(ef - 1075) 2^61
     return b < 0 ? -v : v;
 }
-// a table value in Q60 (0 at the origin, else 1/4 .. 1.53, at the corner of 2048 x 2048 nodes): its mantissa shifted
+// a table value in Q61 (0 at the origin, else 1/4 .. 1.53, at the corner of 2048 x 2048 nodes): its mantissa shifted
 __device__ __forceinline__ long long fx_lgf(double g) {
     const long long b = __double_as_longlong(g);
     const int ef = (int)(b >> 52);
-    return ef ? ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << (ef - 1015) : 0ll;
+    return ef ? ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << (ef - 1014) : 0ll;
 }
 
 // Sum over a chunk of the vortices (blockIdx.y) of Gamma_q sum_{16 x 16 node
@@ -40,9 +40,9 @@ __device__ __forceinline__ long long fx_lgf(double g) {
 // vortices has its weights formed by a thread per vortex and axis, then eight
 // lanes a vortex take one column of the offsets each, so that a table row's
 // seven values are one or two lines for the lanes together (a thread a vortex
-// would touch 49).  Weights in Q61, table and products in Q60 on the integer
-// pipe (FP64 has two multiply-adds a clock and SM), the sum over vortices in
-// FP64 in a fixed order.  p = 0 also sums the chunk's Gamma.  A last row of blocks
+// would touch 49).  Weights, table and products in Q61 on the integer pipe
+// (FP64 has two multiply-adds a clock and SM), the sum over vortices in FP64
+// in a fixed order.  p = 0 also sums the chunk's Gamma.  A last row of blocks
 // forms, for each released vortex j, e_j[p] (position: given, or by the
 // placement rule).
 constexpr int VR_THREADS = 128, VR_ROUND = 64;
@@ -95,30 +95,32 @@ __device__ __forceinline__ bool vr_weights(double z, const Geo& geo, int axis, i
     return ok;
 }
 
-// This lane's column d of the pair sum, in Q60: cx[d] sum_e cy[e] G(base + (d, e)).
-// The middle sum t stays below 2^63: low halves are at most 2^30, the seven |cy|
-// add up to 1.25 at most, and the table's high halves to 7 x 1.53 x 2^29, so t is at most
-// (7 x 1.53 / 2 + 1.25) 2^60 = 6.6 x 2^60.  (With the table in Q61 it passed
-// 2^63 from offsets of about 100 nodes on.)
+// This lane's column d of the pair sum, in Q61: cx[d] sum_e cy[e] G(base + (d, e)).
+// The middle sum is taken in two parts, t0 over four entries and t1 over three:
+// low halves are at most 2^30, the table's high halves 1.53 x 2^30 and the seven
+// |cy| add up to at most 1.25, so t0 is at most (4 x 1.53 + 1.25) 2^60 = 7.4 x
+// 2^60 < 2^63, where all seven together pass 2^63 from offsets of about 100 nodes on.
+// (With the table in Q60 one sum holds them, and a bit is lost.)
 __device__ __forceinline__ long long vr_column(const FxSplit (*c)[8], const int* base, int d, const double* __restrict__ G,
                                                int ld) {
     if (d == 7) return 0;
     int m = base[0] + d;
     m = m < 0 ? -m : m;
-    long long h = 0, t = 1ll << 29;
+    long long h = 0, t0 = 1ll << 29, t1 = 0;
 #pragma unroll
     for (int e = 0; e < 7; ++e) {
         int n = base[1] + e;
         n = n < 0 ? -n : n;
         const FxSplit g = fx_split(fx_lgf(__ldg(G + (size_t)n * ld + m))), w = c[1][e];
         h += fx_mw(g.h, w.h);
-        t += fx_mw(g.h, w.l) + fx_mw(g.l, w.h);
+        (e < 4 ? t0 : t1) += fx_mw(g.h, w.l) + fx_mw(g.l, w.h);
     }
-    return fx_weigh(fx_split((h << 1) + (t >> 30)), c[0][d]);
+    const long long low = (1ll << 30) - 1, t = (t0 >> 30) + (t1 >> 30) + (((t0 & low) + (t1 & low)) >> 30);
+    return fx_weigh(fx_split((h << 1) + t), c[0][d]);
 }
 
-// Q60 to double
-__device__ __forceinline__ double fx_q60_double(long long v) { return fx_to_double(v, -60); }
+// Q61 to double
+__device__ __forceinline__ double fx_q61_double(long long v) { return fx_to_double(v, -61); }
 
 // e_j[p] of the released vortices, eight lanes each
 __device__ __forceinline__ void released(const VortexRhs& A, const Geo& geo, int p, const int (&surf)[2], VrShared& s,
@@ -143,7 +145,7 @@ __device__ __forceinline__ void released(const VortexRhs& A, const Geo& geo, int
     const int j = tid >> 3;                      // ne <= 2 PF_MAX_BODIES = 8 groups of eight lanes
     double u = 0.0;
     const bool ok = j < A.ne && s.base[j][0] < 1 << 20 && s.base[j][1] < 1 << 20;
-    if (ok) u = fx_q60_double(vr_column(s.c[j], s.base[j], lane8, A.table, geo.nx + 1));
+    if (ok) u = fx_q61_double(vr_column(s.c[j], s.base[j], lane8, A.table, geo.nx + 1));
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
     if (j < A.ne && lane8 == 0) {
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(VR_THREADS) k_vortex_rhs(VortexRhs A, Geo geo,
 #pragma unroll 1
             for (int v = tid >> 3; v < VR_ROUND; v += VR_THREADS / 8)
                 if (s.base[v][0] < 1 << 20 && s.base[v][1] < 1 << 20)
-                    acc += s.g[v] * fx_q60_double(vr_column(s.c[v], s.base[v], lane8, A.table, geo.nx + 1));
+                    acc += s.g[v] * fx_q61_double(vr_column(s.c[v], s.base[v], lane8, A.table, geo.nx + 1));
             __syncthreads();
         }
 #pragma unroll
